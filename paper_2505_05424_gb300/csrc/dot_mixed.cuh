@@ -24,7 +24,8 @@ struct SlotParam {
 struct MxFields {
   float* q[kMaxD + 1];     // q_0: T*P; q_d: (T+1)*P padded
   float2* al[kMaxD + 1];   // alpha / sigma (two-float), same shapes as q
-  float2* beta;            // beta / sigma (two-float), K * T * P
+  float2* beta;            // beta / sigma (two-float), K * T * P; component planes for D = 3, for
+                           // D = 2 the pairs of beta2_at
   float* z;                // K * T * P
   float2* phi;             // (T+1)*P two-float potential
   float* b;                // (T+1)*P right-hand side, high part; reused for the correction delta
@@ -40,6 +41,17 @@ struct MxFields {
   const float* somega;     // P or nullptr: sqrt(omega/2)
   const SlotParam* sp;     // G slot parameters
 };
+
+// D = 2: beta is stored as five planes of float4, one per pair of cone components
+// (0, 9), (1, 5), (2, 6), (3, 7), (4, 8) -- the x-face and y-face components of the
+// same kind side by side -- holding both high parts, then both low parts: the lane
+// pairs that the fused pass computes in, loaded and stored without rearranging.
+// Index of component j's high part at cone i (of n0) in floats; its low part is two
+// floats further.
+__host__ __device__ inline long long beta2_at(int j, long long i, long long n0) {
+  const int pair = j == 9 ? 0 : j <= 4 ? j : j - 4, lane = j == 9 || (j >= 5) ? 1 : 0;
+  return (pair * n0 + i) * 4 + lane;
+}
 
 constexpr int kBsumStride = 1024;   // doubles per slot in bsum: partial sums, then mean(b)
 
@@ -135,21 +147,13 @@ void launch_kkt_mx(const Geo& g, int G, const MxFields& f, double* partials, dou
                    const double* socp_part, int nsocp, cudaStream_t s, LaunchCounter lc);
 
 // Fused lines 3-6 for D = 2 (k_fused2d.cu) for every active slot: reads q, alpha,
-// beta of f, writes those of fn; phi, somega, sp from f.  socp_part:
-// fused2d_blocks(g) doubles per slot.
+// beta of f, writes those of fn and the next iteration's lines 1-2 residual into f.r
+// (see launch_solve_residual_mx); phi, somega, sp from f.  socp_part:
+// fused2d_partials(g, G) doubles per slot (the tiling depends on the batch size).
 bool fused2d_supported(const Geo& g);
-long long fused2d_blocks(const Geo& g);
+long long fused2d_partials(const Geo& g, int G);
 void launch_fused2d(const Geo& g, int G, const MxFields& f, const MxFields& fn, double* socp_part,
                     cudaStream_t s, LaunchCounter lc);
-// The same pass with beta staged by TMA (needs N_y even); socp_part:
-// fused2d_tma_blocks(g, G) doubles per slot (the time chunking depends on the batch size).  Returns false if the tensor map cannot
-// be built.
-bool fused2d_tma_supported(const Geo& g);
-long long fused2d_tma_blocks(const Geo& g, int G);
-// residual: also write the next iteration's lines 1-2 residual into f.r (see
-// launch_solve_residual_mx).
-bool launch_fused2d_tma(const Geo& g, int G, const MxFields& f, const MxFields& fn, double* socp_part, int* err,
-                        bool residual, cudaStream_t s, LaunchCounter lc);
 // Fused lines 3-6 for D = 3 (k_fused3d.cu) for every active slot: z and q_0, alpha_0
 // by one pass over the cones, then q_d, alpha_d, beta by a time-marching pass over
 // tiles of cells; reads q, alpha, beta of f, writes those of fn; f.z is scratch.

@@ -196,6 +196,8 @@ Batch* dot_server::new_batch(const Request& r) {
     const long long per = nodes_of(r.grid);
     long long want = (sopt.target_nodes + per - 1) / per;
     G = (int)std::max(1LL, std::min<long long>(want, sopt.max_slots));
+    // element indices over all slots, the cone components included, stay below 2^31
+    while (G > 1 && G * per * g.K >= (1LL << 31)) G /= 2;
   }
   const bool masks = true;
   size_t bytes = MixedBatch::workspace_bytes(g, G, masks);

@@ -212,6 +212,18 @@ __device__ __forceinline__ ff2 ff2_add(ff2 a, ff2 b) {
   s.l = add2(s.l, add2(a.l, b.l));
   return quick_two_sum2(s.h, s.l);
 }
+// lane-wise a - b: two_sum2(a, -b) without forming -b
+__device__ __forceinline__ ff2 two_diff2(float2 a, float2 b) {
+  const float2 s = sub2(a, b);
+  const float2 bb = sub2(s, a);
+  return ff2{s, sub2(sub2(a, sub2(s, bb)), add2(b, bb))};
+}
+// lane-wise ff_add of a and -b
+__device__ __forceinline__ ff2 ff2_sub(ff2 a, ff2 b) {
+  ff2 s = two_diff2(a.h, b.h);
+  s.l = add2(s.l, sub2(a.l, b.l));
+  return quick_two_sum2(s.h, s.l);
+}
 // lane-wise ff_add_f
 __device__ __forceinline__ ff2 ff2_add_f(ff2 a, float2 b) {
   ff2 s = two_sum2(a.h, b);
@@ -260,6 +272,13 @@ __device__ __forceinline__ float2 ff_sqrt_r(float2 a, float* rinv) {
   return quick_two_sum(s, rem * (0.5f * r));
 }
 
+// 1/x to about one ulp (normal x)
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 // Running sum of two-float terms with one normalisation at the end: the high parts
 // are added by TwoSum (each rounding error kept exactly), the low parts and those
 // errors in one FP32 correction.  Same accuracy class as a chain of ff_add.
@@ -288,12 +307,45 @@ __device__ __forceinline__ void acc_add_mul(ff_acc& s, float2 b, float x) {
 }
 __device__ __forceinline__ float2 acc_get(const ff_acc& s) { return quick_two_sum(s.h, s.c); }
 
+// (b - a) invh for two two-float values, as an unevaluated pair: the difference of
+// the high parts by TwoSum
+__device__ __forceinline__ float2 ff_grad(float2 a, float2 b, float invh) {
+  const float2 dh = two_sum(b.x, -a.x);
+  const float dl = (b.y - a.y) + dh.y;
+  return make_float2(dh.x * invh, dl * invh);
+}
+// ff_acc in two lanes
+struct ff2_acc {
+  float2 h, c;
+};
+__device__ __forceinline__ void acc2_add(ff2_acc& s, ff2 b) {
+  const ff2 t = two_sum2(s.h, b.h);
+  s.h = t.h;
+  s.c = add2(s.c, add2(t.l, b.l));
+}
+__device__ __forceinline__ void acc2_add_f(ff2_acc& s, float2 b) {
+  const ff2 t = two_sum2(s.h, b);
+  s.h = t.h;
+  s.c = add2(s.c, t.l);
+}
+// + (b.h + b.c) * x for an unnormalised sum b: the exact product of its high part by
+// TwoProd, its correction's product into the correction
+__device__ __forceinline__ void acc2_add_mul(ff2_acc& s, ff2_acc b, float2 x) {
+  const ff2 p = two_prod2(b.h, x);
+  const ff2 t = two_sum2(s.h, p.h);
+  s.h = t.h;
+  s.c = add2(s.c, add2(t.l, fma2(b.c, x, p.l)));
+}
+
 // Projection onto {y_0 >= |ybar|} (eq. (app-proj)) of a K = 10 cone held as five
-// lane pairs: P[0] = (y_0, y_9), P[k] = (y_{2k-1}, y_{2k}) for k = 1..4.  The same
+// lane pairs: P[0] = (y_0, y_9), P[1..4] = y_1 .. y_8 paired in any order.  The same
 // method as ff_proj_soc (two-float |ybar|, FP32 boundary direction), with |ybar|^2
 // summed in two lanes, the square root from rsqrt and the boundary scale from its
 // reciprocal instead of divisions.
-__device__ __forceinline__ void ff2_proj_soc10(ff2* P) {
+// The three cases are one scale each for the high and low parts, without branches:
+// zr = the result rounded to FP32, pairs as P; *z0 and the returned z_9 are those two
+// components as two-floats.
+__device__ __forceinline__ float2 ff2_project10(const ff2* P, float2* zr, float2* z0) {
   float2 sh = make_float2(0.f, 0.f), sc = make_float2(0.f, 0.f);
 #pragma unroll
   for (int k = 1; k <= 4; ++k) {
@@ -301,9 +353,14 @@ __device__ __forceinline__ void ff2_proj_soc10(ff2* P) {
     const float2 p = mul2(h, h);
     const float2 e0 = make_float2(fmaf(h.x, h.x, -p.x), fmaf(h.y, h.y, -p.y));
     const float2 e = fma2(add2(h, h), P[k].l, e0);
-    const ff2 t = two_sum2(sh, p);
-    sh = t.h;
-    sc = add2(sc, add2(t.l, e));
+    if (k == 1) {
+      sh = p;
+      sc = e;
+    } else {
+      const ff2 t = two_sum2(sh, p);
+      sh = t.h;
+      sc = add2(sc, add2(t.l, e));
+    }
   }
   // y_9 and the two lanes
   const float h9 = P[0].h.y;
@@ -315,19 +372,19 @@ __device__ __forceinline__ void ff2_proj_soc10(ff2* P) {
   float r;
   const float2 nb = ff_sqrt_r(quick_two_sum(t2.x, corr), &r);
   const float2 y0 = ff2_lane0(P[0]);
-  if (ff_le(nb, y0)) return;
-  if (ff_le(nb, ff_neg(y0))) {
-#pragma unroll
-    for (int k = 0; k < 5; ++k) P[k] = ff2{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-    return;
-  }
+  const bool inside = ff_le(nb, y0), below = ff_le(nb, ff_neg(y0));
   const float2 sum = ff_add(y0, nb);
   const float2 a = make_float2(0.5f * sum.x, 0.5f * sum.y);
-  const float scale = (a.x + a.y) * r;
-  const float2 sc2 = make_float2(scale, scale), zero2 = make_float2(0.f, 0.f);
+  // inside: h + l; below: 0; else the boundary point along ybar / |ybar|
+  const float m = inside ? 1.f : 0.f;
+  const float scale = inside ? 1.f : below ? 0.f : (a.x + a.y) * r;
+  *z0 = inside ? y0 : below ? make_float2(0.f, 0.f) : a;
+  const float2 m2 = make_float2(m, m), s2 = make_float2(scale, scale);
 #pragma unroll
-  for (int k = 1; k <= 4; ++k) P[k] = ff2{mul2(sc2, P[k].h), zero2};
-  P[0] = ff2{make_float2(a.x, scale * P[0].h.y), make_float2(a.y, 0.f)};
+  for (int k = 1; k <= 4; ++k) zr[k] = fma2(m2, P[k].l, mul2(s2, P[k].h));
+  const float2 z9 = make_float2(scale * h9, m * P[0].l.y);
+  zr[0] = make_float2(z0->x + z0->y, z9.x + z9.y);
+  return z9;
 }
 
 }  // namespace dot

@@ -1,44 +1,66 @@
 // k_fused2d.cu -- lines 3-6 of Algorithm 2 (cone projection, q and alpha updates,
-// beta update) fused into one pass over the mixed-path state, for D = 2.
+// beta update) fused into one pass over the mixed-path state, for D = 2, and the
+// next iteration's lines 1-2 residual.
 //
-// A CTA owns a 16 x 32 (x, y) tile of the spatial grid and a chunk [ta, tb) of
-// cone times, and marches along time.  At cone time t it
-//   A. projects z(t) = Pi_K(B F q^k + d - beta^k/sigma) for the tile's cones and a
-//      one-cone halo ring, keeps u_v = z_v + beta_v/sigma (v = 1..8, the parts
-//      F^*B^* sends to space faces) in shared memory for two time levels, keeps the
-//      owned cones' z in registers, and updates q_0, alpha_0 of the owned cones
-//      (diagonal 3, Proposition 3.2);
-//   B. updates q_d, alpha_d at the faces of time node t that touch the tile
-//      (including the one halo face per axis that the tile's cones read);
-//   C. updates beta of the owned cones at time t-1, which needs q^{k+1} on the
-//      faces of time nodes t-1 and t (kept in shared memory).
-// beta is read once (plus an L2 re-read in C) and written once; z never reaches
-// HBM.  q, alpha and beta are double-buffered: every read is of iteration k and
-// every write of k+1, so neighbouring CTAs may run at any relative time.
-// Per element: y and the projection tests in two-float arithmetic, FP32 z and q, two-float
-// face right-hand sides and multiplier updates (ffloat.cuh), as in k_fused3d.cu.
+// A CTA works on a TX x 32 (x, y) tile of cells at a time and marches along time.  One
+// thread owns one cone column: the cone (t, x, y) and the two space faces above it,
+// (x + 1/2, y) and (x, y + 1/2).  Three more warps take the one-cone halo: the row
+// x0 - 1 (with the x-faces the tile reads from below), the row x0 + TX, and the columns
+// y0 - 1 (with its y-faces) and y0 + 32.  At time t a thread
+//   A. projects z(t) = Pi_K(B F q^k + d - beta^k/sigma) and publishes the components
+//      that the faces below it read (1 and 3 for the x-face, 5 and 7 for the y-face);
+//      owners update q_0, alpha_0 (diagonal 3, Proposition 3.2);
+//   B. updates q_d, alpha_d of its two faces on time node t, as the two lanes of packed
+//      two-float arithmetic, from its own z and beta and its two neighbours', and
+//      publishes q and w = q - alpha/sigma - A phi of them;
+//   C. (owners) updates beta of the cone at t - 1, which reads q^{k+1} on the faces of
+//      nodes t - 1 and t (kept in registers from step to step), and writes the next
+//      iteration's residual at node t from the faces' w.
+// A thread copies its column's beta one cone time ahead into its own shared-memory
+// slots (cp.async, any N_y), where step A, the faces below it and step C read it.  z
+// never reaches HBM.  q, alpha and beta are double-buffered: every read is of iteration
+// k and every write of k+1, so CTAs may run in any order.
+// Per element: y and the projection tests in two-float arithmetic, FP32 z and q,
+// two-float face right-hand sides and multiplier updates (ffloat.cuh).
+//
+// Bound by instruction issue and by the latency of a time step (two barriers, a
+// dependent chain of some 100 FP operations): on 256^2 x 64 157 M warp instructions,
+// 49% issue, 0.58 of the HBM bandwidth on its 1,026 MB, 257 us per launch.  The form
+// before it (a thread per halo cone, faces dealt out in rounds, beta by TMA in
+// component planes, 80 registers at two CTAs per SM, fixed 16-time chunks): 245 M
+// instructions, 357 us; and for odd N_y, where it could not use TMA, 262 us on
+// 150 x 117 x 37 against 64 now.  Measured on the way: this mapping at two CTAs of 8
+// rows and 80 registers 429 us (spills), one CTA of 12 rows and 128 registers 293; equal
+// shares of work for every SM and beta in lane pairs 267.
 #include <cmath>
 
 #include "dot_internal.cuh"
 #include "dot_mixed.cuh"
-#include "dot_tc.cuh"
 #include "ffloat.cuh"
-
-#ifndef FUSED_V2_MIN_BLOCKS
-#define FUSED_V2_MIN_BLOCKS 2
-#endif
 
 namespace dot {
 namespace {
 
-constexpr int TX = 16, TY = 32;          // owned tile (x rows, y columns)
-constexpr int HX = TX + 2, HY = TY + 2;  // cone halo rectangle
-constexpr int NH = HX * HY;              // 612 cones
-constexpr int NRING = NH - TX * TY;      // 100 halo-ring cones
-constexpr int K2 = 10;                   // 4D + 2 for D = 2
-constexpr int kThreads = 256;
-constexpr int NQ1 = (TX + 1) * TY;       // x-faces per time node: j in [x0-1, x0+15], y owned
-constexpr int NQ2 = TX * (TY + 1);       // y-faces per time node: x owned, j in [y0-1, y0+31]
+constexpr int K2 = 10;                    // 4D + 2 for D = 2
+constexpr int TY = 32;                    // tile columns: one warp per row
+constexpr int kStages = 3;                // beta of cone times t - 1, t, t + 1
+constexpr int kSMs = 152;
+constexpr float kSdef = 0.70710678118654752f;            // sqrt(omega / 2) for omega = 1
+
+// Threads and shared memory of a CTA with TX tile rows.
+template <int TX>
+struct Tile {
+  static constexpr int kWarps = TX + 3;   // owners, rows x0 - 1 and x0 + TX, columns y0 - 1 and y0 + 32
+  static constexpr int kThreads = 32 * kWarps;
+  static_assert(2 * TX <= 32, "one warp holds both halo columns");
+  // bytes: beta slots, then one slot per thread of what its neighbours read
+  static constexpr int kOffZ1 = kStages * (K2 / 2) * kThreads * 16;   // z_(1, 5) of cone time t
+  static constexpr int kOffZ3 = kOffZ1 + kThreads * 8;                // z_(3, 7), two cone times
+  static constexpr int kOffPh = kOffZ3 + 2 * kThreads * 8;            // phi on node t
+  static constexpr int kOffQ = kOffPh + kThreads * 8;                 // q^{k+1} of the (x, y) faces
+  static constexpr int kOffW = kOffQ + kThreads * 8;                  // alpha/sigma + A phi - q of the faces
+  static constexpr int kSmem = kOffW + kThreads * 16;
+};
 
 // The multipliers are stored as alpha/sigma and beta/sigma (k_mixed.cu), so the
 // projection input is BFq + d - (stored beta) and the updates add tau (...).
@@ -46,343 +68,457 @@ struct FusedArgs {
   // iteration k (read)
   const float* q[3];
   const float2* al[3];
-  const float2* beta;
+  const float4* beta;
   // iteration k+1 (write)
   float* qn[3];
   float2* aln[3];
-  float2* betan;
+  float4* betan;
   const float2* phi;   // phi^{k+1}
   const float* somega;
-  float ts;            // tau (set per slot from sp)
-  int tchunk;          // cone times per CTA
-  int nchunk;          // time chunks per slot (grid z = slots x chunks)
+  int G;               // slots
+  int ntx, nty;        // tiles along x and y
+  int unit, nunit;     // cone times per work unit, units per tile
   const SlotParam* sp;
-  double* socp_part;   // per-block sum of |z - B F q^{k+1} - d|^2, or nullptr
-  long long socp_per_slot;
-  int* err;            // set when a pipeline wait gave up
-  // TMA kernel only (nullable r): the next iteration's lines 1-2 residual
+  double* socp_part;   // per work unit: sum of |z - B F q^{k+1} - d|^2
+  // the next iteration's lines 1-2 residual
   // r = A^*(q^{k+1} - alpha^{k+1}/sigma) - c/sigma - A^*A phi^{k+1} at every node
   float* r;
   const float2* c0;
   const float2* c1;
-  float2 isg;          // 1/sigma (set per slot from sp)
+  float ih0, ih1, ih2; // 1/h of time and of the two axes
 };
 
-// The arguments of slot b of a batch.
-__device__ __forceinline__ FusedArgs fused_slot(FusedArgs a, const Geo& g, int b) {
-  const long long nn = (long long)(g.T + 1) * g.P, n0 = (long long)g.T * g.P;
-  a.ts = a.sp[b].tau;
-  a.isg = a.sp[b].isg;
-  if (b == 0) return a;
-  a.q[0] += b * n0;
-  a.al[0] += b * n0;
-  a.qn[0] += b * n0;
-  a.aln[0] += b * n0;
-  for (int d = 1; d < 3; ++d) {
-    a.q[d] += b * nn;
-    a.al[d] += b * nn;
-    a.qn[d] += b * nn;
-    a.aln[d] += b * nn;
+// 16-byte asynchronous copy into this thread's shared-memory slot
+__device__ __forceinline__ void copy16(uint32_t dst, const float4* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+// beta as stored for D = 2: component pairs (0, 9), (1, 5), (2, 6), (3, 7), (4, 8),
+// high parts then low parts
+__device__ __forceinline__ ff2 ff2_of(float4 b) { return ff2{make_float2(b.x, b.y), make_float2(b.z, b.w)}; }
+__device__ __forceinline__ float4 f4_of(ff2 b) { return make_float4(b.h.x, b.h.y, b.l.x, b.l.y); }
+
+__device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
+
+// One segment: cone times [ta, tb) of one tile of one slot.  *pend: the work unit of
+// the segment before whose sums wait in wsum (null: none).  Element indices stay below
+// 2^31 over all slots of a batch (dot_server.cu bounds the batch).
+template <int TX, bool MASKED>
+__device__ __forceinline__ void segment(const Geo& g, const FusedArgs& a, unsigned char* sm, double* wsum, int slot,
+                                        int x0, int y0, int ta, int tb, double* socp_tile, double** pend) {
+  using L = Tile<TX>;
+  constexpr int kThreads = L::kThreads;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int T = g.T, P = (int)g.P, n0 = T * P, N0 = g.N[0], N1 = g.N[1];
+  const float ts = a.sp[slot].tau;
+  const float ih0 = a.ih0, ih1 = a.ih1, ih2 = a.ih2;
+
+  // this thread's cone column, as tile coordinates (xr, yc), and the threads of the
+  // columns above (x + 1, y), (x, y + 1) and below (x - 1, y), (x, y - 1)
+  const bool owner = warp < TX;
+  int xr = warp, yc = lane;
+  int hx = xr == TX - 1 ? tid + 64 : tid + 32, hy = lane == 31 ? (TX + 2) * 32 + TX + xr : tid + 1;
+  const int lx = xr == 0 ? TX * 32 + lane : tid - 32, ly = lane == 0 ? (TX + 2) * 32 + xr : tid - 1;
+  if (!owner) {
+    hx = hy = tid;
+    if (warp == TX) {
+      xr = -1;
+      hx = lane;
+    } else if (warp == TX + 1) {
+      xr = TX;
+    } else if (lane < TX) {
+      xr = lane;
+      yc = -1;
+      hy = lane * 32;
+    } else {
+      xr = lane - TX;
+      yc = TY;
+    }
   }
-  a.beta += b * K2 * n0;
-  a.betan += b * K2 * n0;
-  a.phi += b * nn;
-  if (a.somega) a.somega += b * g.P;
-  if (a.socp_part) a.socp_part += b * a.socp_per_slot;
-  if (a.r) {
-    a.r += b * nn;
-    a.c0 += b * g.P;
-    a.c1 += b * g.P;
+  const int x = x0 + xr, y = y0 + yc;
+  const bool cone_ok = x >= 0 && y >= 0 && x < N0 && y < N1 && (warp < TX + 2 || lane < 2 * TX);
+  // the column's own faces (x + 1/2, y), (x, y + 1/2), where the tile needs them
+  const bool fx = cone_ok && warp <= TX && x <= N0 - 2;
+  const bool fy = cone_ok && (owner || (warp == TX + 2 && lane < TX)) && y <= N1 - 2;
+  const bool own_ok = owner && cone_ok;
+  const bool xl = cone_ok && x >= 1, xh = cone_ok && x <= N0 - 2, yl = cone_ok && y >= 1, yh = cone_ok && y <= N1 - 2;
+
+  // sqrt(omega / 2) of the cone and of the cones across its faces
+  float s = kSdef;
+  float2 sn = f2(kSdef, kSdef);
+  if (MASKED && cone_ok) {
+    const float* w = a.somega + slot * P + x * N1 + y;
+    s = w[0];
+    if (fx) sn.x = w[N1];
+    if (fy) sn.y = w[1];
   }
-  return a;
-}
-
-// halo-ring cone number r (0..99) -> (xh, yh) on the border of the HX x HY rectangle
-__device__ __forceinline__ void ring_pos(int r, int* xh, int* yh) {
-  if (r < HY) { *xh = 0; *yh = r; return; }
-  r -= HY;
-  if (r < HY) { *xh = HX - 1; *yh = r; return; }
-  r -= HY;
-  if (r < HX - 2) { *xh = 1 + r; *yh = 0; return; }
-  r -= HX - 2;
-  *xh = 1 + r;
-  *yh = HY - 1;
-}
-
-__device__ __forceinline__ float2 grad_pair(const float2* phi, long long i, long long j, float invh) {
-  const float2 a = phi[i], b = phi[j];
-  const float2 dh = two_sum(b.x, -a.x);
-  const float dl = (b.y - a.y) + dh.y;
-  return make_float2(dh.x * invh, dl * invh);
-}
-
-__device__ __forceinline__ float grad_minus(float2 g, float q) { return (g.x - q) + g.y; }
-
-// z of cone (t, x, y) from iteration-k data, formed and projected in two-float
-// arithmetic (y = BFq + d - beta/sigma is dominated by beta/sigma); returns false
-// for a cone outside the grid.
-__device__ __forceinline__ bool cone_z(const Geo& g, const FusedArgs& a, int t, int x, int y, float2* z) {
-  if (x < 0 || y < 0 || x >= g.N[0] || y >= g.N[1]) return false;
-  const long long P = g.P, n0 = (long long)g.T * P;
-  const long long N1 = g.N[1];
-  const long long i = (long long)t * P + (long long)x * N1 + y;
-  const float* q1 = a.q[1];
-  const float* q2 = a.q[2];
-  const bool xl = x >= 1, xr = x <= g.N[0] - 2, yl = y >= 1, yr = y <= g.N[1] - 2;
-  float xv[K2 - 1];
-  xv[0] = a.q[0][i];
-  xv[1] = xl ? q1[i - N1] : 0.f;
-  xv[2] = xr ? q1[i] : 0.f;
-  xv[3] = xl ? q1[i + P - N1] : 0.f;
-  xv[4] = xr ? q1[i + P] : 0.f;
-  xv[5] = yl ? q2[i - 1] : 0.f;
-  xv[6] = yr ? q2[i] : 0.f;
-  xv[7] = yl ? q2[i + P - 1] : 0.f;
-  xv[8] = yr ? q2[i + P] : 0.f;
-  const float s = a.somega ? a.somega[(long long)x * N1 + y] : 0.70710678118654752f;
-  z[0] = ff_add(two_sum(-xv[0], 1.f), ff_neg(a.beta[i]));
-#pragma unroll
-  for (int j = 1; j < K2 - 1; ++j)
-    z[j] = ff_add(two_prod(s, xv[j]), ff_neg(a.beta[(long long)j * n0 + i]));
-  z[K2 - 1] = ff_add(two_sum(xv[0], 1.f), ff_neg(a.beta[(long long)(K2 - 1) * n0 + i]));
-  ff_proj_soc<K2>(z);
-  return true;
-}
-
-constexpr int kSmemFused = (2 * 8 * NH) * 8 + (2 * NQ1 + 2 * NQ2) * 4;
-
-__global__ void __launch_bounds__(kThreads, 2) k_fused2d(Geo g, FusedArgs a_in) {
-  const int slot = blockIdx.z / a_in.nchunk, chunk = blockIdx.z - slot * a_in.nchunk;
-  if (!a_in.sp[slot].active) return;
-  const FusedArgs a = fused_slot(a_in, g, slot);
-  // u_1..u_8 (two-float) of every halo cone at two time levels, then q^{k+1} on
-  // the tile's x-faces and y-faces at two node levels
-  extern __shared__ __align__(16) unsigned char fsm[];
-  float2 (*su)[8][NH] = reinterpret_cast<float2 (*)[8][NH]>(fsm);
-  float (*sq1)[NQ1] = reinterpret_cast<float (*)[NQ1]>(fsm + (2 * 8 * NH) * 8);
-  float (*sq2)[NQ2] = reinterpret_cast<float (*)[NQ2]>(fsm + (2 * 8 * NH) * 8 + 2 * NQ1 * 4);
-
-  const int tid = threadIdx.x;
-  const int ly = tid & 31, lx = tid >> 5;   // owned nodes (x0 + lx + 8r, y0 + ly)
-  const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
-  const int ta = chunk * a.tchunk;
-  const int tb = min(g.T, ta + a.tchunk);
-  const bool last_chunk = (tb == g.T);
-  const long long P = g.P, n0 = (long long)g.T * P;
-  const long long N1 = g.N[1];
-  const float ts = a.ts;
-  const float ih0 = (float)g.invh[0], ih1 = (float)g.invh[1], ih2 = (float)g.invh[2];
-  const float s_def = 0.70710678118654752f;
-
-  // registers of the two owned cones: z at the current and previous cone time,
-  // q_0^{k+1} at the previous cone time
-  float zc[2][K2], zp[2][K2];
-  float q0c[2] = {0.f, 0.f}, q0p[2] = {0.f, 0.f};
-  float socp = 0.f;
-  bool own_ok[2];
-#pragma unroll
-  for (int r = 0; r < 2; ++r) own_ok[r] = (x0 + lx + 8 * r) < g.N[0] && (y0 + ly) < g.N[1];
 
   const int tstart = ta > 0 ? ta - 1 : 0;
-  for (int t = tstart; t <= tb; ++t) {
-    const int lev = t & 1;
+  const int tlast = min(tb, T - 1);         // last cone time this segment projects
+  // element of the column on time plane t: of node fields; cone fields and beta's pair 0
+  // at a fixed distance
+  int i = slot * (n0 + P) + tstart * P + x * N1 + y;
+  const int ocone = -slot * P, obeta = slot * (n0 * (K2 / 2 - 1) - P);
+
+  // shared memory: this thread's beta slots (pair k of stage j at (j K/2 + k) kThreads)
+  // and what it publishes
+  float4* bslot = reinterpret_cast<float4*>(sm) + tid;
+  const float* bx = reinterpret_cast<const float*>(reinterpret_cast<float4*>(sm) + hx);
+  const float* by = reinterpret_cast<const float*>(reinterpret_cast<float4*>(sm) + hy) + 1;
+  float2* sz1 = reinterpret_cast<float2*>(sm + L::kOffZ1);
+  float2* sz3 = reinterpret_cast<float2*>(sm + L::kOffZ3);
+  float2* sph = reinterpret_cast<float2*>(sm + L::kOffPh);
+  float2* sq = reinterpret_cast<float2*>(sm + L::kOffQ);
+  float4* sw = reinterpret_cast<float4*>(sm + L::kOffW);
+  const uint32_t bsm = (uint32_t)__cvta_generic_to_shared(bslot);
+  auto fetch = [&](int stage, int ii) {
+    if (cone_ok) {
+      const float4* src = a.beta + ii;
+#pragma unroll
+      for (int k = 0; k < K2 / 2; ++k) copy16(bsm + (stage * (K2 / 2) + k) * kThreads * 16, src + (long long)k * n0);
+    }
+  };
+  int st_c = 0, st_n = 1, st_p = 2;         // stages of cone times t, t + 1, t - 1
+  if (tstart <= tlast) fetch(st_c, i + obeta);
+  asm volatile("cp.async.commit_group;" ::: "memory");
+
+  // F q^k of the column: x-lane and y-lane faces below / above on node t (qa, qb), and
+  // the next cone time's node (qc, qd) with q_0, one cone time ahead; the potential,
+  // alpha_0 of the cone and alpha of the own faces one time ahead too
+  const float2 z2 = f2(0.f, 0.f);
+  float2 qa = z2, qb = z2, qc = z2, qd = z2;
+  float qz = 0.f;
+  float2 ph_t = z2, ph_n = z2, al0 = z2, a1 = z2, a2 = z2;
+  if (cone_ok) {
+    if (xl) qa.x = a.q[1][i - N1];
+    if (yl) qa.y = a.q[2][i - 1];
+    if (xh) qb.x = a.q[1][i];
+    if (yh) qb.y = a.q[2][i];
+    if (tstart <= tlast) {
+      qz = a.q[0][i + ocone];
+      if (xl) qc.x = a.q[1][i + P - N1];
+      if (yl) qc.y = a.q[2][i + P - 1];
+      if (xh) qd.x = a.q[1][i + P];
+      if (yh) qd.y = a.q[2][i + P];
+    }
+    ph_t = a.phi[i];
+    ph_n = a.phi[i + P];                    // tstart <= T - 1
+    if (owner) al0 = a.al[0][i + ocone];
+    if (tstart >= ta) {
+      if (fx) a1 = a.al[1][i];
+      if (fy) a2 = a.al[2][i];
+    }
+  }
+
+  float2 zc[5], zp[5];                      // FP32 z of the cone at t and t - 1: (0, 9), (1, 5), ..., (4, 8)
+#pragma unroll
+  for (int k = 0; k < 5; ++k) zc[k] = zp[k] = z2;
+  float q0c = 0.f, q0p = 0.f;
+  float2 w0c = z2, w0p = z2;                // alpha_0/sigma + A_0 phi - q_0 of cones t and t - 1 (unnormalised)
+  float2 qlp = z2, qop = z2;                // q^{k+1} of the faces below and of the own faces on node t - 1
+  float2 socp = z2;
+  int left = a.unit;                        // cone times to the end of the work unit
+  double* entry = socp_tile + ta / a.unit;
+
+  for (int t = tstart; t <= tb; ++t, i += P) {
+    const int lev = (t & 1) * kThreads;
+    if (t + 1 <= tlast) fetch(st_n, i + obeta + P);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
     // ---------------- A: cones at time t ----------------
-    if (t <= g.T - 1) {
-#pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        const int x = x0 + lx + 8 * r, y = y0 + ly;
-        const int hc = (lx + 8 * r + 1) * HY + (ly + 1);
-        float2 z[K2];
-        const bool ok = own_ok[r] && cone_z(g, a, t, x, y, z);
-        if (ok) {
-          const long long i = (long long)t * P + (long long)x * N1 + y;
-#pragma unroll
-          for (int v = 0; v < 8; ++v) su[lev][v][hc] = ff_add(z[1 + v], a.beta[(long long)(1 + v) * n0 + i]);
-          if (t >= ta && t < tb) {
-            // lines 4-5 on q_0: rhs = A_0 phi + (alpha_0 + beta_{K-1} - beta_0)/sigma + (z_{K-1} - z_0),
-            // diagonal 3, in two-float arithmetic
-            const float2 gp = grad_pair(a.phi, i, i + P, ih0);
-            const float2 al = a.al[0][i];
-            const float2 db = ff_add(a.beta[(long long)(K2 - 1) * n0 + i], ff_neg(a.beta[i]));
-            float2 rhs = ff_add(gp, ff_add(al, db));
-            rhs = ff_add(rhs, ff_add(z[K2 - 1], ff_neg(z[0])));
-            const float qn = ff_round(ff_div_f(rhs, 3.f));
-            a.qn[0][i] = qn;
-            a.aln[0][i] = ff_add_f(al, ts * grad_minus(gp, qn));
-            q0c[r] = qn;   // becomes q0p at the end of this step
-          }
-#pragma unroll
-          for (int j = 0; j < K2; ++j) zc[r][j] = ff_round(z[j]);
-        } else {
-#pragma unroll
-          for (int v = 0; v < 8; ++v) su[lev][v][hc] = make_float2(0.f, 0.f);
+    if (t <= T - 1 && cone_ok) {
+      const float4* bt = bslot + st_c * (K2 / 2) * kThreads;
+      const float2 s2 = f2(s, s);
+      ff2 z[5];
+      // y = B F q + d - beta/sigma as lane pairs (0, 9), (1, 5), (2, 6), (3, 7), (4, 8)
+      z[0] = ff2_sub(two_sum2(f2(-qz, qz), f2(1.f, 1.f)), ff2_of(bt[0]));
+      z[1] = ff2_sub(two_prod2(s2, qa), ff2_of(bt[1 * kThreads]));
+      z[2] = ff2_sub(two_prod2(s2, qb), ff2_of(bt[2 * kThreads]));
+      z[3] = ff2_sub(two_prod2(s2, qc), ff2_of(bt[3 * kThreads]));
+      z[4] = ff2_sub(two_prod2(s2, qd), ff2_of(bt[4 * kThreads]));
+      // the next cone time's q^k: node t + 1 moves down, the rest is loaded now
+      qa = qc;
+      qb = qd;
+      if (t + 1 <= tlast) {
+        qz = a.q[0][i + ocone + P];
+        if (xl) qc.x = a.q[1][i + 2 * P - N1];
+        if (yl) qc.y = a.q[2][i + 2 * P - 1];
+        if (xh) qd.x = a.q[1][i + 2 * P];
+        if (yh) qd.y = a.q[2][i + 2 * P];
+      }
+      float2 z0;
+      const float2 z9 = ff2_project10(z, zc, &z0);
+      sz1[tid] = zc[1];
+      sz3[lev + tid] = zc[3];
+      // q_0 (diagonal 3): rhs = A_0 phi + alpha_0/sigma + u_9 - u_0 with u = z + beta/sigma;
+      // the cone before the segment (t = ta - 1) is updated for the residual only
+      if (owner && t < tb) {
+        const float2 gp = ff_grad(ph_t, ph_n, ih0);
+        const ff2 u = ff2_add(ff2_pack(z0, z9), ff2_of(bt[0]));
+        ff_acc acc = acc_init(gp);
+        acc_add(acc, al0);
+        acc_add(acc, ff2_lane1(u));
+        acc_add(acc, ff_neg(ff2_lane0(u)));
+        const float qn = ff_round(ff_div_f_r(acc_get(acc), 3.f, 1.f / 3.f));
+        const float gm = (gp.x - qn) + gp.y;
+        const float2 aln = ff_add_f(al0, ts * gm);
+        if (t >= ta) {
+          a.qn[0][i + ocone] = qn;
+          a.aln[0][i + ocone] = aln;
+        }
+        q0c = qn;
+        const float2 e = two_sum(aln.x, gm);
+        w0c = f2(e.x, e.y + aln.y);
+        if (t + 1 < tb) al0 = a.al[0][i + ocone + P];
+      }
+    }
+    sph[tid] = ph_t;
+    __syncthreads();
+    if (*pend) {                            // the unit that ended at the last step
+      if (tid == 0) {
+        double b = 0.0;
+        for (int w = 0; w < TX; ++w) b += wsum[w];
+        **pend = b;
+      }
+      *pend = nullptr;
+    }
+    const bool write_node = t >= ta && (t < tb || t == T);
+    float2 qo = z2;
+    ff2 wo{z2, z2};
+    // ---------------- B: the column's faces on time node t ----------------
+    if (t >= ta && (fx || fy)) {
+      // A_d phi as an unevaluated pair, both lanes
+      const float2 pa = sph[hx], pb = sph[hy];
+      const ff2 dp = two_diff2(f2(pa.x, pb.x), f2(ph_t.x, ph_t.x));
+      const float2 ih = f2(ih1, ih2);
+      const float2 gh = mul2(dp.h, ih);
+      const float2 gl = mul2(add2(sub2(f2(pa.y, pb.y), f2(ph_t.y, ph_t.y)), dp.l), ih);
+      const ff2 al = ff2_pack(a1, a2);
+      // sum over the cones reading the face of s (z + beta/sigma): the cone above it on
+      // node times t (components 1, 5) and t - 1 (3, 7), the thread's own (2, 6), (4, 8)
+      ff2_acc an{z2, z2}, ao{z2, z2};       // beta/sigma of the cone above, of the own cone
+      float2 zn = z2, zo = z2;              // their z
+      if (t <= T - 1) {
+        const int o = (st_c * (K2 / 2) + 1) * kThreads * 4;
+        an = ff2_acc{f2(bx[o], by[o]), f2(bx[o + 2], by[o + 2])};
+        const ff2 b2 = ff2_of(bslot[(st_c * (K2 / 2) + 2) * kThreads]);
+        ao = ff2_acc{b2.h, b2.l};
+        zn = f2(sz1[hx].x, sz1[hy].y);
+        zo = zc[2];
+      }
+      if (t >= 1) {
+        const int o = (st_p * (K2 / 2) + 3) * kThreads * 4;
+        acc2_add(an, ff2{f2(bx[o], by[o]), f2(bx[o + 2], by[o + 2])});
+        acc2_add(ao, ff2_of(bslot[(st_p * (K2 / 2) + 4) * kThreads]));
+        const int lp = kThreads - lev;
+        zn = add2(zn, f2(sz3[lp + hx].x, sz3[lp + hy].y));
+        zo = add2(zo, zp[4]);
+      }
+      // (the same operations with and without a mask: a solve served among masked ones
+      // takes the masked kernel, with every weight 1)
+      const float2 so = f2(s, s);
+      ff2_acc acc{gh, gl};
+      acc2_add(acc, al);
+      acc2_add_mul(acc, an, sn);
+      acc2_add_mul(acc, ao, so);
+      acc2_add_f(acc, fma2(sn, zn, mul2(so, zo)));
+      float2 dg = fma2(sn, sn, mul2(so, so));
+      if (t >= 1 && t <= T - 1) dg = add2(dg, dg);
+      const float2 den = add2(dg, f2(1.f, 1.f));
+      const float2 rd = f2(rcp_approx(den.x), rcp_approx(den.y));
+      // q = rhs / (1 + sum s^2)
+      const float2 q1 = mul2(acc.h, rd);
+      const ff2 pr = two_prod2(q1, den);
+      qo = fma2(add2(sub2(sub2(acc.h, pr.h), pr.l), acc.c), rd, q1);
+      const float2 gm = add2(sub2(gh, qo), gl);
+      const ff2 aln = ff2_add_f(al, mul2(f2(ts, ts), gm));
+      wo = two_sum2(aln.h, gm);             // alpha/sigma + A phi - q (unnormalised)
+      wo.l = add2(wo.l, aln.l);
+      if (!fx) { qo.x = 0.f; wo.h.x = 0.f; wo.l.x = 0.f; }
+      if (!fy) { qo.y = 0.f; wo.h.y = 0.f; wo.l.y = 0.f; }
+      if (write_node && owner) {
+        if (fx) {
+          a.qn[1][i] = qo.x;
+          a.aln[1][i] = ff2_lane0(aln);
+        }
+        if (fy) {
+          a.qn[2][i] = qo.y;
+          a.aln[2][i] = ff2_lane1(aln);
         }
       }
-      for (int rr = tid; rr < NRING; rr += kThreads) {
-        int xh, yh;
-        ring_pos(rr, &xh, &yh);
-        const int x = x0 - 1 + xh, y = y0 - 1 + yh;
-        const int hc = xh * HY + yh;
-        float2 z[K2];
-        if (cone_z(g, a, t, x, y, z)) {
-          const long long i = (long long)t * P + (long long)x * N1 + y;
-#pragma unroll
-          for (int v = 0; v < 8; ++v) su[lev][v][hc] = ff_add(z[1 + v], a.beta[(long long)(1 + v) * n0 + i]);
-        } else {
-#pragma unroll
-          for (int v = 0; v < 8; ++v) su[lev][v][hc] = make_float2(0.f, 0.f);
-        }
-      }
+    }
+    sq[tid] = qo;
+    sw[tid] = f4_of(wo);
+    // the next time's potential and alpha / sigma of the faces
+    ph_t = ph_n;
+    if (t < tb) {
+      if (cone_ok && t + 2 <= T) ph_n = a.phi[i + 2 * P];
+      if (fx) a1 = a.al[1][i + P];
+      if (fy) a2 = a.al[2][i + P];
     }
     __syncthreads();
-    // ---------------- B: faces at time node t ----------------
-    const bool write_node = t >= ta && ((t < tb) || (last_chunk && t == g.T));
-    if (t >= ta) {
-      const bool has_now = t <= g.T - 1, has_prev = t >= 1;
-      const int lp = lev ^ 1;
-      for (int e = tid; e < NQ1 + NQ2; e += kThreads) {
-        if (e < NQ1) {
-          // x-face (t, j, y): j = x0 - 1 + e / TY, y = y0 + e % TY
-          const int jx = e / TY, yy = e % TY;
-          const int j = x0 - 1 + jx, y = y0 + yy;
-          float qv = 0.f;
-          if (j >= 0 && j <= g.N[0] - 2 && y < g.N[1]) {
-            const long long i = (long long)t * P + (long long)j * N1 + y;
-            const float2 gp = grad_pair(a.phi, i, i + N1, ih1);
-            // cones (j+1, y) and (j, y) at halo rows jx+1 and jx, column yy+1
-            const int hr = (jx + 1) * HY + (yy + 1), hl = jx * HY + (yy + 1);
-            const float sr = a.somega ? a.somega[(long long)(j + 1) * N1 + y] : s_def;
-            const float sl = a.somega ? a.somega[(long long)j * N1 + y] : s_def;
-            float2 acc = make_float2(0.f, 0.f);
-            float dg = 0.f;
-            if (has_now) {
-              acc = ff_add(acc, ff_add(ff_mul_f(su[lev][0][hr], sr), ff_mul_f(su[lev][1][hl], sl)));
-              dg += sr * sr + sl * sl;
-            }
-            if (has_prev) {
-              acc = ff_add(acc, ff_add(ff_mul_f(su[lp][2][hr], sr), ff_mul_f(su[lp][3][hl], sl)));
-              dg += sr * sr + sl * sl;
-            }
-            const float2 al = a.al[1][i];
-            const float2 rhs = ff_add(ff_add(gp, al), acc);
-            qv = ff_round(ff_div_f(rhs, 1.f + dg));
-            if (write_node && jx >= 1) {
-              a.qn[1][i] = qv;
-              a.aln[1][i] = ff_add_f(al, ts * grad_minus(gp, qv));
-            }
-          }
-          sq1[lev][e] = qv;
-        } else {
-          // y-face (t, x, j): x = x0 + f / (TY+1), j = y0 - 1 + f % (TY+1)
-          const int f = e - NQ1;
-          const int xx = f / (TY + 1), jy = f % (TY + 1);
-          const int x = x0 + xx, j = y0 - 1 + jy;
-          float qv = 0.f;
-          if (x < g.N[0] && j >= 0 && j <= g.N[1] - 2) {
-            const long long i = (long long)t * P + (long long)x * N1 + j;
-            const float2 gp = grad_pair(a.phi, i, i + 1, ih2);
-            // cones (x, j+1) and (x, j) at halo row xx+1, columns jy+1 and jy
-            const int hr = (xx + 1) * HY + (jy + 1), hl = (xx + 1) * HY + jy;
-            const float sr = a.somega ? a.somega[(long long)x * N1 + j + 1] : s_def;
-            const float sl = a.somega ? a.somega[(long long)x * N1 + j] : s_def;
-            float2 acc = make_float2(0.f, 0.f);
-            float dg = 0.f;
-            if (has_now) {
-              acc = ff_add(acc, ff_add(ff_mul_f(su[lev][4][hr], sr), ff_mul_f(su[lev][5][hl], sl)));
-              dg += sr * sr + sl * sl;
-            }
-            if (has_prev) {
-              acc = ff_add(acc, ff_add(ff_mul_f(su[lp][6][hr], sr), ff_mul_f(su[lp][7][hl], sl)));
-              dg += sr * sr + sl * sl;
-            }
-            const float2 al = a.al[2][i];
-            const float2 rhs = ff_add(ff_add(gp, al), acc);
-            qv = ff_round(ff_div_f(rhs, 1.f + dg));
-            if (write_node && jy >= 1) {
-              a.qn[2][i] = qv;
-              a.aln[2][i] = ff_add_f(al, ts * grad_minus(gp, qv));
-            }
-          }
-          sq2[lev][f] = qv;
+    if (own_ok) {
+      const float2 ql = f2(sq[lx].x, sq[ly].y);   // faces below, node t
+      // ---------------- C: beta of the cone at t - 1 ----------------
+      if (t > ta) {
+        const float4* bt = bslot + st_p * (K2 / 2) * kThreads;
+        float4* bn = a.betan + (i + obeta - P);
+        const float2 ns2 = f2(-s, -s), ts2 = f2(ts, ts);
+        float2 inc[5];
+        inc[0] = add2(sub2(zp[0], f2(1.f, 1.f)), f2(q0p, -q0p));
+        inc[1] = fma2(ns2, qlp, zp[1]);
+        inc[2] = fma2(ns2, qop, zp[2]);
+        inc[3] = fma2(ns2, ql, zp[3]);
+        inc[4] = fma2(ns2, qo, zp[4]);
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+          socp = fma2(inc[k], inc[k], socp);
+          bn[(long long)k * n0] = f4_of(ff2_add_f(ff2_of(bt[k * kThreads]), mul2(ts2, inc[k])));
         }
       }
-    }
-    __syncthreads();
-    // ---------------- C: beta of the owned cones at time t-1 ----------------
-    if (t - 1 >= ta && t - 1 < tb) {
-      const int lp = lev ^ 1;   // node t-1 faces; node t faces at lev
-#pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        if (!own_ok[r]) continue;
-        const int xo = lx + 8 * r;   // 0..15
-        const int x = x0 + xo, y = y0 + ly;
-        const long long i = (long long)(t - 1) * P + (long long)x * N1 + y;
-        const bool xl = x >= 1, xr = x <= g.N[0] - 2, yl = y >= 1, yr = y <= g.N[1] - 2;
-        float xv[K2 - 1];
-        xv[0] = q0p[r];
-        // x-faces j = x-1 (row xo) and j = x (row xo+1) of the tile's face list
-        xv[1] = xl ? sq1[lp][xo * TY + ly] : 0.f;
-        xv[2] = xr ? sq1[lp][(xo + 1) * TY + ly] : 0.f;
-        xv[3] = xl ? sq1[lev][xo * TY + ly] : 0.f;
-        xv[4] = xr ? sq1[lev][(xo + 1) * TY + ly] : 0.f;
-        // y-faces j = y-1 (column ly) and j = y (column ly+1)
-        xv[5] = yl ? sq2[lp][xo * (TY + 1) + ly] : 0.f;
-        xv[6] = yr ? sq2[lp][xo * (TY + 1) + ly + 1] : 0.f;
-        xv[7] = yl ? sq2[lev][xo * (TY + 1) + ly] : 0.f;
-        xv[8] = yr ? sq2[lev][xo * (TY + 1) + ly + 1] : 0.f;
-        const float s = a.somega ? a.somega[(long long)x * N1 + y] : s_def;
-        const float* z = zp[r];
-        float inc = (z[0] - 1.f) + xv[0];
-        socp = fmaf(inc, inc, socp);
-        a.betan[i] = ff_add_f(a.beta[i], ts * inc);
-#pragma unroll
-        for (int j = 1; j < K2 - 1; ++j) {
-          const long long o = (long long)j * n0 + i;
-          inc = fmaf(-s, xv[j], z[j]);
-          socp = fmaf(inc, inc, socp);
-          a.betan[o] = ff_add_f(a.beta[o], ts * inc);
+      qlp = ql;
+      // the next iteration's residual at node t: A^* w - c/sigma with w = q - alpha/sigma -
+      // A phi of the node's faces (sw and w0 hold -w, zero at the walls)
+      if (write_node) {
+        const float* wx = reinterpret_cast<const float*>(sw + lx);
+        const float* wy = reinterpret_cast<const float*>(sw + ly) + 1;
+        const ff2 dw = two_diff2(wo.h, f2(wx[0], wy[0]));
+        const float2 dl = add2(dw.l, sub2(wo.l, f2(wx[2], wy[2])));
+        const float2 ih = f2(ih1, ih2);
+        const ff2 pr = two_prod2(dw.h, ih);
+        const float2 pl = fma2(dl, ih, pr.l);
+        const float2 sxy = two_sum(pr.h.x, pr.h.y);
+        ff_acc acc{sxy.x, sxy.y + (pl.x + pl.y)};
+        float2 d0 = z2;
+        if (t < T) d0 = w0c;
+        if (t >= 1) {
+          const float2 e = two_sum(d0.x, -w0p.x);
+          d0 = f2(e.x, e.y + (d0.y - w0p.y));
         }
-        const long long o = (long long)(K2 - 1) * n0 + i;
-        inc = (z[K2 - 1] - 1.f) - xv[0];
-        socp = fmaf(inc, inc, socp);
-        a.betan[o] = ff_add_f(a.beta[o], ts * inc);
+        acc_add_mul(acc, d0, ih0);
+        if (t == 0) acc_add(acc, ff_neg(ff_mul(a.c0[slot * P + x * N1 + y], a.sp[slot].isg)));
+        if (t == T) acc_add(acc, ff_mul(a.c1[slot * P + x * N1 + y], a.sp[slot].isg));
+        a.r[i] = acc.h + acc.c;
       }
     }
-    // the current cone time becomes the previous one
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      q0p[r] = q0c[r];
-#pragma unroll
-      for (int j = 0; j < K2; ++j) zp[r][j] = zc[r][j];
+    // the sum of squared beta increments of a work unit that ends with cone t - 1
+    if (t > ta && (--left == 0 || t == T)) {
+      if (owner) {
+        double v = (double)socp.x + (double)socp.y;
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) wsum[warp] = v;
+        socp = z2;
+      }
+      *pend = entry++;
+      left = a.unit;
     }
-    __syncthreads();
+    qop = qo;
+    q0p = q0c;
+    w0p = w0c;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) zp[k] = zc[k];
+    const int s0 = st_p;
+    st_p = st_c;
+    st_c = st_n;
+    st_n = s0;
+    // no barrier here: step A of t + 1 writes z_1, z_3 (of the other level) and phi, last
+    // read in step B of t; step B of t + 1, which overwrites the face values read above,
+    // follows the barrier after A.  The neighbours read beta of stages t and t - 1 in
+    // step B of t; the copies into stage t - 1's place start after the second barrier.
   }
-  if (a.socp_part) {
-    // block sum of the beta increments' squares (the eta_P^soc term), FP64 tree
-    double v = (double)socp;
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    __shared__ double wsum[kThreads / 32];
-    if ((tid & 31) == 0) wsum[tid >> 5] = v;
-    __syncthreads();
-    if (tid == 0) {
-      double b = 0.0;
-      for (int w = 0; w < kThreads / 32; ++w) b += wsum[w];
-      a.socp_part[(chunk * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = b;
+}
+
+// Work units -- a slot's tile and a run of `unit` cone times -- in the order (active
+// slot, tile, time), cut into one contiguous run per CTA: every SM gets the same
+// number of cone times whatever the grid, and a CTA crosses from one tile to the next
+// at most once more than its share needs.  Each segment projects two cone times more
+// than it owns.
+template <int TX, bool MASKED>
+__global__ void __launch_bounds__(Tile<TX>::kThreads, 1) k_fused2d(const __grid_constant__ Geo g,
+                                                                  const __grid_constant__ FusedArgs a) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  __shared__ double wsum[TX];
+  __shared__ short act[256];
+  __shared__ int nact_s;
+  const int tid = threadIdx.x;
+  if (tid < 32) {   // the active slots, in order
+    int n = 0;
+    for (int b0 = 0; b0 < a.G; b0 += 32) {
+      const int b = b0 + tid;
+      const unsigned m = __ballot_sync(0xffffffffu, b < a.G && a.sp[b].active);
+      if (m >> tid & 1) act[n + __popc(m & ((1u << tid) - 1))] = (short)b;
+      n += __popc(m);
     }
+    if (tid == 0) nact_s = n;
   }
+  __syncthreads();
+  const int ntile = a.ntx * a.nty, nunit = a.nunit;
+  const long long total = (long long)nact_s * ntile * nunit;
+  long long k = total * blockIdx.x / gridDim.x;
+  const long long kend = total * (blockIdx.x + 1) / gridDim.x;
+  double* pend = nullptr;
+  while (k < kend) {
+    const int tl = (int)(k / nunit), u0 = (int)(k - (long long)tl * nunit);
+    const int u1 = (int)min((long long)nunit, u0 + (kend - k));
+    const int s = tl / ntile, tile = tl - s * ntile;
+    const int ty = tile / a.ntx, tx = tile - ty * a.ntx;
+    const int slot = act[s];
+    segment<TX, MASKED>(g, a, sm, wsum, slot, tx * TX, ty * TY, u0 * a.unit, min(g.T, u1 * a.unit),
+                        a.socp_part + ((long long)slot * ntile + tile) * nunit, &pend);
+    k += u1 - u0;
+  }
+  __syncthreads();
+  if (pend && tid == 0) {
+    double b = 0.0;
+    for (int w = 0; w < TX; ++w) b += wsum[w];
+    *pend = b;
+  }
+}
+
+int ntiles(const Geo& g, int tx) { return ((g.N[0] + tx - 1) / tx) * ((g.N[1] + TY - 1) / TY); }
+
+// Tile rows.  13 is the most (16 warps at 128 registers fill an SM) and has the
+// smallest halo; smaller tiles give small grids more CTAs and shorter time steps.
+// A CTA's pass takes its share of the cone times plus the two around each segment, at
+// a time per step that grows with the rows, so the choice is the least of that product
+// (with 1 + 0.2 rows for the step, the fit of: 32^2 x 16 11.7 us with 4 rows, 13.7 with
+// 8, 16.2 with 13; 64^2 x 32 25.1, 23.0, 24.8; 96^2 x 16 27.3, 24.8, 25.0; 128^2 x 32
+// 64.7, 53.9, 53.7; 150 x 117 x 37 78.3, 66.0, 63.6).
+int rows_of(const Geo& g, int G) {
+  const int rows[3] = {13, 8, 4};
+  int best = 13;
+  double t = 1e300;
+  for (int r : rows) {
+    const long long w = (long long)G * ntiles(g, r) * g.T;
+    const double e = (double)((w + kSMs - 1) / kSMs + 2) * (1.0 + 0.2 * r);
+    if (e < t) { t = e; best = r; }
+  }
+  return best;
+}
+
+// Cone times per work unit: about sixteen units per SM, at most eight.
+int unit_of(const Geo& g, int G) {
+  const long long u = (long long)G * ntiles(g, rows_of(g, G)) * g.T / (kSMs * 16);
+  return (int)(u < 1 ? 1 : u > 8 ? 8 : u);
+}
+
+template <int TX, bool MASKED>
+void launch(const Geo& g, const FusedArgs& a, int nb, cudaStream_t s) {
+  static std::atomic<unsigned long long> done{0};
+  smem_optin((const void*)k_fused2d<TX, MASKED>, Tile<TX>::kSmem, &done);
+  k_fused2d<TX, MASKED><<<nb, Tile<TX>::kThreads, Tile<TX>::kSmem, s>>>(g, a);
 }
 
 }  // namespace
 
 bool fused2d_supported(const Geo& g) { return g.D == 2; }
 
-long long fused2d_blocks(const Geo& g) {
-  const int tchunk = g.T <= 16 ? g.T : 16;
-  return (long long)((g.N[0] + TX - 1) / TX) * ((g.N[1] + TY - 1) / TY) * ((g.T + tchunk - 1) / tchunk);
+long long fused2d_partials(const Geo& g, int G) {
+  const int u = unit_of(g, G);
+  return (long long)ntiles(g, rows_of(g, G)) * ((g.T + u - 1) / u);
 }
 
-void launch_fused2d(const Geo& g, int G, const MxFields& f, const MxFields& fn, double* socp_part,
-                    cudaStream_t s, LaunchCounter lc) {
+void launch_fused2d(const Geo& g, int G, const MxFields& f, const MxFields& fn, double* socp_part, cudaStream_t s,
+                    LaunchCounter lc) {
   FusedArgs a;
   for (int d = 0; d < 3; ++d) {
     a.q[d] = f.q[d];
@@ -390,553 +526,31 @@ void launch_fused2d(const Geo& g, int G, const MxFields& f, const MxFields& fn, 
     a.qn[d] = fn.q[d];
     a.aln[d] = fn.al[d];
   }
-  a.beta = f.beta;
-  a.betan = fn.beta;
+  a.beta = reinterpret_cast<const float4*>(f.beta);
+  a.betan = reinterpret_cast<float4*>(fn.beta);
   a.phi = f.phi;
   a.somega = f.somega;
-  a.ts = 0.f;
-  a.tchunk = g.T <= 16 ? g.T : 16;
-  a.nchunk = (g.T + a.tchunk - 1) / a.tchunk;
+  a.G = G;
+  const int tx = rows_of(g, G);
+  a.ntx = (g.N[0] + tx - 1) / tx;
+  a.nty = (g.N[1] + TY - 1) / TY;
+  a.unit = unit_of(g, G);
+  a.nunit = (g.T + a.unit - 1) / a.unit;
   a.sp = f.sp;
   a.socp_part = socp_part;
-  a.socp_per_slot = fused2d_blocks(g);
-  a.err = nullptr;
-  a.r = nullptr;
-  a.c0 = a.c1 = nullptr;
-  dim3 grid((unsigned)((g.N[0] + TX - 1) / TX), (unsigned)((g.N[1] + TY - 1) / TY), (unsigned)(a.nchunk * G));
-  static std::atomic<unsigned long long> smem_done{0};
-  smem_optin((const void*)k_fused2d, kSmemFused, &smem_done);
-  k_fused2d<<<grid, kThreads, kSmemFused, s>>>(g, a);
-  lc.launched(KID_FUSED);
-}
-
-}  // namespace dot
-
-// ---------------------------------------------------------------------------
-// v2: the same pass with beta staged through shared memory by TMA.
-//
-// beta is three quarters of the pass's traffic.  One elected thread loads each
-// time step's beta tile -- all 10 components of a 10 x 36 (x, y) window around
-// the CTA's 8 x 32 tile -- with one 4-D TMA box into a ring of three buffers, so
-// the load for cone time t+1 runs while the CTA computes time t (buffer t-1 is
-// still needed by the faces and the beta update).  q, alpha and phi are small and
-// read directly.  Requires N_y even (TMA: 16-byte row strides and an even start
-// column for 8-byte elements).
-namespace dot {
-namespace {
-
-#ifndef FUSED_V2_VX
-#define FUSED_V2_VX 8
-#endif
-#ifndef FUSED_V2_THREADS
-#define FUSED_V2_THREADS 352
-#endif
-#ifndef FUSED_V2_TCHUNK
-#define FUSED_V2_TCHUNK 16
-#endif
-constexpr int VX = FUSED_V2_VX, VY = 32;     // owned tile: one cone per thread
-constexpr int VHX = VX + 2, VHY = VY + 2;    // cone halo 10 x 34
-constexpr int VNH = VHX * VHY;               // 340 cones
-constexpr int VBW = VY + 4;                  // beta tile columns: y in [y0-2, y0+34)
-constexpr int VNQ1 = (VX + 1) * VY;          // 288 x-faces: j in [x0-1, x0+7], y owned
-constexpr int VNQ2 = VX * (VY + 1);          // 264 y-faces: x owned, j in [y0-1, y0+31]
-constexpr int kBetaTile = K2 * VHX * VBW;    // 3600 two-floats = 28800 bytes
-constexpr int kBetaTileBytes = kBetaTile * 8;
-// z of the halo cones: components 1, 2, 5, 6 of cone time t (read by the faces of
-// node t) once, components 3, 4, 7, 8 (read by the faces of node t+1) for two
-// cone times
-constexpr int kOffZ = 3 * kBetaTileBytes;                 // ztn [4][VNH] floats
-constexpr int kOffZP = kOffZ + 4 * VNH * 4;               // ztp [2][4][VNH] floats
-constexpr int kOffQ1 = kOffZP + 2 * 4 * VNH * 4;          // [2][VNQ1] floats
-constexpr int kOffQ2 = kOffQ1 + 2 * VNQ1 * 4;             // [2][VNQ2] floats
-constexpr int kOffW1 = kOffQ2 + 2 * VNQ2 * 4;             // [VNQ1] two-float q - alpha/sigma - A phi
-constexpr int kOffW2 = kOffW1 + VNQ1 * 8;                 // [VNQ2] two-float
-constexpr int kOffBar = (kOffW2 + VNQ2 * 8 + 15) / 16 * 16;
-constexpr int kSmemV2 = kOffBar + 64;
-static_assert(kOffW1 % 16 == 0, "two-float face arrays are 16-byte aligned");
-// 11 warps: one thread per cone of the 10 x 34 halo rectangle (256 owned + 84
-// ring cones), so phase A takes one round; 552 faces take two
-constexpr int kThreadsV2 = FUSED_V2_THREADS;
-static_assert(kThreadsV2 >= VX * VY + 2 * (VX + VY + 2) && kThreadsV2 % 32 == 0, "a thread per halo cone");
-constexpr int kMinBlocksV2 = FUSED_V2_MIN_BLOCKS;
-// most cone times per CTA (fused2d_tma_tchunk)
-constexpr int kTchunkV2 = FUSED_V2_TCHUNK;
-
-__device__ __forceinline__ uint32_t sa(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ bool bar_wait(uint64_t* bar, unsigned parity) { return mbar_wait_bounded(sa(bar), parity); }
-
-__device__ __forceinline__ void issue_beta(const CUtensorMap* tm, float2* dst, uint64_t* bar, int y, int x, int t,
-                                           int slot) {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(sa(bar)), "r"(kBetaTileBytes)
-               : "memory");
-  asm volatile(
-      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6, %7}], [%2];"
-      ::"r"(sa(dst)), "l"(tm), "r"(sa(bar)), "r"(y), "r"(x), "r"(t), "r"(0), "r"(slot)
-      : "memory");
-}
-
-// beta of halo cone (xh, yh) component c in a tile (column yw = yh + 1)
-__device__ __forceinline__ float2 bt(const float2* tile, int c, int xh, int yh) {
-  return tile[(c * VHX + xh) * VBW + yh + 1];
-}
-
-// z components 1..8 of a halo cone into the tiles, from the lane pairs of
-// ff2_proj_soc10: (1, 2), (5, 6) -> ztn; (3, 4), (7, 8) -> ztp
-__device__ __forceinline__ void put_z(float (*ztn)[VNH], float (*ztp)[VNH], int hc, const ff2* P) {
-  const float2 r1 = add2(P[1].h, P[1].l), r2 = add2(P[2].h, P[2].l);
-  const float2 r3 = add2(P[3].h, P[3].l), r4 = add2(P[4].h, P[4].l);
-  ztn[0][hc] = r1.x;
-  ztn[1][hc] = r1.y;
-  ztn[2][hc] = r3.x;
-  ztn[3][hc] = r3.y;
-  ztp[0][hc] = r2.x;
-  ztp[1][hc] = r2.y;
-  ztp[2][hc] = r4.x;
-  ztp[3][hc] = r4.y;
-}
-__device__ __forceinline__ void put_z0(float (*ztn)[VNH], float (*ztp)[VNH], int hc) {
-#pragma unroll
-  for (int v = 0; v < 4; ++v) {
-    ztn[v][hc] = 0.f;
-    ztp[v][hc] = 0.f;
-  }
-}
-// The q^k values a cone (t, x, y) reads: q_0 at the cone, and the q_1, q_2 faces on
-// either side of it on time nodes t (v = 1, 2) and t+1 (v = 3, 4), zero where F
-// has no source face.  A thread keeps its cone column for all cone times, and the
-// node-(t+1) values of cone t are the node-t values of cone t+1, so per cone time
-// it loads q_0 and the node-(t+1) pairs only.
-struct ConeQ {
-  float x0;
-  float2 xb, xd;   // (q_1 left, right), (q_2 left, right) on node t+1
-};
-__device__ __forceinline__ void load_cone_q(const Geo& g, const FusedArgs& a, int t, int x, int y, ConeQ* c) {
-  const int P_ = (int)g.P, N1 = g.N[1];
-  const int i = t * P_ + x * N1 + y;
-  const bool xl = x >= 1, xr = x <= g.N[0] - 2, yl = y >= 1, yr = y <= g.N[1] - 2;
-  c->x0 = a.q[0][i];
-  c->xb = make_float2(xl ? a.q[1][i + P_ - N1] : 0.f, xr ? a.q[1][i + P_] : 0.f);
-  c->xd = make_float2(yl ? a.q[2][i + P_ - 1] : 0.f, yr ? a.q[2][i + P_] : 0.f);
-}
-// the node-t pairs (at the first cone time of a chunk)
-__device__ __forceinline__ void load_cone_q_node(const Geo& g, const FusedArgs& a, int t, int x, int y, float2* xa,
-                                                 float2* xc) {
-  const int P_ = (int)g.P, N1 = g.N[1];
-  const int i = t * P_ + x * N1 + y;
-  const bool xl = x >= 1, xr = x <= g.N[0] - 2, yl = y >= 1, yr = y <= g.N[1] - 2;
-  *xa = make_float2(xl ? a.q[1][i - N1] : 0.f, xr ? a.q[1][i] : 0.f);
-  *xc = make_float2(yl ? a.q[2][i - 1] : 0.f, yr ? a.q[2][i] : 0.f);
-}
-// z of a cone from its q^k values and its beta tile entries, in two-float
-// arithmetic, as five lane pairs P[0] = (z_0, z_9), P[k] = (z_{2k-1}, z_{2k}).
-__device__ __forceinline__ void cone_z(float x0, float2 xa, float2 xb, float2 xc, float2 xd, float s,
-                                       const float2* tile, int xh, int yh, ff2* P) {
-  const float2 s2 = make_float2(s, s);
-  // y = B F q + d - beta/sigma: (1 - x_0, s x_1, ..., s x_8, 1 + x_0) - beta/sigma
-  P[0] = ff2_add(two_sum2(make_float2(-x0, x0), make_float2(1.f, 1.f)),
-                 ff2_neg(ff2_pack(bt(tile, 0, xh, yh), bt(tile, K2 - 1, xh, yh))));
-  P[1] = ff2_add(two_prod2(s2, xa), ff2_neg(ff2_pack(bt(tile, 1, xh, yh), bt(tile, 2, xh, yh))));
-  P[2] = ff2_add(two_prod2(s2, xb), ff2_neg(ff2_pack(bt(tile, 3, xh, yh), bt(tile, 4, xh, yh))));
-  P[3] = ff2_add(two_prod2(s2, xc), ff2_neg(ff2_pack(bt(tile, 5, xh, yh), bt(tile, 6, xh, yh))));
-  P[4] = ff2_add(two_prod2(s2, xd), ff2_neg(ff2_pack(bt(tile, 7, xh, yh), bt(tile, 8, xh, yh))));
-  ff2_proj_soc10(P);
-}
-
-__device__ __forceinline__ float2 grad_of(float2 a, float2 b, float invh) {
-  const float2 dh = two_sum(b.x, -a.x);
-  const float dl = (b.y - a.y) + dh.y;
-  return make_float2(dh.x * invh, dl * invh);
-}
-
-// One space face's update (line 4-5 of Algorithm 2 for q_d, alpha_d at one face):
-// rhs = A_d phi + alpha/sigma + sum over the cones reading the face of
-// s (z + beta/sigma), q = rhs / (1 + sum s^2), alpha/sigma += tau (A_d phi - q).
-// Returns q; *w = q - alpha/sigma - A_d phi (the next residual's face term).
-__device__ __forceinline__ float face_update(float2 gp, float2 al, bool has_now, bool has_prev, float2 bnr,
-                                             float2 bnl, float2 bpr, float2 bpl, float znr, float znl, float zpr,
-                                             float zpl, float sr, float sl, float ts, float2* alnew, float2* w) {
-  ff_acc acc = acc_init(gp);
-  acc_add(acc, al);
-  float zs = 0.f, dg = 0.f;
-  if (has_now) {
-    acc_add_mul(acc, bnr, sr);
-    acc_add_mul(acc, bnl, sl);
-    zs += sr * znr + sl * znl;
-    dg += sr * sr + sl * sl;
-  }
-  if (has_prev) {
-    acc_add_mul(acc, bpr, sr);
-    acc_add_mul(acc, bpl, sl);
-    zs += sr * zpr + sl * zpl;
-    dg += sr * sr + sl * sl;
-  }
-  acc_add_f(acc, zs);
-  const float den = 1.f + dg;
-  const float qv = ff_round(ff_div_f_r(acc_get(acc), den, __frcp_rn(den)));
-  const float gm = grad_minus(gp, qv);
-  *alnew = ff_add_f(al, ts * gm);
-  *w = ff_add_f(ff_neg(*alnew), -gm);
-  return qv;
-}
-
-__global__ void __launch_bounds__(kThreadsV2, kMinBlocksV2) k_fused2d_tma(const __grid_constant__ CUtensorMap tmb, Geo g,
-                                                        FusedArgs a_in) {
-  const int slot = blockIdx.z / a_in.nchunk, chunk = blockIdx.z - slot * a_in.nchunk;
-  if (!a_in.sp[slot].active) return;
-  const FusedArgs a = fused_slot(a_in, g, slot);
-  extern __shared__ __align__(128) unsigned char sm[];
-  float2* btiles = reinterpret_cast<float2*>(sm);
-  float (*ztn)[VNH] = reinterpret_cast<float (*)[VNH]>(sm + kOffZ);
-  float (*ztp)[4][VNH] = reinterpret_cast<float (*)[4][VNH]>(sm + kOffZP);
-  float (*sq1)[VNQ1] = reinterpret_cast<float (*)[VNQ1]>(sm + kOffQ1);
-  float (*sq2)[VNQ2] = reinterpret_cast<float (*)[VNQ2]>(sm + kOffQ2);
-  float2* sw1 = reinterpret_cast<float2*>(sm + kOffW1);
-  float2* sw2 = reinterpret_cast<float2*>(sm + kOffW2);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sm + kOffBar);
-
-  const int tid = threadIdx.x;
-  const bool owner = tid < VX * VY;             // threads 0..255 own a cone column
-  const int ly = tid & 31, lx = tid >> 5;       // owned node (x0 + lx, y0 + ly)
-  const int x0 = blockIdx.x * VX, y0 = blockIdx.y * VY;
-  const int ta = chunk * a.tchunk;
-  const int tb = min(g.T, ta + a.tchunk);
-  const bool last_chunk = (tb == g.T);
-  const int P = (int)g.P, n0 = g.T * P, N1 = g.N[1];
-  const float ts = a.ts;
-  const float ih0 = (float)g.invh[0], ih1 = (float)g.invh[1], ih2 = (float)g.invh[2];
-  const float s_def = 0.70710678118654752f;
-  const int xo = x0 + lx, yo = y0 + ly;
-  const bool own_ok = owner && xo < g.N[0] && yo < g.N[1];
-  const int tstart = ta > 0 ? ta - 1 : 0;
-  const int tlast_cone = min(tb, g.T - 1);      // last cone time whose beta tile is loaded
-
-  // this thread's cone column: its owned cone, or one of the 84 halo-ring cones
-  // (threads 256..339); the same for every cone time
-  int cxh = -1, cyh = -1;
-  if (owner) {
-    cxh = lx + 1;
-    cyh = ly + 1;
-  } else if (tid < VNH) {
-    int r = tid - VX * VY;
-    if (r < VHY) { cxh = 0; cyh = r; }
-    else if ((r -= VHY) < VHY) { cxh = VHX - 1; cyh = r; }
-    else if ((r -= VHY) < VHX - 2) { cxh = 1 + r; cyh = 0; }
-    else { r -= VHX - 2; cxh = 1 + r; cyh = VHY - 1; }
-  }
-  const int cx = x0 - 1 + cxh, cy = y0 - 1 + cyh, chc = cxh * VHY + cyh;
-  const bool cone_ok = cxh >= 0 && cx >= 0 && cy >= 0 && cx < g.N[0] && cy < g.N[1];
-  const float cs = (cone_ok && a.somega) ? a.somega[cx * N1 + cy] : s_def;
-  // q^k of the cone column (node-t pairs and the next cone time's values), and the
-  // owner's potential on node t and alpha_0 / sigma of its cone, loaded a step ahead
-  float2 xa = make_float2(0.f, 0.f), xc = make_float2(0.f, 0.f);
-  ConeQ cq;
-  cq.x0 = 0.f;
-  cq.xb = cq.xd = make_float2(0.f, 0.f);
-  float2 ph_t = make_float2(0.f, 0.f), ph_n = make_float2(0.f, 0.f), al0 = make_float2(0.f, 0.f);
-  if (cone_ok && tstart <= g.T - 1) {
-    load_cone_q_node(g, a, tstart, cx, cy, &xa, &xc);
-    load_cone_q(g, a, tstart, cx, cy, &cq);
-    if (owner && tstart < tb) {
-      const int i = tstart * P + xo * N1 + yo;
-      ph_t = a.phi[i];
-      ph_n = a.phi[i + P];
-      al0 = a.al[0][i];
-    }
-  }
-
-  if (tid == 0) {
-    for (int b = 0; b < 3; ++b)
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sa(&bars[b])));
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncthreads();
-  unsigned phase[3] = {0u, 0u, 0u};
-  bool inflight[3] = {false, false, false};   // meaningful on the issuing thread
-  if (tid == 0 && tstart <= tlast_cone) {
-    issue_beta(&tmb, btiles + (tstart % 3) * kBetaTile, &bars[tstart % 3], y0 - 2, x0 - 1, tstart, slot);
-    inflight[tstart % 3] = true;
-  }
-
-  // FP32 z of the owned cone at times t (zc) and t-1 (zp), lane pairs as ff2_proj_soc10
-  float2 zc[5], zp[5];
-#pragma unroll
-  for (int k = 0; k < 5; ++k) zc[k] = zp[k] = make_float2(0.f, 0.f);
-  float q0c = 0.f, q0p = 0.f;
-  float2 socp = make_float2(0.f, 0.f);
-  float2 w0c = make_float2(0.f, 0.f), w0p = make_float2(0.f, 0.f);   // q_0 - alpha_0/sigma - A_0 phi, cones t, t-1
-  bool failed = false;
-
-  for (int t = tstart; t <= tb; ++t) {
-    const int lev = t & 1, lp = lev ^ 1;
-    const int bcur = t % 3, bprev = (t + 2) % 3;
-    const float2* tcur = btiles + bcur * kBetaTile;
-    const float2* tprev = btiles + bprev * kBetaTile;
-    // every thread waits for the tile of cone time t itself; a wait that gives up
-    // is made uniform at the barrier after step A
-    bool ok = true;
-    if (t <= g.T - 1) {
-      ok = bar_wait(&bars[bcur], phase[bcur]);
-      if (ok) {
-        phase[bcur] ^= 1u;
-        inflight[bcur] = false;
-      }
-    }
-    // ---------------- A: cones at time t ----------------
-    if (t <= g.T - 1 && cxh >= 0) {
-      if (cone_ok) {
-        ff2 z[5];
-        cone_z(cq.x0, xa, cq.xb, xc, cq.xd, cs, tcur, cxh, cyh, z);
-        put_z(ztn, ztp[lev], chc, z);
-        // the cone before the chunk (t = ta - 1) is updated for the residual only
-        if (owner && t < tb) {
-          const int i = t * P + xo * N1 + yo;
-          const float2 gp = grad_of(ph_t, ph_n, ih0);
-          const float2 al = al0;
-          // q_0 (diagonal 3): rhs = A_0 phi + alpha_0/sigma + u_9 - u_0 with
-          // u = z + beta/sigma (F^*B^* of components 0 and K-1)
-          const ff2 u = ff2_add(z[0], ff2_pack(bt(tcur, 0, cxh, cyh), bt(tcur, K2 - 1, cxh, cyh)));
-          ff_acc acc = acc_init(gp);
-          acc_add(acc, al);
-          acc_add(acc, ff2_lane1(u));
-          acc_add(acc, ff_neg(ff2_lane0(u)));
-          const float qn = ff_round(ff_div_f_r(acc_get(acc), 3.f, 1.f / 3.f));
-          const float gm = grad_minus(gp, qn);
-          const float2 aln = ff_add_f(al, ts * gm);
-          if (t >= ta) {
-            a.qn[0][i] = qn;
-            a.aln[0][i] = aln;
-          }
-          q0c = qn;
-          w0c = ff_add_f(ff_neg(aln), -gm);   // q - alpha/sigma - A phi
-          // the next cone time's potential and alpha_0 / sigma
-          ph_t = ph_n;
-          if (t + 1 < tb) {
-            ph_n = a.phi[i + 2 * P];
-            al0 = a.al[0][i + P];
-          }
-        }
-        if (owner) {
-#pragma unroll
-          for (int k = 0; k < 5; ++k) zc[k] = add2(z[k].h, z[k].l);
-        }
-        // the next cone time's q^k: node t+1 pairs move down, the rest is loaded now
-        xa = cq.xb;
-        xc = cq.xd;
-        if (t + 1 <= tlast_cone) load_cone_q(g, a, t + 1, cx, cy, &cq);
-      } else {
-        put_z0(ztn, ztp[lev], chc);
-      }
-    }
-    if (__syncthreads_or(!ok)) { failed = true; break; }
-    // prefetch the next cone time's beta into buffer (t+1) % 3 = (t-2) % 3, whose
-    // last reader (step C of t-1) every thread has left at the barrier above
-    if (tid == 0 && t + 1 <= tlast_cone) {
-      const int nb = (t + 1) % 3;
-      issue_beta(&tmb, btiles + nb * kBetaTile, &bars[nb], y0 - 2, x0 - 1, t + 1, slot);
-      inflight[nb] = true;
-    }
-    // ---------------- B: faces at time node t ----------------
-    const bool write_node = t >= ta && ((t < tb) || (last_chunk && t == g.T));
-    if (t >= ta) {
-      const bool has_now = t <= g.T - 1, has_prev = t >= 1;
-      const float2 z2 = make_float2(0.f, 0.f);
-      for (int e = tid; e < VNQ1 + VNQ2; e += kThreadsV2) {
-        if (e < VNQ1) {
-          const int jx = e / VY, yy = e % VY;
-          const int j = x0 - 1 + jx, y = y0 + yy;
-          float qv = 0.f;
-          float2 wv = z2;
-          if (j >= 0 && j <= g.N[0] - 2 && y < g.N[1]) {
-            const int i = t * P + j * N1 + y;
-            const int xr = jx + 1, xl = jx, yh = yy + 1;
-            const float sr = a.somega ? a.somega[(j + 1) * N1 + y] : s_def;
-            const float sl = a.somega ? a.somega[j * N1 + y] : s_def;
-            float2 aln;
-            qv = face_update(grad_pair(a.phi, i, i + N1, ih1), a.al[1][i], has_now, has_prev,
-                             has_now ? bt(tcur, 1, xr, yh) : z2, has_now ? bt(tcur, 2, xl, yh) : z2,
-                             has_prev ? bt(tprev, 3, xr, yh) : z2, has_prev ? bt(tprev, 4, xl, yh) : z2,
-                             ztn[0][xr * VHY + yh], ztn[1][xl * VHY + yh], ztp[lp][0][xr * VHY + yh],
-                             ztp[lp][1][xl * VHY + yh], sr, sl, ts, &aln, &wv);
-            if (write_node && jx >= 1) {
-              a.qn[1][i] = qv;
-              a.aln[1][i] = aln;
-            }
-          }
-          sq1[lev][e] = qv;
-          sw1[e] = wv;
-        } else {
-          const int f = e - VNQ1;
-          const int xx = f / (VY + 1), jy = f % (VY + 1);
-          const int x = x0 + xx, j = y0 - 1 + jy;
-          float qv = 0.f;
-          float2 wv = z2;
-          if (x < g.N[0] && j >= 0 && j <= g.N[1] - 2) {
-            const int i = t * P + x * N1 + j;
-            const int xh = xx + 1, yr = jy + 1, yl = jy;
-            const float sr = a.somega ? a.somega[x * N1 + j + 1] : s_def;
-            const float sl = a.somega ? a.somega[x * N1 + j] : s_def;
-            float2 aln;
-            qv = face_update(grad_pair(a.phi, i, i + 1, ih2), a.al[2][i], has_now, has_prev,
-                             has_now ? bt(tcur, 5, xh, yr) : z2, has_now ? bt(tcur, 6, xh, yl) : z2,
-                             has_prev ? bt(tprev, 7, xh, yr) : z2, has_prev ? bt(tprev, 8, xh, yl) : z2,
-                             ztn[2][xh * VHY + yr], ztn[3][xh * VHY + yl], ztp[lp][2][xh * VHY + yr],
-                             ztp[lp][3][xh * VHY + yl], sr, sl, ts, &aln, &wv);
-            if (write_node && jy >= 1) {
-              a.qn[2][i] = qv;
-              a.aln[2][i] = aln;
-            }
-          }
-          sq2[lev][f] = qv;
-          sw2[f] = wv;
-        }
-      }
-    }
-    __syncthreads();
-    // ---------------- C: beta of the owned cone at time t-1 ----------------
-    if (own_ok && t - 1 >= ta && t - 1 < tb) {
-      const int i = (t - 1) * P + xo * N1 + yo;
-      const bool xl = xo >= 1, xr = xo <= g.N[0] - 2, yl = yo >= 1, yr = yo <= g.N[1] - 2;
-      const float2 xa = make_float2(xl ? sq1[lp][lx * VY + ly] : 0.f, xr ? sq1[lp][(lx + 1) * VY + ly] : 0.f);
-      const float2 xb = make_float2(xl ? sq1[lev][lx * VY + ly] : 0.f, xr ? sq1[lev][(lx + 1) * VY + ly] : 0.f);
-      const float2 xc = make_float2(yl ? sq2[lp][lx * (VY + 1) + ly] : 0.f, yr ? sq2[lp][lx * (VY + 1) + ly + 1] : 0.f);
-      const float2 xd = make_float2(yl ? sq2[lev][lx * (VY + 1) + ly] : 0.f, yr ? sq2[lev][lx * (VY + 1) + ly + 1] : 0.f);
-      const float s = a.somega ? a.somega[xo * N1 + yo] : s_def;
-      const int xh = lx + 1, yh = ly + 1;
-      const float2 ns2 = make_float2(-s, -s), ts2 = make_float2(ts, ts);
-      // increments z - B F q^{k+1} - d, lane pairs as zp
-      float2 inc[5];
-      inc[0] = add2(sub2(zp[0], make_float2(1.f, 1.f)), make_float2(q0p, -q0p));
-      inc[1] = fma2(ns2, xa, zp[1]);
-      inc[2] = fma2(ns2, xb, zp[2]);
-      inc[3] = fma2(ns2, xc, zp[3]);
-      inc[4] = fma2(ns2, xd, zp[4]);
-#pragma unroll
-      for (int k = 0; k < 5; ++k) socp = fma2(inc[k], inc[k], socp);
-      const int c0 = 0, c1 = K2 - 1;
-      ff2 B = ff2_add_f(ff2_pack(bt(tprev, c0, xh, yh), bt(tprev, c1, xh, yh)), mul2(ts2, inc[0]));
-      a.betan[c0 * n0 + i] = ff2_lane0(B);
-      a.betan[c1 * n0 + i] = ff2_lane1(B);
-#pragma unroll
-      for (int k = 1; k <= 4; ++k) {
-        const int j = 2 * k - 1;
-        B = ff2_add_f(ff2_pack(bt(tprev, j, xh, yh), bt(tprev, j + 1, xh, yh)), mul2(ts2, inc[k]));
-        a.betan[j * n0 + i] = ff2_lane0(B);
-        a.betan[(j + 1) * n0 + i] = ff2_lane1(B);
-      }
-    }
-    // the next iteration's residual at the owned node of time t:
-    // r = A^*(q - alpha/sigma) - c/sigma - A^*A phi = A^*(q - alpha/sigma - A phi) - c/sigma,
-    // with q - alpha/sigma - A phi of the node's faces from steps A and B
-    if (a.r && own_ok && write_node) {
-      const int i = t * P + xo * N1 + yo;
-      const int p = xo * N1 + yo;
-      ff_acc acc{0.f, 0.f};
-      if (t >= 1) acc_add_mul(acc, w0p, ih0);
-      if (t < g.T) acc_add_mul(acc, w0c, -ih0);
-      // faces j = x - 1 / x (and y - 1 / y); the slots beyond the walls hold zero
-      acc_add_mul(acc, sw1[lx * VY + ly], ih1);
-      acc_add_mul(acc, sw1[(lx + 1) * VY + ly], -ih1);
-      acc_add_mul(acc, sw2[lx * (VY + 1) + ly], ih2);
-      acc_add_mul(acc, sw2[lx * (VY + 1) + ly + 1], -ih2);
-      if (t == 0) acc_add(acc, ff_neg(ff_mul(a.c0[p], a.isg)));
-      if (t == g.T) acc_add(acc, ff_mul(a.c1[p], a.isg));
-      a.r[i] = acc.h + acc.c;
-    }
-    q0p = q0c;
-    w0p = w0c;
-#pragma unroll
-    for (int k = 0; k < 5; ++k) zp[k] = zc[k];
-    // no barrier here: step A of t+1 writes only ztn and ztp[lev of t+1] (read by
-    // step B of t, which every thread finished before step C) and registers; step B
-    // of t+1, which overwrites the faces step C reads, follows the barrier after A
-  }
-  if (failed) {
-    // a tile load did not complete in time: wait (bounded) for the loads this
-    // CTA still has in flight, then report through the error flag
-    if (tid == 0) {
-      for (int b = 0; b < 3; ++b)
-        if (inflight[b]) bar_wait(&bars[b], phase[b]);
-      atomicExch(a.err, 1);
-    }
-    return;
-  }
-  if (a.socp_part) {
-    double v = (double)socp.x + (double)socp.y;
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    __shared__ double wsum[kThreadsV2 / 32];
-    if ((tid & 31) == 0) wsum[tid >> 5] = v;
-    __syncthreads();
-    if (tid == 0) {
-      double b = 0.0;
-      for (int w = 0; w < kThreadsV2 / 32; ++w) b += wsum[w];
-      a.socp_part[(chunk * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = b;
-    }
-  }
-}
-
-}  // namespace
-}  // namespace dot
-
-namespace dot {
-
-bool fused2d_tma_supported(const Geo& g) { return g.D == 2 && g.N[1] % 2 == 0; }
-
-// Cone times per CTA for a batch of G solves of grid g: kTchunkV2, halved (down to 2)
-// while the launch would have fewer than 256 CTAs, so that small grids still occupy
-// the GPU (measured: 128^2 x 32 80 -> 60 us per launch with 8, 32^2 x 16 66 -> 19 us
-// with 2); each chunk recomputes one cone time before it (1/tchunk extra work).
-int fused2d_tma_tchunk(const Geo& g, int G) {
-  const long long tiles = (long long)((g.N[0] + VX - 1) / VX) * ((g.N[1] + VY - 1) / VY) * G;
-  int tc = g.T <= kTchunkV2 ? g.T : kTchunkV2;
-  while (tc > 2 && tiles * ((g.T + tc - 1) / tc) < 256) tc = (tc + 1) / 2;
-  return tc;
-}
-
-long long fused2d_tma_blocks(const Geo& g, int G) {
-  const int tchunk = fused2d_tma_tchunk(g, G);
-  return (long long)((g.N[0] + VX - 1) / VX) * ((g.N[1] + VY - 1) / VY) * ((g.T + tchunk - 1) / tchunk);
-}
-
-bool launch_fused2d_tma(const Geo& g, int G, const MxFields& f, const MxFields& fn, double* socp_part, int* err,
-                        bool residual, cudaStream_t s, LaunchCounter lc) {
-  FusedArgs a;
-  for (int d = 0; d < 3; ++d) {
-    a.q[d] = f.q[d];
-    a.al[d] = f.al[d];
-    a.qn[d] = fn.q[d];
-    a.aln[d] = fn.al[d];
-  }
-  a.beta = f.beta;
-  a.betan = fn.beta;
-  a.phi = f.phi;
-  a.somega = f.somega;
-  a.ts = 0.f;
-  a.tchunk = fused2d_tma_tchunk(g, G);
-  a.nchunk = (g.T + a.tchunk - 1) / a.tchunk;
-  a.sp = f.sp;
-  a.socp_part = socp_part;
-  a.socp_per_slot = fused2d_tma_blocks(g, G);
-  a.err = err;
-  a.r = residual ? f.r : nullptr;
+  a.r = f.r;
   a.c0 = f.c0;
   a.c1 = f.c1;
-  a.isg = make_float2(0.f, 0.f);
-  // beta as a 5-D tensor of 8-byte elements: (y, x, t, component, slot)
-  CUtensorMap tm;
-  const cuuint64_t dims[5] = {(cuuint64_t)g.N[1], (cuuint64_t)g.N[0], (cuuint64_t)g.T, (cuuint64_t)K2,
-                              (cuuint64_t)G};
-  const cuuint64_t str[4] = {(cuuint64_t)g.N[1] * 8, (cuuint64_t)g.P * 8, (cuuint64_t)g.T * g.P * 8,
-                             (cuuint64_t)K2 * g.T * g.P * 8};
-  const cuuint32_t box[5] = {VBW, VHX, 1, K2, 1};
-  if (!encode_tensor_map(&tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 5, f.beta, dims, str, box)) return false;
-  static std::atomic<unsigned long long> smem_done{0};
-  smem_optin((const void*)k_fused2d_tma, kSmemV2, &smem_done);
-  dim3 grid((unsigned)((g.N[0] + VX - 1) / VX), (unsigned)((g.N[1] + VY - 1) / VY), (unsigned)(a.nchunk * G));
-  k_fused2d_tma<<<grid, kThreadsV2, kSmemV2, s>>>(tm, g, a);
+  a.ih0 = (float)g.invh[0];
+  a.ih1 = (float)g.invh[1];
+  a.ih2 = (float)g.invh[2];
+  const long long units = (long long)G * a.ntx * a.nty * a.nunit;
+  const int nb = (int)(units < kSMs ? units : kSMs);
+  const bool m = f.somega != nullptr;
+  if (tx == 13) m ? launch<13, true>(g, a, nb, s) : launch<13, false>(g, a, nb, s);
+  else if (tx == 8) m ? launch<8, true>(g, a, nb, s) : launch<8, false>(g, a, nb, s);
+  else m ? launch<4, true>(g, a, nb, s) : launch<4, false>(g, a, nb, s);
   lc.launched(KID_FUSED);
-  return true;
 }
 
 }  // namespace dot

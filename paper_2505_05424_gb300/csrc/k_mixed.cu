@@ -237,7 +237,16 @@ __global__ void k_rescale(Geo g, MxFields fb) {
 #pragma unroll
   for (int d = 0; d < D; ++d)
     for (long long i = i0; i < nn; i += stride) f.al[1 + d][i] = ff_mul(f.al[1 + d][i], sp.rescale);
-  for (long long i = i0; i < (long long)g.K * n0; i += stride) f.beta[i] = ff_mul(f.beta[i], sp.rescale);
+  if (D == 2) {
+    float4* b = reinterpret_cast<float4*>(f.beta);
+    for (long long i = i0; i < (long long)(g.K / 2) * n0; i += stride) {
+      const float4 v = b[i];
+      const float2 p = ff_mul(make_float2(v.x, v.z), sp.rescale), q = ff_mul(make_float2(v.y, v.w), sp.rescale);
+      b[i] = make_float4(p.x, q.x, p.y, q.y);
+    }
+  } else {
+    for (long long i = i0; i < (long long)g.K * n0; i += stride) f.beta[i] = ff_mul(f.beta[i], sp.rescale);
+  }
 }
 
 // phi^{k+1} = phi^k + delta (delta in phi1).
@@ -263,6 +272,21 @@ __global__ void k_combine(Geo g, MxFields fb, float2* __restrict__ out) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x)
     phi[i] = two_sum(phi1[i], delta[i]);
+}
+
+// beta / sigma of component j at cone i, and its high part alone.
+template <int D>
+__device__ __forceinline__ float2 beta_ff(const float2* beta, int j, long long i, long long n0) {
+  if (D == 2) {
+    const float* p = reinterpret_cast<const float*>(beta) + beta2_at(j, i, n0);
+    return make_float2(p[0], p[2]);
+  }
+  return beta[(long long)j * n0 + i];
+}
+template <int D>
+__device__ __forceinline__ float beta_hi(const float2* beta, int j, long long i, long long n0) {
+  if (D == 2) return reinterpret_cast<const float*>(beta)[beta2_at(j, i, n0)];
+  return beta[(long long)j * n0 + i].x;
 }
 
 template <int D>
@@ -359,7 +383,7 @@ __device__ __forceinline__ void kkt_cone(const Geo& g, const MxFields& f, float 
     r = (f.z[(long long)(K - 1) * n0 + i] - 1.f) - q0;
     acc[R_SOCP] += r * r;
   }
-  const float2 bK = f.beta[(long long)(K - 1) * n0 + i], b0 = f.beta[i];
+  const float2 bK = beta_ff<D>(f.beta, K - 1, i, n0), b0 = beta_ff<D>(f.beta, 0, i, n0);
   const float fbb = sg * ((bK.x - b0.x) + (bK.y - b0.y));
   acc[R_SOCD] += (fbb + a0) * (fbb + a0);
   acc[R_FBB] += fbb * fbb;
@@ -388,12 +412,11 @@ __device__ __forceinline__ void kkt_face(const Geo& g, const MxFields& f, float 
   const float s_l = f.somega ? f.somega[p] : s_default, s_r = f.somega ? f.somega[p + s] : s_default;
   if (t <= g.T - 1) {
     den += om_r * a0[i + s].x + om_l * a0[i].x;
-    fbb += s_r * f.beta[(long long)(cbase + 0) * n0 + i + s].x + s_l * f.beta[(long long)(cbase + 1) * n0 + i].x;
+    fbb += s_r * beta_hi<D>(f.beta, cbase + 0, i + s, n0) + s_l * beta_hi<D>(f.beta, cbase + 1, i, n0);
   }
   if (t >= 1) {
     den += om_r * a0[i - g.P + s].x + om_l * a0[i - g.P].x;
-    fbb += s_r * f.beta[(long long)(cbase + 2) * n0 + i - g.P + s].x +
-           s_l * f.beta[(long long)(cbase + 3) * n0 + i - g.P].x;
+    fbb += s_r * beta_hi<D>(f.beta, cbase + 2, i - g.P + s, n0) + s_l * beta_hi<D>(f.beta, cbase + 3, i - g.P, n0);
   }
   den *= 0.25f * sg;
   fbb *= sg;

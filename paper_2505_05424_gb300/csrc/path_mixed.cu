@@ -36,9 +36,6 @@ struct MixedBatch::Buffers {
 
 namespace {
 
-// per-slot partial sums of |z - BFq - d|^2 written by either fused kernel for a batch of G
-long long socp_blocks(const Geo& g, int G) { return std::max(fused2d_blocks(g), fused2d_tma_blocks(g, G)); }
-
 void carve(const Geo& g, int G, bool masks, Carver& cv, MixedBatch::Buffers* B) {
   const size_t nn = (size_t)(g.T + 1) * g.P, n0 = (size_t)g.T * g.P, P = (size_t)g.P;
   const size_t Gs = (size_t)G;
@@ -62,7 +59,7 @@ void carve(const Geo& g, int G, bool masks, Carver& cv, MixedBatch::Buffers* B) 
   }
   if (fused2d_supported(g)) {
     B->f.z = nullptr;                       // z never leaves the fused kernel
-    B->socp = cv.take<double>(Gs * socp_blocks(g, G));
+    B->socp = cv.take<double>(Gs * fused2d_partials(g, G));
   } else {
     B->f.z = cv.take<float>(Gs * g.K * n0);
     B->socp = nullptr;
@@ -163,7 +160,6 @@ int MixedBatch::init(char* ws, size_t bytes, cudaStream_t s, std::string* err) {
   ps_.w2 = B_->w2;
   Buffers& B = *B_;
   fused_ = fused2d_supported(g_);
-  tma_ = fused_ && fused2d_tma_supported(g_);
   fused3_ = fused3d_supported(g_);
   if (G_ > 1 && !batchable(g_)) {
     *err = "this grid cannot be batched (needs D = 2 and every axis on the tensor cores)";
@@ -277,7 +273,7 @@ cudaError_t MixedBatch::zero_slot(int b, cudaStream_t s) {
   }
   if (e == cudaSuccess && B.f.z) e = cudaMemsetAsync(B.f.z + b * g_.K * n0, 0, (size_t)g_.K * n0 * 4, s);
   if (e == cudaSuccess && B.socp)
-    e = cudaMemsetAsync(B.socp + b * socp_blocks(g_, G_), 0, (size_t)socp_blocks(g_, G_) * sizeof(double), s);
+    e = cudaMemsetAsync(B.socp + b * fused2d_partials(g_, G_), 0, (size_t)fused2d_partials(g_, G_) * sizeof(double), s);
   return e;
 }
 
@@ -369,9 +365,7 @@ cudaError_t MixedBatch::upload_params(cudaStream_t s) {
 void MixedBatch::end_period() {
   // the fused kernels leave every slot's residual in f.r; the last period's first
   // iteration assembled the flagged slots, so the next one reuses them all unless a
-  // flag is set again (the D = 2 kernel without TMA, for odd N_y, leaves no residual:
-  // flags stay set)
-  if (!(tma_ || fused3_)) return;
+  // flag is set again
   for (SlotParam& p : hp_)
     if (p.assemble) {
       p.assemble = 0;
@@ -388,9 +382,9 @@ void MixedBatch::iterate(cudaStream_t s, LaunchCounter lc) {
     // sigma may change, or after a state or slot change)
     if (r_valid_) launch_solve_residual_mx(g_, G_, fc, ps_, s, lc);
     else launch_assemble_solve_mx(g_, G_, fc, ps_, s, lc);
-    // lines 3-6 (the TMA kernel also leaves the next residual in f.r)
-    r_valid_ = tma_ && launch_fused2d_tma(g_, G_, fc, fn, B_->socp, B_->err, true, s, lc);
-    if (!r_valid_) launch_fused2d(g_, G_, fc, fn, B_->socp, s, lc);
+    // lines 3-6, and the next iteration's residual in f.r
+    launch_fused2d(g_, G_, fc, fn, B_->socp, s, lc);
+    r_valid_ = true;
     cur_ ^= 1;
   } else if (fused3_) {
     const MxFields& fc = cur();
@@ -409,7 +403,7 @@ void MixedBatch::kkt(cudaStream_t s, LaunchCounter lc) {
   // every slot whose assemble flag is set (and reuses f.r for the others)
   r_valid_ = false;
   launch_kkt_mx(g_, G_, cur(), B_->partials, B_->red, fused_ ? B_->socp : nullptr,
-                fused_ ? (int)socp_blocks(g_, G_) : 0, s, lc);
+                fused_ ? (int)fused2d_partials(g_, G_) : 0, s, lc);
 }
 
 namespace {
@@ -512,7 +506,16 @@ int MixedBatch::read_state(int b, double* q, double* al, double* beta, cudaStrea
     std::vector<float2> t(nb);
     e = down(t.data(), fc.beta, nb * 8, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    for (size_t i = 0; i < nb; ++i) beta[i] = sig * ((double)t[i].x + (double)t[i].y);
+    if (g_.D == 2) {
+      const float* p = reinterpret_cast<const float*>(t.data());
+      for (int j = 0; j < g_.K; ++j)
+        for (size_t i = 0; i < n0; ++i) {
+          const long long o = beta2_at(j, (long long)i, (long long)n0);
+          beta[j * n0 + i] = sig * ((double)p[o] + (double)p[o + 2]);
+        }
+    } else {
+      for (size_t i = 0; i < nb; ++i) beta[i] = sig * ((double)t[i].x + (double)t[i].y);
+    }
   }
   if (e != cudaSuccess) { *err = std::string("read_state: ") + cudaGetErrorString(e); return DOT_ECUDA; }
   return DOT_OK;
@@ -543,7 +546,18 @@ int MixedBatch::write_state(int b, const double* q, const double* al, const doub
   }
   const size_t nb = (size_t)g_.K * n0;
   std::vector<float2> tb(nb);
-  for (size_t i = 0; i < nb; ++i) tb[i] = split_ff(beta[i] * is);
+  if (g_.D == 2) {
+    float* p = reinterpret_cast<float*>(tb.data());
+    for (int j = 0; j < g_.K; ++j)
+      for (size_t i = 0; i < n0; ++i) {
+        const float2 v = split_ff(beta[j * n0 + i] * is);
+        const long long o = beta2_at(j, (long long)i, (long long)n0);
+        p[o] = v.x;
+        p[o + 2] = v.y;
+      }
+  } else {
+    for (size_t i = 0; i < nb; ++i) tb[i] = split_ff(beta[i] * is);
+  }
   if (e == cudaSuccess) e = up(fc.beta, tb.data(), nb * 8, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) { *err = std::string("write_state: ") + cudaGetErrorString(e); return DOT_ECUDA; }
