@@ -3,6 +3,7 @@
 #include <cmath>
 #include <cstring>
 
+#include "dot_fft.cuh"
 #include "dot_paths.cuh"
 
 namespace dot {
@@ -39,10 +40,11 @@ namespace {
 
 struct F64Buffers {
   F64Fields f;
-  double* w2;
+  double* w2;              // right-hand side of poisson_op, scratch
   DctTables64 dct;
   double* Cbuf[kMaxD + 1];
   double* lbuf[kMaxD + 1];
+  double2* ftab[kMaxD];
   double* m0;
   double* m1;
   double* omega;
@@ -76,6 +78,7 @@ void carve_f64(const Geo& g, Carver& cv, F64Buffers* B) {
     B->Cbuf[a] = cv.take<double>(M * M);
     B->lbuf[a] = cv.take<double>(M);
   }
+  for (int d = 0; d < kMaxD; ++d) B->ftab[d] = d < g.D ? cv.take<double2>(fft_table_pairs(g.N[d])) : nullptr;
   B->partials = cv.take<double>((size_t)kkt_partials_len(g));
   B->red = cv.take<double>(R_NSLOTS);
 }
@@ -115,6 +118,18 @@ class PathF64 : public Path {
       B_.dct.C[a] = B_.Cbuf[a];
       B_.dct.lam[a] = B_.lbuf[a];
     }
+    fast_ = fast_poisson_supported(g_, sizeof(double));
+    std::memset(&fp_, 0, sizeof(fp_));
+    fp_.w1 = B_.f.w1;
+    fp_.w2 = B_.w2;
+    hf_.resize(g_.D);
+    for (int d = 0; d < g_.D && fast_; ++d) {
+      hf_[d] = fft_tables_host(g_.N[d]);
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(B_.ftab[d], hf_[d].data(), hf_[d].size() * sizeof(double), cudaMemcpyHostToDevice, s);
+      fp_.tab[d] = B_.ftab[d];
+      fp_.lam[d] = B_.lbuf[1 + d];
+    }
     if (e == cudaSuccess) e = zero_iterate(s);
     if (e != cudaSuccess) { *err = std::string("init: ") + cudaGetErrorString(e); return DOT_ECUDA; }
     return DOT_OK;
@@ -122,7 +137,7 @@ class PathF64 : public Path {
 
   void iterate(double sigma, double tau, cudaStream_t s, LaunchCounter lc) override {
     launch_assemble_b_f64(g_, B_.f, sigma, s, lc);                         // line 1
-    launch_poisson_f64(g_, B_.dct, B_.f.b, B_.f.w1, B_.f.phi, s, lc);     // line 2
+    poisson(B_.f.b, B_.f.phi, s, lc);                                     // line 2
     launch_project_f64(g_, B_.f, sigma, s, lc);                            // line 3
     launch_update_q_alpha_f64(g_, B_.f, sigma, tau, s, lc);                // lines 4-5
     launch_update_beta_f64(g_, B_.f, sigma, tau, s, lc);                   // line 6
@@ -177,7 +192,7 @@ class PathF64 : public Path {
     // every iteration, so the iterate (phi, q, alpha, beta, z) is left untouched).
     cudaError_t e = cudaMemcpyAsync(B_.w2, b, nn * sizeof(double), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) {
-      launch_poisson_f64(g_, B_.dct, B_.w2, B_.f.w1, B_.f.b, s, lc);
+      poisson(B_.w2, B_.f.b, s, lc);
       e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(phi, B_.f.b, nn * sizeof(double), cudaMemcpyDeviceToHost, s);
@@ -187,6 +202,12 @@ class PathF64 : public Path {
   }
 
  private:
+  // phi = (A^*A)^dagger b; b is overwritten (it and w1, w2 are scratch)
+  void poisson(double* b, double* phi, cudaStream_t s, LaunchCounter lc) {
+    if (fast_) launch_fast_poisson(g_, 1, fp_, b, phi, s, lc);
+    else launch_poisson_f64(g_, B_.dct, b, B_.f.w1, phi, s, lc);
+  }
+
   cudaError_t zero_iterate(cudaStream_t s) {
     const size_t nn = (size_t)(g_.T + 1) * g_.P, n0 = (size_t)g_.T * g_.P;
     cudaError_t e = cudaMemsetAsync(B_.f.phi, 0, nn * sizeof(double), s);
@@ -236,7 +257,9 @@ class PathF64 : public Path {
   Geo g_;
   F64Buffers B_;
   std::vector<double> hom_, hsom_;
-  std::vector<std::vector<double>> hC_, hl_;
+  std::vector<std::vector<double>> hC_, hl_, hf_;
+  FastPoisson<double> fp_;
+  bool fast_ = false;
 };
 
 }  // namespace
