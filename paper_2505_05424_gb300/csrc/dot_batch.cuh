@@ -92,7 +92,7 @@ class MixedBatch {
   SlotParam* dparams_ = nullptr;
   std::vector<SlotParam> hp_;
   std::vector<double> hs_;   // sigma per slot (host)
-  std::vector<std::vector<float>> hT_;
+  std::vector<std::vector<float>> hT_, hF_;
 
   const MxFields& cur() const;
   const MxFields& other() const;

@@ -1,5 +1,6 @@
 // dot_mixed.cuh -- fields and Poisson-solver tables of the mixed-precision path.
 #pragma once
+#include "dot_fft.cuh"
 #include "dot_internal.cuh"
 
 namespace dot {
@@ -104,6 +105,8 @@ struct MxPoisson {
   float* w2;
   int* err;                       // set by a tensor-core pass whose pipeline wait timed out
   bool use_tc;                    // run eligible passes on the tensor cores
+  FastPoisson<float> fast;        // the solve of each iteration, where the grid fits it
+  bool use_fast;
 };
 
 // Row stride of the padded time axis (a multiple of 4 floats: 16-byte TMA rows).

@@ -19,6 +19,15 @@
 // accurate to a few ulps for the smallest lambda.  The column lambda = 0 is singular:
 // its mean is removed from b and from x (the zero mode of the DCT), in FP64.
 //
+// FP32 (every iteration of the mixed path): each pass reads and writes the field once,
+// from L2 up to about 4 M nodes; a dense transform on the tensor cores in 3xTF32 needs
+// 256 multiply-adds per element in three passes and a table stream per CTA, and two
+// passes along time.  256^2 x 64, per iteration: 4 x 16.3 + 18.5 us (tensor cores
+// 4 x 25.4 + 2 x 23.6); 1024^2 x 32: 4 x 115 + 62 (4 x 396 + 2 x 162); 64^3 x 32:
+// 6 x 20.2 + 20.7 (6 x 30 + 2 x 54); 150 x 117 x 37, where the dense transform ran on
+// the FP32 units: 4 x 12.5 + 10 (4 x 22 + 19).  A cold solve's error is 2 to 5 times
+// smaller than the 3xTF32 one's.
+//
 // FP64: GB300 issues two FP64 lanes per SM and clock, so the count of operations is the
 // time: 17 per element and axis here against 256 multiply-adds of a dense 256-point
 // transform.  256^2 x 64, per iteration: four axis passes of 141 us and the time solve
@@ -269,9 +278,94 @@ __device__ __forceinline__ void put(float* dst, float2* accum, long long i, floa
 }
 __device__ __forceinline__ void put(double* dst, float2*, long long i, double v) { dst[i] = v; }
 
-// The DCT-II (INV false) or DCT-III of NP pairs of sequences.
+// Four neighbouring values (16-byte aligned rows), read-only for the kernel's lifetime.
+__device__ __forceinline__ void load4(const float* p, float* v) {
+  const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+  v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+}
+__device__ __forceinline__ void load4(const double* p, double* v) {
+  const double2 t = __ldg(reinterpret_cast<const double2*>(p)), u = __ldg(reinterpret_cast<const double2*>(p) + 1);
+  v[0] = t.x; v[1] = t.y; v[2] = u.x; v[3] = u.y;
+}
+__device__ __forceinline__ void store4(float* p, const float* v) {
+  *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void store4(double* p, const double* v) {
+  reinterpret_cast<double2*>(p)[0] = make_double2(v[0], v[1]);
+  reinterpret_cast<double2*>(p)[1] = make_double2(v[2], v[3]);
+}
+// accum[i .. i + 3] += v, the old values in old (loaded ahead)
+__device__ __forceinline__ void load_old(const float2* accum, long long i, float4* old) {
+  old[0] = reinterpret_cast<const float4*>(accum + i)[0];
+  old[1] = reinterpret_cast<const float4*>(accum + i)[1];
+}
+__device__ __forceinline__ void add4(float2* accum, long long i, const float4* old, const float* v) {
+  const float2 a = ff_add_f(make_float2(old[0].x, old[0].y), v[0]), b = ff_add_f(make_float2(old[0].z, old[0].w), v[1]);
+  const float2 c = ff_add_f(make_float2(old[1].x, old[1].y), v[2]), d = ff_add_f(make_float2(old[1].z, old[1].w), v[3]);
+  reinterpret_cast<float4*>(accum + i)[0] = make_float4(a.x, a.y, b.x, b.y);
+  reinterpret_cast<float4*>(accum + i)[1] = make_float4(c.x, c.y, d.x, d.y);
+}
+
+// Z[k] = V_a[k] + i V_b[k] of the inverse transform from X[k], X[N - k] of both sequences:
+// V_a = (c ak + s am) + i (s ak - c am)
+template <class V>
+__device__ __forceinline__ V zk(V w, V xk, V xm) {
+  return mk<V>((w.x * xk.x + w.y * xm.x) - (w.y * xk.y - w.x * xm.y),
+               (w.y * xk.x - w.x * xm.x) + (w.x * xk.y + w.y * xm.y));
+}
+// (X_a[k], X_b[k]) from Z[k], Z[N - k]: X_a = c (zr + mr) + s (zi - mi),
+// X_b = c (zi + mi) + s (mr - zr)
+template <class V>
+__device__ __forceinline__ V xk_of(V w, V z, V y) {
+  return mk<V>(w.x * (z.x + y.x) + w.y * (z.y - y.y), w.x * (z.y + y.y) - w.y * (z.x - y.x));
+}
+
+// Whether any slot of the pairs [p0, p0 + np) holds a solve.
+template <class R>
+__device__ __forceinline__ bool any_active(const FftArgs<R>& a, long long p0, int np) {
+  if (!a.sp) return true;
+  const long long last = min(p0 + np, a.npair) - 1;
+  bool on = false;
+  for (long long b = p0 / a.slot_pairs; b <= last / a.slot_pairs; ++b) on = on || a.sp[b].active;
+  return on;
+}
+
+// A pair of neighbouring columns of a strided axis, in 8-byte (FP64: 16) accesses where
+// the rows are even.
+template <class R>
+struct Columns {
+  using V = typename Vec2<R>::type;
+  const FftArgs<R>& a;
+  bool ok, two, vec;
+  long long base;
+  __device__ __forceinline__ Columns(const FftArgs<R>& args, long long pg) : a(args) {
+    ok = pg < a.npair;
+    const long long o = ok ? (long long)fdiv((unsigned)pg, a.fpi) : 0;
+    const int ci = ok ? 2 * (int)(pg - o * a.pin) : 0;
+    two = ok && ci + 1 < a.inner;
+    vec = a.inner % 2 == 0;
+    base = o * a.plan.N * a.inner + ci;
+  }
+  __device__ __forceinline__ V get(int j) const {
+    if (!ok) return mk<V>((R)0, (R)0);
+    const R* s = a.src + base + (long long)j * a.inner;
+    if (vec) return __ldg(reinterpret_cast<const V*>(s));
+    return mk<V>(__ldg(s), two ? __ldg(s + 1) : (R)0);
+  }
+  __device__ __forceinline__ void set(int j, V v) const {
+    const long long i = base + (long long)j * a.inner;
+    if (vec && !a.accum) {
+      *reinterpret_cast<V*>(a.dst + i) = v;
+    } else {
+      put(a.dst, a.accum, i, v.x);
+      if (two) put(a.dst, a.accum, i + 1, v.y);
+    }
+  }
+};
+
+// The DCT-II (INV false) or DCT-III of NP pairs of sequences of any length.
 template <class R, int NP, bool INV>
-__global__ void __launch_bounds__(kThreads) k_dct_fft(const __grid_constant__ FftArgs<R> a) {
+__global__ void __launch_bounds__(kThreads) k_dct_any(const __grid_constant__ FftArgs<R> a) {
   using V = typename Vec2<R>::type;
   constexpr int kPitch = NP + 1;
   extern __shared__ __align__(16) unsigned char fsm[];
@@ -280,121 +374,340 @@ __global__ void __launch_bounds__(kThreads) k_dct_fft(const __grid_constant__ Ff
   V* B = A + N * kPitch;
   V* tw = B + N * kPitch;
   const long long p0 = (long long)blockIdx.x * NP;
-  if (a.sp) {   // nothing to do where every slot of the CTA's pairs is empty
-    const long long last = min(p0 + NP, a.npair) - 1;
-    bool on = false;
-    for (long long b = p0 / a.slot_pairs; b <= last / a.slot_pairs; ++b) on = on || a.sp[b].active;
-    if (!on) return;
-  }
+  if (!any_active(a, p0, NP)) return;
   const V* rotf = a.tab + (INV ? 2 : 1) * N;
   for (int j = threadIdx.x; j < N; j += kThreads) tw[j] = a.tab[j];
-  const R zero = (R)0;
+  const V zero = mk<V>((R)0, (R)0);
   if (a.inner > 1) {
     // a thread keeps its pair of columns
-    const int pr = threadIdx.x % NP, j0 = threadIdx.x / NP;
-    const long long pg = p0 + pr;
-    const bool ok = pg < a.npair;
-    const long long o = ok ? (long long)fdiv((unsigned)pg, a.fpi) : 0;
-    const int ci = ok ? 2 * (int)(pg - o * a.pin) : 0;
-    const bool two = ok && ci + 1 < a.inner;
-    const long long base = o * N * a.inner + ci;
     constexpr int kStep = kThreads / NP;
+    const int pr = threadIdx.x % NP, j0 = threadIdx.x / NP;
+    const Columns<R> c(a, p0 + pr);
     if (!INV) {
-      for (int j = j0; j < N; j += kStep) {
-        const R* s = a.src + base + (long long)j * a.inner;
-        const int pos = (j & 1) ? N - 1 - (j >> 1) : j >> 1;
-        A[pos * kPitch + pr] = mk<V>(ok ? s[0] : zero, two ? s[1] : zero);
-      }
+#pragma unroll 4
+      for (int j = j0; j < N; j += kStep) A[((j & 1) ? N - 1 - (j >> 1) : j >> 1) * kPitch + pr] = c.get(j);
     } else {
+#pragma unroll 2
       for (int k = j0; k <= N / 2; k += kStep) {
-        const int m = k ? N - k : 0;
-        const R* sk = a.src + base + (long long)k * a.inner;
-        const R* sm = a.src + base + (long long)m * a.inner;
-        const R ak = ok ? sk[0] : zero, bk = two ? sk[1] : zero;
-        const R am = ok && k ? sm[0] : zero, bm = two && k ? sm[1] : zero;
-        const V w = rotf[k];
-        // V_a = (c ak + s am) + i (s ak - c am), Z = V_a + i V_b
-        A[k * kPitch + pr] = mk<V>((w.x * ak + w.y * am) - (w.y * bk - w.x * bm),
-                                   (w.y * ak - w.x * am) + (w.x * bk + w.y * bm));
-        if (k && m != k) {
-          const V u = rotf[m];
-          A[m * kPitch + pr] = mk<V>((u.x * am + u.y * ak) - (u.y * bm - u.x * bk),
-                                     (u.y * am - u.x * ak) + (u.x * bm + u.y * bk));
-        }
+        const int m = N - k;
+        const V xk = c.get(k), xm = k ? c.get(m) : zero;
+        A[k * kPitch + pr] = zk(rotf[k], xk, xm);
+        if (k && m != k) A[m * kPitch + pr] = zk(rotf[m], xm, xk);
       }
     }
     __syncthreads();
     const V* Z = transform<NP, INV>(A, B, tw, a.plan);
-    if (!ok) return;
+    if (!c.ok) return;
     if (!INV) {
+#pragma unroll 2
       for (int k = j0; k <= N / 2; k += kStep) {
         const int m = k ? N - k : 0;
         const V z = Z[k * kPitch + pr], y = Z[m * kPitch + pr];
-        const V w = rotf[k];
-        const V sp = cadd(z, y), sd = csub(z, y);
-        // X_a = c (zr + mr) + s (zi - mi), X_b = c (zi + mi) + s (mr - zr)
-        const long long ik = base + (long long)k * a.inner;
-        put(a.dst, a.accum, ik, w.x * sp.x + w.y * sd.y);
-        if (two) put(a.dst, a.accum, ik + 1, w.x * sp.y - w.y * sd.x);
-        if (k && m != k) {
-          const V u = rotf[m];
-          const long long im = base + (long long)m * a.inner;
-          put(a.dst, a.accum, im, u.x * sp.x - u.y * sd.y);
-          if (two) put(a.dst, a.accum, im + 1, u.x * sp.y + u.y * sd.x);
-        }
+        c.set(k, xk_of(rotf[k], z, y));
+        if (k && m != k) c.set(m, xk_of(rotf[m], y, z));
       }
     } else {
-      for (int j = j0; j < N; j += kStep) {
-        const int pos = (j & 1) ? N - 1 - (j >> 1) : j >> 1;
-        const V z = Z[pos * kPitch + pr];
-        const long long ij = base + (long long)j * a.inner;
-        put(a.dst, a.accum, ij, z.x);
-        if (two) put(a.dst, a.accum, ij + 1, z.y);
-      }
+#pragma unroll 4
+      for (int j = j0; j < N; j += kStep) c.set(j, Z[((j & 1) ? N - 1 - (j >> 1) : j >> 1) * kPitch + pr]);
     }
   } else {
     // pairs of contiguous rows: neighbouring threads take neighbouring elements
-    const int np = (int)min((long long)NP, a.npair - p0);
-    if (!INV) {
-      for (int e = threadIdx.x; e < NP * N; e += kThreads) {
-        const int pr = (int)fdiv((unsigned)e, a.plan.fN), j = e - pr * N;
-        const long long row = 2 * (p0 + pr);
-        const R* s = a.src + row * N + j;
-        const int pos = (j & 1) ? N - 1 - (j >> 1) : j >> 1;
-        A[pos * kPitch + pr] = mk<V>(row < a.nseq ? s[0] : zero, row + 1 < a.nseq ? s[N] : zero);
-      }
-    } else {
-      for (int e = threadIdx.x; e < NP * N; e += kThreads) {
-        const int pr = (int)fdiv((unsigned)e, a.plan.fN), k = e - pr * N;
-        const long long row = 2 * (p0 + pr);
-        const bool ok = row < a.nseq, two = row + 1 < a.nseq;
-        const R* s = a.src + row * N;
-        const int m = N - k;
-        const R ak = ok ? s[k] : zero, bk = two ? s[N + k] : zero;
-        const R am = ok && k ? s[m] : zero, bm = two && k ? s[N + m] : zero;
-        const V w = rotf[k];
-        A[k * kPitch + pr] = mk<V>((w.x * ak + w.y * am) - (w.y * bk - w.x * bm),
-                                   (w.y * ak - w.x * am) + (w.x * bk + w.y * bm));
-      }
+#pragma unroll 4
+    for (int e = threadIdx.x; e < NP * N; e += kThreads) {
+      const int pr = (int)fdiv((unsigned)e, a.plan.fN), j = e - pr * N;
+      const long long row = 2 * (p0 + pr);
+      const R* s = a.src + row * N + j;
+      const V v = mk<V>(row < a.nseq ? __ldg(s) : (R)0, row + 1 < a.nseq ? __ldg(s + N) : (R)0);
+      if (INV) B[j * kPitch + pr] = v;
+      else A[((j & 1) ? N - 1 - (j >> 1) : j >> 1) * kPitch + pr] = v;
     }
     __syncthreads();
+    if (INV) {
+      for (int e = threadIdx.x; e < NP * (N / 2 + 1); e += kThreads) {
+        const int pr = e % NP, k = e / NP, m = N - k;
+        const V xk = B[k * kPitch + pr], xm = k ? B[m * kPitch + pr] : zero;
+        A[k * kPitch + pr] = zk(rotf[k], xk, xm);
+        if (k && m != k) A[m * kPitch + pr] = zk(rotf[m], xm, xk);
+      }
+      __syncthreads();
+    }
     const V* Z = transform<NP, INV>(A, B, tw, a.plan);
+    const int np = (int)min((long long)NP, a.npair - p0);
+#pragma unroll 4
     for (int e = threadIdx.x; e < np * N; e += kThreads) {
       const int pr = (int)fdiv((unsigned)e, a.plan.fN), k = e - pr * N;
       const long long row = 2 * (p0 + pr);
-      R xa, xb;
-      if (!INV) {
-        const V z = Z[k * kPitch + pr], y = Z[(k ? N - k : 0) * kPitch + pr];
-        const V w = rotf[k];
-        xa = w.x * (z.x + y.x) + w.y * (z.y - y.y);
-        xb = w.x * (z.y + y.y) - w.y * (z.x - y.x);
-      } else {
-        const V z = Z[((k & 1) ? N - 1 - (k >> 1) : k >> 1) * kPitch + pr];
-        xa = z.x;
-        xb = z.y;
+      const V x = INV ? Z[((k & 1) ? N - 1 - (k >> 1) : k >> 1) * kPitch + pr]
+                      : xk_of(rotf[k], Z[k * kPitch + pr], Z[(k ? N - k : 0) * kPitch + pr]);
+      put(a.dst, a.accum, row * N + k, x.x);
+      if (row + 1 < a.nseq) put(a.dst, a.accum, (row + 1) * N + k, x.y);
+    }
+  }
+}
+
+// ---- power-of-two axes ------------------------------------------------------------
+//
+// The same transform with the length known at compile time: a thread holds sixteen
+// complex elements in registers and runs a radix-16 butterfly (then radix 2 .. 16 ones on
+// the rest), in place in shared memory; the columns of a strided axis enter the first
+// butterfly (forward) and leave the last one (inverse) without passing through it.
+
+// w_16^m, m = 1, 2, 3, 4, 6, 9 (conjugated for the inverse)
+template <bool INV, int M, class V>
+__device__ __forceinline__ V mul16(V a) {
+  using S = std::remove_reference_t<decltype(a.x)>;
+  const S c = (S)0.92387953251128675613, s = (S)0.38268343236508977173, h = (S)0.70710678118654752440;
+  if constexpr (M == 1) return cmulw<INV>(a, mk<V>(c, -s));
+  else if constexpr (M == 2) { const V r = rot<INV>(a); return mk<V>(h * (a.x + r.x), h * (a.y + r.y)); }
+  else if constexpr (M == 3) return cmulw<INV>(a, mk<V>(s, -c));
+  else if constexpr (M == 4) return rot<INV>(a);
+  else if constexpr (M == 6) { const V r = rot<INV>(a); return mk<V>(h * (r.x - a.x), h * (r.y - a.y)); }
+  else return cmulw<INV>(a, mk<V>(-c, s));
+}
+// Output k + 4 l of the 16-point DFT ends in x[4 k + l].
+template <bool INV, class V>
+__device__ __forceinline__ void dft16(V* x) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j) dft4<INV>(x[j], x[j + 4], x[j + 8], x[j + 12]);
+  x[5] = mul16<INV, 1>(x[5]);
+  x[6] = mul16<INV, 2>(x[6]);
+  x[7] = mul16<INV, 3>(x[7]);
+  x[9] = mul16<INV, 2>(x[9]);
+  x[10] = mul16<INV, 4>(x[10]);
+  x[11] = mul16<INV, 6>(x[11]);
+  x[13] = mul16<INV, 3>(x[13]);
+  x[14] = mul16<INV, 6>(x[14]);
+  x[15] = mul16<INV, 9>(x[15]);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) dft4<INV>(x[4 * k], x[4 * k + 1], x[4 * k + 2], x[4 * k + 3]);
+}
+// register of output k of a RAD-point DFT
+template <int RAD>
+__device__ __forceinline__ constexpr int reg_of(int k) { return RAD == 16 ? 4 * (k % 4) + k / 4 : k; }
+
+template <int N, int NP>
+struct Pow2 {
+  static constexpr int kThreads = N / 16 * NP;   // a radix-16 butterfly each
+  // radix of the stage that starts at stride S
+  static constexpr int radix(int S) {
+    const int rest = N / S;
+    return S == 1 ? 16 : rest <= 16 ? rest : 8;
+  }
+};
+
+// The stage at stride S on the thread's registers x: 16 / RAD butterflies, bb = b + i kNb.
+template <int N, int NP, int S, bool INV, class V>
+__device__ __forceinline__ void p2_compute(V* x, int b, const V* tw) {
+  constexpr int RAD = Pow2<N, NP>::radix(S), kNb = N / 16;
+#pragma unroll
+  for (int i = 0; i < 16 / RAD; ++i) {
+    V* y = x + i * RAD;
+    if constexpr (RAD == 16) dft16<INV>(y);
+    else dft<RAD, INV>(y);
+    if constexpr (S * RAD < N) {
+      const int p = (b + i * kNb) / S;
+#pragma unroll
+      for (int k = 1; k < RAD; ++k) y[reg_of<RAD>(k)] = cmulw<INV>(y[reg_of<RAD>(k)], tw[S * p * k]);
+    }
+  }
+}
+template <int N, int NP, int S, class V>
+__device__ __forceinline__ void p2_read(V* x, const V* A, int b, int pr) {
+  constexpr int RAD = Pow2<N, NP>::radix(S), kNb = N / 16, kPitch = NP + 1;
+#pragma unroll
+  for (int i = 0; i < 16 / RAD; ++i)
+#pragma unroll
+    for (int j = 0; j < RAD; ++j) x[i * RAD + j] = A[(b + i * kNb + (N / RAD) * j) * kPitch + pr];
+}
+// position of output k of butterfly bb
+template <int S, int RAD>
+__device__ __forceinline__ int p2_pos(int bb, int k) { return bb % S + S * (RAD * (bb / S) + k); }
+template <int N, int NP, int S, class V>
+__device__ __forceinline__ void p2_write(const V* x, V* A, int b, int pr) {
+  constexpr int RAD = Pow2<N, NP>::radix(S), kNb = N / 16, kPitch = NP + 1;
+#pragma unroll
+  for (int i = 0; i < 16 / RAD; ++i)
+#pragma unroll
+    for (int k = 0; k < RAD; ++k) A[p2_pos<S, RAD>(b + i * kNb, k) * kPitch + pr] = x[i * RAD + reg_of<RAD>(k)];
+}
+// Stages from stride S to the end; the last one leaves its results in x when KEEP.
+template <int N, int NP, int S, bool INV, bool KEEP, class V>
+__device__ __forceinline__ void p2_stages(V* x, V* A, const V* tw, int b, int pr) {
+  constexpr int RAD = Pow2<N, NP>::radix(S);
+  p2_read<N, NP, S>(x, A, b, pr);
+  p2_compute<N, NP, S, INV>(x, b, tw);
+  if constexpr (S * RAD < N) {
+    __syncthreads();
+    p2_write<N, NP, S>(x, A, b, pr);
+    __syncthreads();
+    p2_stages<N, NP, S * RAD, INV, KEEP>(x, A, tw, b, pr);
+  } else if constexpr (!KEEP) {
+    __syncthreads();
+    p2_write<N, NP, S>(x, A, b, pr);
+    __syncthreads();
+  }
+}
+template <int N, int NP>
+__host__ __device__ constexpr int p2_last() {   // stride of the last stage
+  int S = 1;
+  while (S * Pow2<N, NP>::radix(S) < N) S *= Pow2<N, NP>::radix(S);
+  return S;
+}
+
+template <class R, int N, int NP, bool INV, bool ROWS>
+__global__ void __launch_bounds__(Pow2<N, NP>::kThreads) k_dct_pow2(const __grid_constant__ FftArgs<R> a) {
+  using V = typename Vec2<R>::type;
+  constexpr int kPitch = NP + 1, kNb = N / 16, kT = Pow2<N, NP>::kThreads;
+  extern __shared__ __align__(16) unsigned char fsm[];
+  V* A = reinterpret_cast<V*>(fsm);
+  V* tw = A + N * kPitch;
+  const long long p0 = (long long)blockIdx.x * NP;
+  if (!any_active(a, p0, NP)) return;
+  const V* rotf = a.tab + (INV ? 2 : 1) * N;
+  const int tid = threadIdx.x, pr = tid % NP, b = tid / NP;
+  for (int j = tid; j < N; j += kT) tw[j] = __ldg(a.tab + j);
+  V x[16];
+  const V zero = mk<V>((R)0, (R)0);
+  if constexpr (!ROWS) {
+    const Columns<R> c(a, p0 + pr);
+    if constexpr (!INV) {
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        const int n = b + kNb * j;
+        x[j] = c.get(j < 8 ? 2 * n : 2 * (N - n) - 1);
       }
-      put(a.dst, a.accum, row * N + k, xa);
-      if (row + 1 < a.nseq) put(a.dst, a.accum, (row + 1) * N + k, xb);
+      __syncthreads();   // tw
+      p2_compute<N, NP, 1, INV>(x, b, tw);
+      p2_write<N, NP, 1>(x, A, b, pr);
+      __syncthreads();
+      if constexpr (N > 16) p2_stages<N, NP, 16, INV, false>(x, A, tw, b, pr);
+      if (!c.ok) return;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int k = b + kNb * i, m = k ? N - k : N / 2;
+        const V z = A[k * kPitch + pr], y = A[m * kPitch + pr];
+        c.set(k, xk_of(__ldg(rotf + k), z, k ? y : z));
+        c.set(m, xk_of(__ldg(rotf + m), y, k ? z : y));
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int k = b + kNb * i, m = k ? N - k : N / 2;
+        x[2 * i] = c.get(k);
+        x[2 * i + 1] = c.get(m);
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int k = b + kNb * i, m = k ? N - k : N / 2;
+        A[k * kPitch + pr] = zk(__ldg(rotf + k), x[2 * i], k ? x[2 * i + 1] : zero);
+        A[m * kPitch + pr] = zk(__ldg(rotf + m), x[2 * i + 1], k ? x[2 * i] : x[2 * i + 1]);
+      }
+      __syncthreads();
+      p2_stages<N, NP, 1, INV, true>(x, A, tw, b, pr);
+      if (!c.ok) return;
+      constexpr int S = p2_last<N, NP>(), RAD = N / S;
+#pragma unroll
+      for (int i = 0; i < 16 / RAD; ++i)
+#pragma unroll
+        for (int k = 0; k < RAD; ++k) {
+          const int n = p2_pos<S, RAD>(b + i * kNb, k);
+          c.set(n < N / 2 ? 2 * n : 2 * (N - n) - 1, x[i * RAD + reg_of<RAD>(k)]);
+        }
+    }
+  } else {
+    // pairs of contiguous rows, four neighbouring elements of both per thread and step
+    constexpr int kQ = N / 4, kIt = 4;                 // kT kIt chunks in all
+    static_assert(kT * kIt == NP * kQ, "four chunks per thread");
+    R va[kIt][4], vb[kIt][4];
+#pragma unroll
+    for (int u = 0; u < kIt; ++u) {
+      const int e = tid + u * kT, j = 4 * (e % kQ);
+      const long long row = 2 * (p0 + e / kQ);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) va[u][q] = vb[u][q] = (R)0;
+      if (row < a.nseq) load4(a.src + row * N + j, va[u]);
+      if (row + 1 < a.nseq) load4(a.src + (row + 1) * N + j, vb[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < kIt; ++u) {
+      const int e = tid + u * kT, j = 4 * (e % kQ), r = e / kQ;
+      if (!INV) {   // the reordered sequence
+        V* lo = A + (j / 2) * kPitch + r;
+        V* hi = A + (N - 1 - j / 2) * kPitch + r;
+        lo[0] = mk<V>(va[u][0], vb[u][0]);
+        hi[0] = mk<V>(va[u][1], vb[u][1]);
+        lo[kPitch] = mk<V>(va[u][2], vb[u][2]);
+        hi[-kPitch] = mk<V>(va[u][3], vb[u][3]);
+      } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) A[(j + q) * kPitch + r] = mk<V>(va[u][q], vb[u][q]);
+      }
+    }
+    __syncthreads();
+    if constexpr (INV) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {   // in place: a thread owns its pairs k, N - k
+        const int k = b + kNb * i, m = k ? N - k : N / 2;
+        const V xk = A[k * kPitch + pr], xm = A[m * kPitch + pr];
+        A[k * kPitch + pr] = zk(__ldg(rotf + k), xk, k ? xm : zero);
+        A[m * kPitch + pr] = zk(__ldg(rotf + m), xm, k ? xk : xm);
+      }
+      __syncthreads();
+    }
+    p2_stages<N, NP, 1, INV, false>(x, A, tw, b, pr);
+    if constexpr (INV && sizeof(R) == 4) {
+      if (a.accum) {
+#pragma unroll
+        for (int u = 0; u < kIt; u += 2) {
+          float4 oa[2][2], ob[2][2];
+#pragma unroll
+          for (int v = 0; v < 2; ++v) {
+            const int e = tid + (u + v) * kT, j = 4 * (e % kQ);
+            const long long row = 2 * (p0 + e / kQ);
+            if (row < a.nseq) load_old(a.accum, row * N + j, oa[v]);
+            if (row + 1 < a.nseq) load_old(a.accum, (row + 1) * N + j, ob[v]);
+          }
+#pragma unroll
+          for (int v = 0; v < 2; ++v) {
+            const int e = tid + (u + v) * kT, j = 4 * (e % kQ), r = e / kQ;
+            const long long row = 2 * (p0 + r);
+            const V* lo = A + (j / 2) * kPitch + r;
+            const V* hi = A + (N - 1 - j / 2) * kPitch + r;
+            const V z[4] = {lo[0], hi[0], lo[kPitch], hi[-kPitch]};
+            const float xa[4] = {z[0].x, z[1].x, z[2].x, z[3].x};
+            const float xb[4] = {z[0].y, z[1].y, z[2].y, z[3].y};
+            if (row < a.nseq) add4(a.accum, row * N + j, oa[v], xa);
+            if (row + 1 < a.nseq) add4(a.accum, (row + 1) * N + j, ob[v], xb);
+          }
+        }
+        return;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kIt; ++u) {
+      const int e = tid + u * kT, j = 4 * (e % kQ), r = e / kQ;
+      const long long row = 2 * (p0 + r);
+      R xa[4], xb[4];
+      if constexpr (!INV) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int k = j + q;
+          const V v = xk_of(__ldg(rotf + k), A[k * kPitch + r], A[(k ? N - k : 0) * kPitch + r]);
+          xa[q] = v.x;
+          xb[q] = v.y;
+        }
+      } else {
+        const V* lo = A + (j / 2) * kPitch + r;
+        const V* hi = A + (N - 1 - j / 2) * kPitch + r;
+        const V v[4] = {lo[0], hi[0], lo[kPitch], hi[-kPitch]};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          xa[q] = v[q].x;
+          xb[q] = v[q].y;
+        }
+      }
+      if (row < a.nseq) store4(a.dst + row * N + j, xa);
+      if (row + 1 < a.nseq) store4(a.dst + (row + 1) * N + j, xb);
     }
   }
 }
@@ -413,6 +726,7 @@ struct TimeArgs {
   const R* lam[kMaxD];
   R a;                 // 1 / h_0^2
   long long ncol;      // columns over all slots
+  int slots;
   const SlotParam* sp;
 };
 
@@ -435,7 +749,7 @@ __device__ __forceinline__ double warp_before(double v) {
 // x_t = x_0 - sum_{i < t} S_i / a with S_i = sum_{j <= i} (b_j - mean(b)).  A lane holds a
 // run of time nodes.
 template <class R>
-__device__ void zero_column(const R* b, R* x, int M, long long P, double a) {
+__device__ void zero_column(const R* b, R* x, int M, long long P, double ia) {
   const int lane = threadIdx.x & 31, C = (M + 31) / 32;
   const int t0 = min(M, lane * C), t1 = min(M, t0 + C);
   double v = 0.0;
@@ -451,7 +765,7 @@ __device__ void zero_column(const R* b, R* x, int M, long long P, double a) {
   double u = U0, xs = 0.0;
   S = S0;
   for (int t = t0; t < t1; ++t) {
-    xs -= u / a;
+    xs -= u * ia;
     S += (double)b[t * P] - mean;
     u += S;
   }
@@ -460,55 +774,67 @@ __device__ void zero_column(const R* b, R* x, int M, long long P, double a) {
   S = S0;
   for (int t = t0; t < t1; ++t) {
     const double bt = (double)b[t * P];
-    x[t * P] = (R)(-u / a - shift);
+    x[t * P] = (R)(-u * ia - shift);
     S += bt - mean;
     u += S;
   }
 }
 
-// (lambda I + L_t) x = b along time, one thread per column of spatial frequencies; the
-// eliminated right-hand sides and the pivots' reciprocals wait in shared memory.
+__device__ __forceinline__ void copy_async(uint32_t dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_async(uint32_t dst, const double* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+}
+
+// (lambda I + L_t) x = b along time, one thread per column of spatial frequencies.  The
+// whole column is copied to shared memory at once while the pivots, which do not need
+// it, are formed; the eliminated right-hand sides and the pivots' reciprocals stay
+// there.  The first `slots` blocks take the singular columns, a warp each.
 template <class R, int THREADS>
 __global__ void __launch_bounds__(THREADS) k_time_solve(const __grid_constant__ Geo g,
                                                         const __grid_constant__ TimeArgs<R> ta) {
   extern __shared__ __align__(16) unsigned char fsm[];
-  const long long col = (long long)blockIdx.x * THREADS + threadIdx.x;
   const long long P = g.P;
-  // the singular columns (p = 0 of a slot), by the first warp of the block they fall in
-  {
-    const long long c0 = (long long)blockIdx.x * THREADS;
-    const long long z0 = (c0 + P - 1) / P;   // first slot whose column 0 is not before c0
-    if (threadIdx.x < 32)
-      for (long long z = z0; z * P < min(c0 + THREADS, ta.ncol); ++z)
-        if (!ta.sp || ta.sp[z].active)
-          zero_column(ta.src + z * (g.T + 1) * P, ta.dst + z * (g.T + 1) * P, g.T + 1, P, (double)ta.a);
+  const int M = g.T + 1;
+  if ((int)blockIdx.x < ta.slots) {
+    const int z = blockIdx.x;
+    if (threadIdx.x < 32 && (!ta.sp || ta.sp[z].active))
+      zero_column(ta.src + z * M * P, ta.dst + z * M * P, M, P, 1.0 / (double)ta.a);
+    return;
   }
+  const long long col = (long long)(blockIdx.x - ta.slots) * THREADS + threadIdx.x;
   if (col >= ta.ncol) return;
   const int slot = (int)fdiv((unsigned)col, g.fP), p = (int)(col - slot * P);
-  if (p == 0) return;
-  if (ta.sp && !ta.sp[slot].active) return;
-  const int M = g.T + 1;
+  if (p == 0 || (ta.sp && !ta.sp[slot].active)) return;
   const R* b = ta.src + slot * M * P + p;
   R* x = ta.dst + slot * M * P + p;
   R* y = reinterpret_cast<R*>(fsm) + threadIdx.x;        // y[t THREADS]
   R* rr = y + (size_t)M * THREADS;                       // 1 / d_t
+  const uint32_t ys = (uint32_t)__cvta_generic_to_shared(y);
+#pragma unroll 8
+  for (int t = 0; t < M; ++t) copy_async(ys + t * THREADS * sizeof(R), b + t * P);
+  asm volatile("cp.async.commit_group;" ::: "memory");
   R lam = (R)0;
   for (int d = 0; d < g.D; ++d) lam += ta.lam[d][coord(g, p, d)];
   const R a = ta.a;
-  R s = lam, yp = b[0];
-  R r = recip(a + s);
-  y[0] = yp;
+  R s = lam, r = recip(a + s);
   rr[0] = r;
-#pragma unroll 8
-  for (int t = 1; t < M; ++t) {
-    const R ar = a * r;
-    s = lam + ar * s;
-    yp = b[t * P] + ar * yp;
-    r = recip(t < M - 1 ? a + s : s);
-    y[t * THREADS] = yp;
+  for (int t = 1; t < M - 1; ++t) {
+    s = lam + a * r * s;
+    r = recip(a + s);
     rr[t * THREADS] = r;
   }
-  R xp = yp * r;
+  s = lam + a * r * s;
+  rr[(M - 1) * THREADS] = recip(s);
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  R yp = y[0];
+#pragma unroll 8
+  for (int t = 1; t < M; ++t) {
+    yp = y[t * THREADS] + a * rr[(t - 1) * THREADS] * yp;
+    y[t * THREADS] = yp;
+  }
+  R xp = yp * rr[(M - 1) * THREADS];
   x[(M - 1) * P] = xp;
 #pragma unroll 8
   for (int t = M - 2; t >= 0; --t) {
@@ -526,8 +852,48 @@ size_t fft_smem(int N, int NP) { return (size_t)(2 * N * (NP + 1) + N) * 2 * siz
 template <class R, int NP, bool INV>
 void launch_np(const FftArgs<R>& a, cudaStream_t s) {
   static std::atomic<unsigned long long> done{0};
-  smem_optin((const void*)k_dct_fft<R, NP, INV>, kMaxSmem, &done);
-  k_dct_fft<R, NP, INV><<<(unsigned)((a.npair + NP - 1) / NP), kThreads, fft_smem<R>(a.plan.N, NP), s>>>(a);
+  smem_optin((const void*)k_dct_any<R, NP, INV>, kMaxSmem, &done);
+  k_dct_any<R, NP, INV><<<(unsigned)((a.npair + NP - 1) / NP), kThreads, fft_smem<R>(a.plan.N, NP), s>>>(a);
+}
+
+template <class R, int N, int NP, bool INV, bool ROWS>
+void launch_pow2(const FftArgs<R>& a, cudaStream_t s) {
+  const size_t sm = (size_t)(N * (NP + 1) + N) * 2 * sizeof(R);
+  static std::atomic<unsigned long long> done{0};
+  smem_optin((const void*)k_dct_pow2<R, N, NP, INV, ROWS>, (int)sm, &done);
+  k_dct_pow2<R, N, NP, INV, ROWS><<<(unsigned)((a.npair + NP - 1) / NP), Pow2<N, NP>::kThreads, sm, s>>>(a);
+}
+template <class R, int N, int NP, int NPS, bool INV>
+bool try_pow2_np(const FftArgs<R>& a, cudaStream_t s) {
+  const bool rows = a.inner == 1;
+  if (a.npair >= (long long)NP * 152) {
+    if (rows) launch_pow2<R, N, NP, INV, true>(a, s);
+    else launch_pow2<R, N, NP, INV, false>(a, s);
+    return true;
+  }
+  if constexpr (sizeof(R) == 4) {
+    if (rows) launch_pow2<R, N, NPS, INV, true>(a, s);
+    else launch_pow2<R, N, NPS, INV, false>(a, s);
+    return true;
+  }
+  return false;
+}
+// Axes of 32 to 1024 points take the compile-time form: with many sequences 4,096
+// elements per CTA, with few ones 1,024 to 2,048 for more CTAs (FP64: the general form).
+// In FP32 the form may not depend on the number of solves in a batch, whose results are
+// the same bit for bit whatever they are served with; the pairs per CTA change no value.
+template <class R, bool INV>
+bool try_pow2(const FftArgs<R>& a, cudaStream_t s) {
+  constexpr bool f = sizeof(R) == 4;
+  switch (a.plan.N) {
+    case 32: return f && try_pow2_np<float, 32, 64, 32, INV>(reinterpret_cast<const FftArgs<float>&>(a), s);
+    case 64: return try_pow2_np<R, 64, 32, 16, INV>(a, s);
+    case 128: return try_pow2_np<R, 128, 16, 8, INV>(a, s);
+    case 256: return try_pow2_np<R, 256, f ? 16 : 8, 8, INV>(a, s);
+    case 512: return try_pow2_np<R, 512, 8, 4, INV>(a, s);
+    case 1024: return try_pow2_np<R, 1024, f ? 8 : 4, 2, INV>(a, s);
+    default: return false;
+  }
 }
 
 // One axis of G solves.  Pairs per CTA: 16 (8 in FP64: 128-byte segments of a strided
@@ -551,6 +917,10 @@ void fft_axis(const Geo& g, int G, int axis, const FastPoisson<R>& fp, const R* 
   a.plan = make_plan(N);
   a.sp = G > 1 ? fp.sp : nullptr;
   a.slot_pairs = G > 1 ? a.npair / G : a.npair;
+  if (try_pow2<R, INV>(a, s)) {
+    lc.launched(KID_DCT_AXIS);
+    return;
+  }
   int np = sizeof(R) == 4 ? 16 : 8;
   while (np > 2 && (fft_smem<R>(N, np) > (size_t)kMaxSmem / 2 || (a.npair + np - 1) / np < 2 * 152)) np /= 2;
   while (np > 1 && fft_smem<R>(N, np) > (size_t)kMaxSmem) np /= 2;
@@ -583,10 +953,11 @@ void fast_poisson(const Geo& g, int G, const FastPoisson<R>& fp, const R* src, R
   for (int d = 0; d < g.D; ++d) ta.lam[d] = fp.lam[d];
   ta.a = (R)(g.invh[0] * g.invh[0]);
   ta.ncol = (long long)G * g.P;
+  ta.slots = G;
   ta.sp = G > 1 ? fp.sp : nullptr;
   static std::atomic<unsigned long long> done{0};
   smem_optin((const void*)k_time_solve<R, kT>, kMaxSmem, &done);
-  k_time_solve<R, kT><<<(unsigned)((ta.ncol + kT - 1) / kT), kT, (size_t)2 * (g.T + 1) * kT * sizeof(R), s>>>(g, ta);
+  k_time_solve<R, kT><<<(unsigned)(G + (ta.ncol + kT - 1) / kT), kT, (size_t)2 * (g.T + 1) * kT * sizeof(R), s>>>(g, ta);
   lc.launched(KID_SCALE);
   cur = w[nx];
   nx ^= 1;

@@ -564,6 +564,10 @@ void poisson_refined_tmpl(const Geo& g, int G, const MxFields& f, const MxPoisso
 void poisson_add_tmpl(const Geo& g, int G, const MxFields& f, const MxPoisson& ps, cudaStream_t s,
                       LaunchCounter lc) {
   const long long nn = (long long)(g.T + 1) * g.P;
+  if (ps.use_fast) {
+    launch_fast_poisson(g, G, ps.fast, f.r, f.phi1, f.phi, s, lc);
+    return;
+  }
   if (launch_poisson_mx(g, G, ps, f.r, f.phi1, s, lc, f.phi)) return;
   k_phi_add<<<dim3(grid_for(nn), G), kThreads, 0, s>>>(g, f);
   lc.launched(KID_COMBINE);

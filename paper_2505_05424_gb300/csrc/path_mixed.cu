@@ -26,6 +26,7 @@ struct MixedBatch::Buffers {
   float* tab[kMaxD + 1][6];   // C, C^T, C hi, C lo, C^T hi, C^T lo
   float* tpad[4];             // time axis, rows padded to time_ld(g)
   float* lbuf[kMaxD + 1];
+  float2* ftab[kMaxD];        // tables of the fast Poisson solve
   double* partials;
   double* red;
   int* err;
@@ -83,6 +84,7 @@ void carve(const Geo& g, int G, bool masks, Carver& cv, MixedBatch::Buffers* B) 
     for (int j = 0; j < 6; ++j) B->tab[a][j] = cv.take<float>(M * M);
     B->lbuf[a] = cv.take<float>(M);
   }
+  for (int d = 0; d < g.D; ++d) B->ftab[d] = cv.take<float2>(fft_table_pairs(g.N[d]));
   const size_t ldt = (size_t)time_ld(g);
   for (int j = 0; j < 4; ++j) B->tpad[j] = cv.take<float>((size_t)(g.T + 1) * ldt);
   B->partials = cv.take<double>(Gs * kkt_partials_len_mx(g));
@@ -233,6 +235,18 @@ int MixedBatch::init(char* ws, size_t bytes, cudaStream_t s, std::string* err) {
         ps_.tpad[j] = B.tpad[j];
       }
     }
+  }
+  ps_.use_fast = fast_poisson_supported(g_, sizeof(float));
+  ps_.fast.w1 = ps_.w1;
+  ps_.fast.w2 = ps_.w2;
+  ps_.fast.sp = B.params;
+  hF_.assign(g_.D, {});
+  for (int d = 0; d < g_.D; ++d) {
+    const std::vector<double> t = fft_tables_host(g_.N[d]);
+    hF_[d].assign(t.begin(), t.end());
+    if (e == cudaSuccess) e = up(B.ftab[d], hF_[d].data(), hF_[d].size() * 4, s);
+    ps_.fast.tab[d] = B.ftab[d];
+    ps_.fast.lam[d] = B.lbuf[1 + d];
   }
   ps_.err = B.err;
   ps_.use_tc = true;

@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 
 GRIDS = [(1, [3, 2]), (16, [32, 32]), (5, [33, 65]),       # 4 rows
          (20, [100, 60]), (33, [57, 70]),                  # 8 rows
-         (31, [130, 97]), (40, [200, 131])]  # 13 rows
+         (31, [130, 97]), (40, [200, 131]), (9, [14, 600])]  # 13 rows
 
 
 @pytest.fixture(scope="module", autouse=True)
