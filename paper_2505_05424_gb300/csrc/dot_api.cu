@@ -57,6 +57,7 @@ Geo dot::make_geo(const dot_grid& gr) {
   g.P = st;
   g.invh[0] = (double)gr.T;
   for (int d = 0; d < gr.D; ++d) g.invh[1 + d] = (double)gr.N[d];
+  for (int d = 0; d <= kMaxD; ++d) g.ih[d] = (float)g.invh[d];
   g.fP = make_fastdiv((unsigned)g.P);
   for (int d = 0; d < kMaxD; ++d) {
     g.fS[d] = make_fastdiv((unsigned)g.sst[d]);

@@ -103,6 +103,7 @@ struct Geo {
   long long P;           // nodes per time plane
   long long sst[kMaxD];  // element stride of spatial axis d inside a plane
   double invh[kMaxD + 1];  // 1/h: invh[0] = T, invh[1 + d] = N_d
+  float ih[kMaxD + 1];     // the same in FP32 (converting in a kernel takes FP64 issue slots)
   FastDiv fP;            // division by P
   FastDiv fS[kMaxD];     // division by sst[d]
   FastDiv fN[kMaxD];     // division by N[d]

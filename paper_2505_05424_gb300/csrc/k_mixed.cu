@@ -128,7 +128,7 @@ __global__ void k_residual(Geo g, MxFields fb) {
       float2 s = make_float2(0.f, 0.f);
       if (t >= 1) s = ff_add(s, ff_sub_exact(xi, x[i - g.P]));
       if (t < g.T) s = ff_add(s, ff_sub_exact(xi, x[i + g.P]));
-      const float ih = (float)g.invh[0];
+      const float ih = g.ih[0];
       acc = ff_add(acc, ff_mul_f(s, ih * ih));
     }
 #pragma unroll
@@ -138,7 +138,7 @@ __global__ void k_residual(Geo g, MxFields fb) {
       float2 s = make_float2(0.f, 0.f);
       if (xd >= 1) s = ff_add(s, ff_sub_exact(xi, x[i - st]));
       if (xd <= g.N[d] - 2) s = ff_add(s, ff_sub_exact(xi, x[i + st]));
-      const float ih = (float)g.invh[1 + d];
+      const float ih = g.ih[1 + d];
       acc = ff_add(acc, ff_mul_f(s, ih * ih));
     }
     const float2 r = ff_add(make_float2(f.b[i], f.blo[i]), ff_neg(ff_add(acc, mean)));
@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(kThreads, D == 2 ? 4 : 3) k_assemble_residual(
        i += (long long)gridDim.x * blockDim.x) {
     const int t = plane_of(g, i);
     const long long p = i - (long long)t * g.P;
-    const float ih0 = (float)g.invh[0];
+    const float ih0 = g.ih[0];
     float2 acc = make_float2(0.f, 0.f);    // b
     float2 lap = make_float2(0.f, 0.f);    // A^*A phi
     const float2 xi = x[i];
@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(kThreads, D == 2 ? 4 : 3) k_assemble_residual(
       const float* qd = f.q[1 + d];
       const float2* ad = f.al[1 + d];
       const long long s = g.sst[d];
-      const float ih = (float)g.invh[1 + d];
+      const float ih = g.ih[1 + d];
       float2 sd = make_float2(0.f, 0.f);
       if (xd >= 1) {
         const float2 w = ff_add_f(ff_neg(ad[i - s]), qd[i - s]);
@@ -276,84 +276,115 @@ __global__ void k_combine(Geo g, MxFields fb, float2* __restrict__ out) {
 
 // beta / sigma of component j at cone i, and its high part alone.
 template <int D>
-__device__ __forceinline__ float2 beta_ff(const float2* beta, int j, long long i, long long n0) {
+__device__ __forceinline__ float2 beta_ff(const float2* beta, int j, int i, int n0) {
   if (D == 2) {
     const float* p = reinterpret_cast<const float*>(beta) + beta2_at(j, i, n0);
     return make_float2(p[0], p[2]);
   }
-  return beta[(long long)j * n0 + i];
+  return beta[j * n0 + i];
 }
 template <int D>
-__device__ __forceinline__ float beta_hi(const float2* beta, int j, long long i, long long n0) {
+__device__ __forceinline__ float beta_hi(const float2* beta, int j, int i, int n0) {
   if (D == 2) return reinterpret_cast<const float*>(beta)[beta2_at(j, i, n0)];
-  return beta[(long long)j * n0 + i].x;
+  return beta[j * n0 + i].x;
 }
 
 template <int D>
-__device__ __forceinline__ void gather_Fq(const Geo& g, float* const* q, long long i, long long p, float* x) {
+__device__ __forceinline__ void gather_Fq(const Geo& g, float* const* q, int i, int p, float* x) {
+  const int P = (int)g.P;
   x[0] = q[0][i];
 #pragma unroll
   for (int d = 0; d < D; ++d) {
     const int xd = coord(g, p, d);
     const float* qd = q[1 + d];
-    const long long s = g.sst[d];
+    const int s = (int)g.sst[d];
     const bool lo = xd >= 1, hi = xd <= g.N[d] - 2;
     x[1 + 4 * d + 0] = lo ? qd[i - s] : 0.f;
     x[1 + 4 * d + 1] = hi ? qd[i] : 0.f;
-    x[1 + 4 * d + 2] = lo ? qd[i + g.P - s] : 0.f;
-    x[1 + 4 * d + 3] = hi ? qd[i + g.P] : 0.f;
+    x[1 + 4 * d + 2] = lo ? qd[i + P - s] : 0.f;
+    x[1 + 4 * d + 3] = hi ? qd[i + P] : 0.f;
   }
 }
 
 // ---- stopping measures: FP32 terms, per-thread FP32 sums, FP64 tree -----------
+//
+// Kinds of blocks run side by side -- cones, faces (D = 2: both axes of a node, which
+// share beta's pairs; D = 3: a kind per axis) and nodes -- each over its own sums.  A
+// 32-lane FP64 instruction occupies an SM for 16 cycles, so nothing per element is FP64
+// but the two planes that carry c, a block adds up only the sums of its kind, and a
+// warp's tree halves the number of sums a lane carries at every exchange (16 additions
+// for 16 sums instead of 80).  Bound by the latency of each element's loads; per check
+// on 256^2 x 64 219 us (0.73 GB read; 350 us when every block ran all kinds in turn with
+// FP64 on every node), 128^2 x 32 41 (86), 32^2 x 16 14 (49), 64^3 x 32 585 (983).  Four
+// CTAs per SM for D = 2 (three 241 us, five 237), three for D = 3 (four 643 us, five 618).
 
-#ifndef KKT_MIN_BLOCKS
-#define KKT_MIN_BLOCKS 3
-#endif
-// most blocks per slot of the stopping-measure kernel: one wave of KKT_MIN_BLOCKS
-// CTAs on each of the GPU's 152 SMs
-constexpr int kKktBlocks = 152 * KKT_MIN_BLOCKS;
+constexpr int kKktBlocks = 152 * 3;   // most blocks per slot and kind
+__host__ __device__ constexpr int kkt_kinds(int D) { return D == 2 ? 3 : 5; }
 
+// Partial sums of a slot: [R_NSLOTS][kinds * blocks].
 __host__ __device__ inline long long kkt_partials_len_slot(const Geo& g) {
-  return (long long)(g.D + 2) * kKktBlocks * R_NSLOTS;
+  return (long long)kkt_kinds(g.D) * kKktBlocks * R_NSLOTS;
 }
 
-// Blocks per slot of each stopping-measure kernel (at most kKktBlocks).
+// Blocks per slot of each kind (at most kKktBlocks; of the grid alone).
 inline int kkt_blocks(const Geo& g) {
   const long long nn = (long long)(g.T + 1) * g.P;
-  const long long b = (nn + 4 * kThreads - 1) / (4 * kThreads);
+  const long long b = (nn + kThreads - 1) / kThreads;
   return (int)(b < 1 ? 1 : (b > kKktBlocks ? kKktBlocks : b));
 }
 
-__device__ __forceinline__ void block_reduce_store(const float* accf, const double* accd, double* out_row) {
-  __shared__ double sh[kThreads / 32][R_NSLOTS];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// Sums of v[0 .. 15] over the warp: lane l returns the sum of v[l / 2].
+__device__ __forceinline__ double warp_sums16(double* v) {
+  const int lane = threadIdx.x & 31;
 #pragma unroll
-  for (int k = 0; k < R_NSLOTS; ++k) {
-    double v = (double)accf[k] + accd[k];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) sh[warp][k] = v;
+  for (int h = 8; h >= 1; h /= 2) {   // lanes exchange at distance 2 h and keep half of their sums
+    const bool up = lane & (2 * h);
+#pragma unroll
+    for (int k = 0; k < h; ++k) {
+      const double send = up ? v[k] : v[k + h], keep = up ? v[k + h] : v[k];
+      v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * h);
+    }
   }
+  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+// The block's sums of the slots listed in `which` (n of them) into out[slot rows + row].
+template <int NS>
+__device__ __forceinline__ void block_reduce_store(const double (&val)[NS], const int (&which)[NS], double* out,
+                                                   int rows, int row) {
+  static_assert(NS <= 16, "one exchange tree");
+  __shared__ double sh[kThreads / 32][16];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double v[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) v[k] = k < NS ? val[k < NS ? k : 0] : 0.0;
+  const double t = warp_sums16(v);
+  if ((lane & 1) == 0) sh[warp][lane >> 1] = t;
   __syncthreads();
   if (threadIdx.x < R_NSLOTS) {
-    double v = 0.0;
-    for (int w = 0; w < kThreads / 32; ++w) v += sh[w][threadIdx.x];
-    out_row[threadIdx.x] = v;
+    int at = -1;
+#pragma unroll
+    for (int k = 0; k < NS; ++k)
+      if (which[k] == (int)threadIdx.x) at = k;
+    double s = 0.0;
+    if (at >= 0)
+      for (int w = 0; w < kThreads / 32; ++w) s += sh[w][at];
+    out[(long long)threadIdx.x * rows + row] = s;
   }
 }
 
 // One node's share of the stopping measures: its cone (t < T), its faces along
 // every axis (the face after the node), and the node itself.
 template <int D>
-__device__ __forceinline__ void kkt_cone(const Geo& g, const MxFields& f, float sg, long long i, long long p,
+__device__ __forceinline__ void kkt_cone(const Geo& g, const MxFields& f, float sg, int i, int p,
                                          int use_z, float* acc) {
   constexpr int K = 4 * D + 2;
-  const long long n0 = (long long)g.T * g.P;
+  const int P = (int)g.P, n0 = g.T * P;
   const float s_default = 0.70710678118654752f;
-  const float ih0 = (float)g.invh[0];
+  const float ih0 = g.ih[0];
   float x[K - 1];
   gather_Fq<D>(g, f.q, i, p, x);
-  const float2 gp = grad_pair(f.phi, i, i + g.P, ih0);
+  const float2 gp = grad_pair(f.phi, i, i + P, ih0);
   const float aphi = gp.x + gp.y;
   const float q0 = x[0];
   const float dq = grad_minus(gp, q0);
@@ -377,10 +408,10 @@ __device__ __forceinline__ void kkt_cone(const Geo& g, const MxFields& f, float 
     acc[R_SOCP] += r * r;
 #pragma unroll
     for (int j = 1; j < K - 1; ++j) {
-      r = fmaf(-s, x[j], f.z[(long long)j * n0 + i]);
+      r = fmaf(-s, x[j], f.z[j * n0 + i]);
       acc[R_SOCP] += r * r;
     }
-    r = (f.z[(long long)(K - 1) * n0 + i] - 1.f) - q0;
+    r = (f.z[(K - 1) * n0 + i] - 1.f) - q0;
     acc[R_SOCP] += r * r;
   }
   const float2 bK = beta_ff<D>(f.beta, K - 1, i, n0), b0 = beta_ff<D>(f.beta, 0, i, n0);
@@ -390,16 +421,16 @@ __device__ __forceinline__ void kkt_cone(const Geo& g, const MxFields& f, float 
 }
 
 template <int D>
-__device__ __forceinline__ void kkt_face(const Geo& g, const MxFields& f, float sg, int d, long long i, int t,
-                                         long long p, float* acc, float2* dual) {
-  const long long n0 = (long long)g.T * g.P;
+__device__ __forceinline__ void kkt_face(const Geo& g, const MxFields& f, float sg, int d, int i, int t, int p,
+                                         float* acc, float2* dual) {
+  const int P = (int)g.P, n0 = g.T * P;
   const float s_default = 0.70710678118654752f;
-  const long long s = g.sst[d];
+  const int s = (int)g.sst[d];
   const float* qd = f.q[1 + d];
   const float2* ad = f.al[1 + d];
   const float2* a0 = f.al[0];
   const int cbase = 1 + 4 * d;
-  const float ih = (float)g.invh[1 + d];
+  const float ih = g.ih[1 + d];
   const float2 gp = grad_pair(f.phi, i, i + s, ih);
   const float aphi = gp.x + gp.y;
   const float q = qd[i];
@@ -415,8 +446,8 @@ __device__ __forceinline__ void kkt_face(const Geo& g, const MxFields& f, float 
     fbb += s_r * beta_hi<D>(f.beta, cbase + 0, i + s, n0) + s_l * beta_hi<D>(f.beta, cbase + 1, i, n0);
   }
   if (t >= 1) {
-    den += om_r * a0[i - g.P + s].x + om_l * a0[i - g.P].x;
-    fbb += s_r * beta_hi<D>(f.beta, cbase + 2, i - g.P + s, n0) + s_l * beta_hi<D>(f.beta, cbase + 3, i - g.P, n0);
+    den += om_r * a0[i - P + s].x + om_l * a0[i - P].x;
+    fbb += s_r * beta_hi<D>(f.beta, cbase + 2, i - P + s, n0) + s_l * beta_hi<D>(f.beta, cbase + 3, i - P, n0);
   }
   den *= 0.25f * sg;
   fbb *= sg;
@@ -432,111 +463,118 @@ __device__ __forceinline__ void kkt_face(const Geo& g, const MxFields& f, float 
   acc[R_FBB] += fbb * fbb;
 }
 
-// A^*alpha + c at a node (in two-float arithmetic: the divergence of alpha cancels
-// against c to the level of the dual residual) and <c, phi> in FP64.
+// The faces of axis AX of every node; D = 2: of both axes of a node together (they share
+// beta's pairs).
+template <int D, int AX>
+__device__ __forceinline__ void kkt_face_loop(const Geo& g, const MxFields& f, float sg, int i0, int stride, float* acc,
+                                              float2* dual) {
+  const int P = (int)g.P, n = (g.T + 1) * P;
+#pragma unroll 1
+  for (int i = i0; i < n; i += stride) {
+    const int t = plane_of(g, i), p = i - t * P;
+    if (coord(g, p, AX) <= g.N[AX] - 2) kkt_face<D>(g, f, sg, AX, i, t, p, acc, dual);
+    if (D == 2 && coord(g, p, 1) <= g.N[1] - 2) kkt_face<D>(g, f, sg, 1, i, t, p, acc, dual);
+  }
+}
+
+// A^*alpha at a node in two-float arithmetic (on the planes that carry c, the divergence
+// of alpha cancels against c to the level of the dual residual).
 template <int D>
-__device__ __forceinline__ void kkt_node(const Geo& g, const MxFields& f, float2 sg2, long long i, int t,
-                                         long long p, float* acc, double* dres, double* cphi) {
+__device__ __forceinline__ float2 kkt_div(const Geo& g, const MxFields& f, float2 sg2, int i, int t, int p) {
+  const int P = (int)g.P;
   float2 v = make_float2(0.f, 0.f);
-  const float ih0 = (float)g.invh[0];
-  if (t >= 1) v = ff_add(v, ff_mul_f(f.al[0][i - g.P], ih0));
-  if (t < g.T) v = ff_add(v, ff_mul_f(ff_neg(f.al[0][i]), ih0));
+  if (t >= 1) v = ff_add(v, ff_mul_f(f.al[0][i - P], g.ih[0]));
+  if (t < g.T) v = ff_add(v, ff_mul_f(ff_neg(f.al[0][i]), g.ih[0]));
 #pragma unroll
   for (int d = 0; d < D; ++d) {
     const int x = coord(g, p, d);
     const float2* ad = f.al[1 + d];
-    const long long s = g.sst[d];
-    const float ih = (float)g.invh[1 + d];
+    const int s = (int)g.sst[d];
+    const float ih = g.ih[1 + d];
     if (x >= 1) v = ff_add(v, ff_mul_f(ad[i - s], ih));
     if (x <= g.N[d] - 2) v = ff_add(v, ff_mul_f(ff_neg(ad[i]), ih));
   }
-  v = ff_mul(v, sg2);   // A^* alpha = sigma A^*(alpha / sigma)
-  double c = 0.0;
-  if (t == 0) c += f.m0[p];
-  if (t == g.T) c -= f.m1[p];
-  if (c != 0.0) {
-    const double res = ff_to_double(v) + c;
-    *dres += res * res;
-    *cphi += c * ff_to_double(f.phi[i]);
-  } else {
-    const float res = v.x + v.y;
-    acc[R_DUALRES] += res * res;
-  }
+  return ff_mul(v, sg2);   // A^* alpha = sigma A^*(alpha / sigma)
 }
 
-// All stopping-measure sums (one partial row per block), in D + 2 passes over the
-// nodes: the cones, the faces of each axis, the nodes.  Separate loops keep each
-// pass's loads in flight with few registers (one fused loop body needed ~220).
+// All stopping-measure sums: blockIdx.z picks the kind.  socp (nullable): per-slot sums of
+// |z - BFq - d|^2 left by the fused D = 2 pass; without it the cones read z.
 template <int D>
-__global__ void __launch_bounds__(kThreads, KKT_MIN_BLOCKS) k_kkt(Geo g, MxFields fb, double* partials_all, int use_z) {
-  const int slot = blockIdx.y;
+__global__ void __launch_bounds__(kThreads, D == 2 ? 4 : 3) k_kkt(const __grid_constant__ Geo g,
+                                                     const __grid_constant__ MxFields fb, double* partials_all,
+                                                     const double* socp_all, int nsocp) {
+  const int slot = blockIdx.y, kind = blockIdx.z;
   if (!fb.sp[slot].active) return;
   const MxFields f = slot_view(fb, g, slot);
   const float2 sg2 = fb.sp[slot].sg;
   const float sg = sg2.x + sg2.y;
   double* partials = partials_all + slot * kkt_partials_len_slot(g);
+  const int rows = kkt_kinds(D) * gridDim.x, row = kind * gridDim.x + blockIdx.x;
+  const int P = (int)g.P, n = (g.T + 1) * P, n0 = g.T * P;
+  const int i0 = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
   float acc[R_NSLOTS];
 #pragma unroll
   for (int k = 0; k < R_NSLOTS; ++k) acc[k] = 0.f;
-  double dres = 0.0, cphi = 0.0;
-  float2 dual = make_float2(0.f, 0.f);
-  const long long n = (long long)(g.T + 1) * g.P, n0 = (long long)g.T * g.P;
-  const long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
+  if (kind == 0) {
+    const int use_z = socp_all == nullptr;
 #pragma unroll 1
-  for (long long i = i0; i < n0; i += stride) {
-    const int t = plane_of(g, i);
-    kkt_cone<D>(g, f, sg, i, i - (long long)t * g.P, use_z, acc);
-  }
+    for (int i = i0; i < n0; i += stride) kkt_cone<D>(g, f, sg, i, i - plane_of(g, i) * P, use_z, acc);
+    constexpr int w[9] = {R_PRIM, R_APHI, R_Q, R_COMP0, R_ALPHA0, R_F, R_SOCP, R_SOCD, R_FBB};
+    double v[9];
 #pragma unroll
-  for (int d = 0; d < D; ++d) {
-#pragma unroll 1
-    for (long long i = i0; i < n; i += stride) {
+    for (int k = 0; k < 9; ++k) v[k] = acc[w[k]];
+    block_reduce_store(v, w, partials, rows, row);
+  } else if (kind < kkt_kinds(D) - 1) {
+    float2 dual = make_float2(0.f, 0.f);
+    if (kind == 1) kkt_face_loop<D, 0>(g, f, sg, i0, stride, acc, &dual);
+    else if (kind == 2) kkt_face_loop<D, 1>(g, f, sg, i0, stride, acc, &dual);
+    else kkt_face_loop<D, D - 1>(g, f, sg, i0, stride, acc, &dual);
+    constexpr int w[9] = {R_PRIM, R_APHI, R_Q, R_COMPD, R_ALPHAB, R_G, R_SOCD, R_FBB, R_DUALOBJ};
+    double v[9];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = acc[w[k]];
+    v[8] = ff_to_double(dual);
+    block_reduce_store(v, w, partials, rows, row);
+  } else {
+    // planes 1 .. T - 1 carry no c
+#pragma unroll 2
+    for (int i = P + i0; i < n0; i += stride) {
       const int t = plane_of(g, i);
-      const long long p = i - (long long)t * g.P;
-      if (coord(g, p, d) <= g.N[d] - 2) kkt_face<D>(g, f, sg, d, i, t, p, acc, &dual);
+      const float2 v = kkt_div<D>(g, f, sg2, i, t, i - t * P);
+      const float res = v.x + v.y;
+      acc[R_DUALRES] += res * res;
     }
-  }
+    double dres = 0.0, cphi = 0.0, socp = 0.0;
 #pragma unroll 1
-  for (long long i = i0; i < n; i += stride) {
-    const int t = plane_of(g, i);
-    kkt_node<D>(g, f, sg2, i, t, i - (long long)t * g.P, acc, &dres, &cphi);
+    for (int j = i0; j < 2 * P; j += stride) {
+      const int t = j < P ? 0 : g.T, p = j < P ? j : j - P;
+      const double c = j < P ? f.m0[p] : -f.m1[p];
+      const double res = ff_to_double(kkt_div<D>(g, f, sg2, t * P + p, t, p)) + c;
+      dres += res * res;
+      cphi += c * ff_to_double(f.phi[t * P + p]);
+    }
+    if (socp_all)
+      for (int i = i0; i < nsocp; i += stride) socp += socp_all[(long long)slot * nsocp + i];
+    constexpr int w[3] = {R_DUALRES, R_SOCP, R_CPHI};
+    const double v[3] = {(double)acc[R_DUALRES] + dres, socp, cphi};
+    block_reduce_store(v, w, partials, rows, row);
   }
-  double accd[R_NSLOTS];
-#pragma unroll
-  for (int k = 0; k < R_NSLOTS; ++k) accd[k] = 0.0;
-  accd[R_DUALRES] = dres;
-  accd[R_CPHI] = cphi;
-  accd[R_DUALOBJ] = ff_to_double(dual);
-  block_reduce_store(acc, accd, partials + (long long)blockIdx.x * R_NSLOTS);
 }
 
-// rows: kernel groups (D + 2) x kb blocks; group j's partials start at row j * kKktBlocks.
-__global__ void k_kkt_final(Geo g, const SlotParam* sp, const double* partials_all, int groups, int kb,
-                            double* out_all, const double* socp_all, int nsocp) {
-  const int slot = blockIdx.x;
+// out[slot][k] = the sum of the rows of partials, a block per sum.
+__global__ void __launch_bounds__(128) k_kkt_final(Geo g, const SlotParam* sp, const double* partials_all, int rows,
+                                                   double* out_all) {
+  const int slot = blockIdx.x, k = blockIdx.y;
   if (!sp[slot].active) return;
-  const double* partials = partials_all + slot * kkt_partials_len_slot(g);
-  double* out = out_all + slot * R_NSLOTS;
-  const double* socp_part = socp_all ? socp_all + (long long)slot * nsocp : nullptr;
-  const int rows = groups * kb;
-  __shared__ double sh[kThreads];
-  for (int k = 0; k < R_NSLOTS; ++k) {
-    double v = 0.0;
-    for (int e = threadIdx.x; e < rows; e += blockDim.x) {
-      const int j = e / kb, r = e - j * kb;
-      v += partials[((long long)j * kKktBlocks + r) * R_NSLOTS + k];
-    }
-    if (k == R_SOCP && socp_part)
-      for (int r = threadIdx.x; r < nsocp; r += blockDim.x) v += socp_part[r];
-    sh[threadIdx.x] = v;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-      if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) out[k] = sh[0];
-    __syncthreads();
-  }
+  const double* p = partials_all + slot * kkt_partials_len_slot(g) + (long long)k * rows;
+  double v = 0.0;
+#pragma unroll 4
+  for (int r = threadIdx.x; r < rows; r += 128) v += p[r];
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  __shared__ double sh[4];
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) out_all[slot * R_NSLOTS + k] = (sh[0] + sh[1]) + (sh[2] + sh[3]);
 }
 
 // Line 2 with one refinement step: phi1 = P(b); r = b - A^*A phi1 (exact);
@@ -587,8 +625,8 @@ template <int D>
 void launch_kkt_tmpl(const Geo& g, int G, const MxFields& f, double* partials, double* out,
                      const double* socp_part, int nsocp, cudaStream_t s, LaunchCounter lc) {
   const int kb = kkt_blocks(g);
-  k_kkt<D><<<dim3(kb, G), kThreads, 0, s>>>(g, f, partials, socp_part ? 0 : 1);
-  k_kkt_final<<<G, kThreads, 0, s>>>(g, f.sp, partials, 1, kb, out, socp_part, nsocp);
+  k_kkt<D><<<dim3(kb, G, kkt_kinds(D)), kThreads, 0, s>>>(g, f, partials, socp_part, nsocp);
+  k_kkt_final<<<dim3(G, R_NSLOTS), 128, 0, s>>>(g, f.sp, partials, kkt_kinds(D) * kb, out);
   lc.launched(KID_KKT, 2);
 }
 
