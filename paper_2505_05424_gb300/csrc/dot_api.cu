@@ -537,7 +537,6 @@ int dot_kkt(dot_ctx* c, double* kkt) {
 int dot_get(dot_ctx* c, double* rho, double* m, double* phi, double* objective, double* kkt) {
   if (!c) return fail(nullptr, DOT_EINVAL, "ctx is NULL");
   DeviceScope dev(c->device);
-  const Geo& g = c->geo;
   if (objective || kkt) {
     int rc = compute_kkt(c);
     if (rc != DOT_OK) return rc;
@@ -547,16 +546,6 @@ int dot_get(dot_ctx* c, double* rho, double* m, double* phi, double* objective, 
   std::string perr;
   int rc = c->path->read_fields(rho, m, phi, c->stream, &perr);
   if (rc != DOT_OK) return fail(c, rc, perr);
-  const double invh0 = (double)g.T;   // rho = alpha_0 / h_0, m = alpha_bar / h_0
-  if (rho) {
-    const long long n0 = (long long)g.T * g.P;
-    for (long long i = 0; i < n0; ++i) rho[i] *= invh0;
-  }
-  if (m) {
-    long long nm = 0;
-    for (int d = 0; d < g.D; ++d) nm += (long long)(g.T + 1) * g.P / g.N[d] * (g.N[d] - 1);
-    for (long long i = 0; i < nm; ++i) m[i] *= invh0;
-  }
   return DOT_OK;
 }
 

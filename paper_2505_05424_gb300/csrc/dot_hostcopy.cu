@@ -1,0 +1,114 @@
+// dot_hostcopy.cu -- device fields to packed FP64 host arrays (dot_get).
+//
+// Converting a field on one host thread after one copy into pageable memory ran at
+// about 4 GB/s, page faults of the caller's fresh arrays included, and took as long as
+// 60 iterations on 256^2 x 64.  The fields are cut into chunks that a few threads
+// take in turn: copy the chunk into the thread's pinned buffer, convert it into the
+// caller's array.  Fields below 4 MB stay on the calling thread: starting threads and
+// pinning buffers costs about as much as converting them.
+#include <algorithm>
+#include <atomic>
+#include <system_error>
+#include <thread>
+
+#include "dot_hostcopy.cuh"
+
+namespace dot {
+namespace {
+
+constexpr size_t kChunk = 512 * 1024;            // bytes of one copy
+constexpr size_t kThreadedBytes = 4 << 20;
+constexpr int kWorkers = 8;
+
+struct Task {
+  const HostRead* part;
+  size_t r0, nr, c0, nc;   // nr rows from r0, columns [c0, c0 + nc)
+};
+
+size_t elem_bytes(HostElem e) { return e == HOST_F32 ? 4 : e == HOST_FF || e == HOST_F64 ? 8 : 16; }
+
+cudaError_t run_task(const Task& t, void* buf, cudaStream_t s) {
+  const HostRead& p = *t.part;
+  const size_t eb = elem_bytes(p.elem);
+  const char* src = static_cast<const char*>(p.src) + (t.r0 * p.pitch + t.c0) * eb;
+  cudaError_t e;
+  if (t.nr == 1 || (t.nc == p.pitch)) e = cudaMemcpyAsync(buf, src, t.nr * t.nc * eb, cudaMemcpyDeviceToHost, s);
+  else e = cudaMemcpy2DAsync(buf, t.nc * eb, src, p.pitch * eb, t.nc * eb, t.nr, cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) return e;
+  double* d = p.dst + t.r0 * p.width + t.c0;
+  const size_t n = t.nr * t.nc;
+  const double s1 = p.s1, s2 = p.s2;
+  if (p.elem == HOST_F32) {
+    const float* v = static_cast<const float*>(buf);
+    for (size_t i = 0; i < n; ++i) d[i] = (double)v[i] * s1 * s2;
+  } else if (p.elem == HOST_FF) {
+    const float2* v = static_cast<const float2*>(buf);
+    for (size_t i = 0; i < n; ++i) d[i] = s1 * ((double)v[i].x + (double)v[i].y) * s2;
+  } else if (p.elem != HOST_F64) {
+    const float* v = static_cast<const float*>(buf) + (p.elem == HOST_LANE1 ? 1 : 0);
+    for (size_t i = 0; i < n; ++i) d[i] = s1 * ((double)v[4 * i] + (double)v[4 * i + 2]) * s2;
+  } else {
+    const double* v = static_cast<const double*>(buf);
+    for (size_t i = 0; i < n; ++i) d[i] = v[i] * s1 * s2;
+  }
+  return cudaSuccess;
+}
+
+}  // namespace
+
+cudaError_t read_to_host(const std::vector<HostRead>& parts, cudaStream_t s) {
+  cudaError_t e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) return e;
+  std::vector<Task> tasks;
+  size_t bytes = 0;
+  for (const HostRead& p : parts) {
+    const size_t eb = elem_bytes(p.elem), cap = kChunk / eb;
+    bytes += p.width * p.rows * eb;
+    if (p.width == 0 || p.rows == 0) continue;
+    if (p.width >= cap) {
+      for (size_t r = 0; r < p.rows; ++r)
+        for (size_t c = 0; c < p.width; c += cap) tasks.push_back({&p, r, 1, c, std::min(cap, p.width - c)});
+    } else {
+      const size_t nr = cap / p.width;
+      for (size_t r = 0; r < p.rows; r += nr) tasks.push_back({&p, r, std::min(nr, p.rows - r), 0, p.width});
+    }
+  }
+  const int hw = (int)std::thread::hardware_concurrency();
+  int workers = bytes < kThreadedBytes ? 1 : std::min(kWorkers, std::max(1, hw));
+  workers = std::min<int>(workers, std::max<size_t>(1, tasks.size()));
+  char* pinned = nullptr;
+  if (workers > 1 && cudaMallocHost(&pinned, workers * kChunk) != cudaSuccess) {
+    cudaGetLastError();
+    pinned = nullptr;
+    workers = 1;
+  }
+  std::vector<char> pageable(pinned ? 0 : kChunk);
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::atomic<size_t> next{0};
+  std::atomic<int> err{cudaSuccess};
+  auto work = [&](char* buf) {
+    for (size_t k; (k = next.fetch_add(1)) < tasks.size() && err.load() == cudaSuccess;) {
+      const cudaError_t r = run_task(tasks[k], buf, s);
+      if (r != cudaSuccess) err.store(r);
+    }
+  };
+  std::vector<std::thread> th;
+  th.reserve(workers);
+  for (int w = 1; w < workers; ++w) {
+    try {
+      th.emplace_back([&, w] {
+        if (cudaSetDevice(dev) == cudaSuccess) work(pinned + w * kChunk);
+      });
+    } catch (const std::system_error&) {
+      break;                                     // the threads that did start share the tasks
+    }
+  }
+  work(pinned ? pinned : pageable.data());
+  for (std::thread& t : th) t.join();
+  if (pinned) cudaFreeHost(pinned);
+  return (cudaError_t)err.load();
+}
+
+}  // namespace dot

@@ -81,7 +81,8 @@ class Path {
   // Stopping-measure sums into red_out() (device, R_NSLOTS doubles).
   virtual void kkt(cudaStream_t s, LaunchCounter lc) = 0;
   virtual const double* red_out() const = 0;
-  // alpha_0 (natural layout) into rho, alpha_bar (natural layout) into m, phi; NULL = skip.
+  // alpha_0 / h_0 (natural layout) into rho, alpha_bar / h_0 (natural layout) into m, phi;
+  // NULL = skip.
   virtual int read_fields(double* rho, double* m, double* phi, cudaStream_t s, std::string* err) = 0;
   virtual int read_state(double* q, double* al, double* beta, cudaStream_t s, std::string* err) = 0;
   // The state with the penalty sigma it belongs to (the next iterate uses sigma).

@@ -396,13 +396,8 @@ void dot_server::retire(Batch& b, int k, int status) {
     r->m.resize(nm);
     r->phi.resize(nn);
     std::string why;
-    if (b.mb->read_fields(k, r->rho.data(), r->m.data(), r->phi.data(), b.stream, &why) != DOT_OK) {
+    if (b.mb->read_fields(k, r->rho.data(), r->m.data(), r->phi.data(), b.stream, &why) != DOT_OK)
       status = DOT_ECUDA;
-    } else {
-      const double invh0 = (double)g.T;   // rho = alpha_0 / h_0, m = alpha_bar / h_0
-      for (double& v : r->rho) v *= invh0;
-      for (double& v : r->m) v *= invh0;
-    }
   }
   r->objective = -2.0 * r->kkt[DOT_KKT_PRIMAL] / (double)b.geo.P;
   b.mb->set_active(k, false);

@@ -4,6 +4,7 @@
 #include <cstring>
 
 #include "dot_fft.cuh"
+#include "dot_hostcopy.cuh"
 #include "dot_paths.cuh"
 
 namespace dot {
@@ -147,18 +148,18 @@ class PathF64 : public Path {
   const double* red_out() const override { return B_.red; }
 
   int read_fields(double* rho, double* m, double* phi, cudaStream_t s, std::string* err) override {
-    cudaError_t e = cudaSuccess;
     const size_t n0 = (size_t)g_.T * g_.P, nn = (size_t)(g_.T + 1) * g_.P;
-    if (rho) e = cudaMemcpyAsync(rho, B_.f.al[0], n0 * sizeof(double), cudaMemcpyDeviceToHost, s);
-    if (m && e == cudaSuccess) {
-      double* dst = m;
-      for (int fam = 1; fam <= g_.D && e == cudaSuccess; ++fam) {
-        e = copy_face_d2h(fam, B_.f.al[fam], dst, s);
-        dst += natural_face_count(g_, fam);
-      }
+    const double invh0 = (double)g_.T;
+    std::vector<HostRead> parts;
+    if (rho) parts.push_back({B_.f.al[0], rho, n0, n0, 1, HOST_F64, 1.0, invh0});
+    for (int fam = 1; m && fam <= g_.D; ++fam) {
+      size_t w, p, h;
+      face_copy_shape(g_, fam, &w, &p, &h);
+      parts.push_back({B_.f.al[fam], m, w, p, h, HOST_F64, 1.0, invh0});
+      m += natural_face_count(g_, fam);
     }
-    if (phi && e == cudaSuccess) e = cudaMemcpyAsync(phi, B_.f.phi, nn * sizeof(double), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (phi) parts.push_back({B_.f.phi, phi, nn, nn, 1, HOST_F64, 1.0, 1.0});
+    const cudaError_t e = read_to_host(parts, s);
     if (e != cudaSuccess) { *err = std::string("read_fields: ") + cudaGetErrorString(e); return DOT_ECUDA; }
     return DOT_OK;
   }

@@ -9,6 +9,7 @@
 #include <cstring>
 
 #include "dot_batch.cuh"
+#include "dot_hostcopy.cuh"
 
 namespace dot {
 
@@ -422,25 +423,7 @@ void MixedBatch::kkt(cudaStream_t s, LaunchCounter lc) {
 
 namespace {
 
-// padded device face field (T+1 planes) <-> natural host layout
-cudaError_t face_f_d2h(const Geo& g, int fam, const float* src, double* dst, cudaStream_t s) {
-  size_t w, p, h;
-  face_copy_shape(g, fam, &w, &p, &h);
-  std::vector<float> t(w * h);
-  cudaError_t e = cudaMemcpy2DAsync(t.data(), w * 4, src, p * 4, w * 4, h, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  for (size_t i = 0; i < w * h; ++i) dst[i] = t[i];
-  return e;
-}
-cudaError_t face_ff_d2h(const Geo& g, int fam, const float2* src, double* dst, cudaStream_t s) {
-  size_t w, p, h;
-  face_copy_shape(g, fam, &w, &p, &h);
-  std::vector<float2> t(w * h);
-  cudaError_t e = cudaMemcpy2DAsync(t.data(), w * 8, src, p * 8, w * 8, h, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  for (size_t i = 0; i < w * h; ++i) dst[i] = (double)t[i].x + (double)t[i].y;
-  return e;
-}
+// natural host layout -> padded device face field (T+1 planes)
 cudaError_t face_h2d(const Geo& g, int fam, float* qd, float2* ad, const double* q, const double* al,
                      double ascale, cudaStream_t s) {
   size_t w, p, h;
@@ -457,80 +440,48 @@ cudaError_t face_h2d(const Geo& g, int fam, float* qd, float2* ad, const double*
 }  // namespace
 
 int MixedBatch::read_fields(int b, double* rho, double* m, double* phi, cudaStream_t s, std::string* err) {
-  cudaError_t e = cudaSuccess;
   const size_t n0 = (size_t)g_.T * g_.P, nn = (size_t)(g_.T + 1) * g_.P;
   const MxFields fc = slot_view(cur(), g_, b);
-  const double sig = hs_[b];   // the stored multipliers are alpha / sigma
-  if (rho) {
-    std::vector<float2> t(n0);
-    e = down(t.data(), fc.al[0], n0 * 8, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    for (size_t i = 0; i < n0; ++i) rho[i] = sig * ((double)t[i].x + (double)t[i].y);
+  const double sig = hs_[b], invh0 = (double)g_.T;   // the stored multipliers are alpha / sigma
+  std::vector<HostRead> parts;
+  if (rho) parts.push_back({fc.al[0], rho, n0, n0, 1, HOST_FF, sig, invh0});
+  for (int fam = 1; m && fam <= g_.D; ++fam) {
+    size_t w, p, h;
+    face_copy_shape(g_, fam, &w, &p, &h);
+    parts.push_back({fc.al[fam], m, w, p, h, HOST_FF, sig, invh0});
+    m += natural_face_count(g_, fam);
   }
-  if (m && e == cudaSuccess) {
-    double* dst = m;
-    for (int fam = 1; fam <= g_.D && e == cudaSuccess; ++fam) {
-      e = face_ff_d2h(g_, fam, fc.al[fam], dst, s);
-      const long long n = natural_face_count(g_, fam);
-      for (long long i = 0; i < n; ++i) dst[i] *= sig;
-      dst += n;
-    }
-  }
-  if (phi && e == cudaSuccess) {
-    std::vector<float2> t(nn);
-    e = down(t.data(), fc.phi, nn * 8, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    for (size_t i = 0; i < nn; ++i) phi[i] = (double)t[i].x + (double)t[i].y;
-  }
+  if (phi) parts.push_back({fc.phi, phi, nn, nn, 1, HOST_FF, 1.0, 1.0});
+  const cudaError_t e = read_to_host(parts, s);
   if (e != cudaSuccess) { *err = std::string("read_fields: ") + cudaGetErrorString(e); return DOT_ECUDA; }
   return DOT_OK;
 }
 
 int MixedBatch::read_state(int b, double* q, double* al, double* beta, cudaStream_t s, std::string* err) {
-  cudaError_t e = cudaSuccess;
   const size_t n0 = (size_t)g_.T * g_.P;
   const MxFields fc = slot_view(cur(), g_, b);
-  if (q) {
-    std::vector<float> t(n0);
-    e = down(t.data(), fc.q[0], n0 * 4, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    for (size_t i = 0; i < n0; ++i) q[i] = t[i];
-    double* dst = q + n0;
-    for (int fam = 1; fam <= g_.D && e == cudaSuccess; ++fam) {
-      e = face_f_d2h(g_, fam, fc.q[fam], dst, s);
-      dst += natural_face_count(g_, fam);
-    }
-  }
   const double sig = hs_[b];   // the stored multipliers are alpha / sigma, beta / sigma
-  if (al && e == cudaSuccess) {
-    std::vector<float2> t(n0);
-    e = down(t.data(), fc.al[0], n0 * 8, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    for (size_t i = 0; i < n0; ++i) al[i] = sig * ((double)t[i].x + (double)t[i].y);
-    double* dst = al + n0;
-    for (int fam = 1; fam <= g_.D && e == cudaSuccess; ++fam) {
-      e = face_ff_d2h(g_, fam, fc.al[fam], dst, s);
-      const long long n = natural_face_count(g_, fam);
-      for (long long i = 0; i < n; ++i) dst[i] *= sig;
-      dst += n;
-    }
+  std::vector<HostRead> parts;
+  if (q) parts.push_back({fc.q[0], q, n0, n0, 1, HOST_F32, 1.0, 1.0});
+  if (al) parts.push_back({fc.al[0], al, n0, n0, 1, HOST_FF, sig, 1.0});
+  size_t off = n0;
+  for (int fam = 1; fam <= g_.D; ++fam) {
+    size_t w, p, h;
+    face_copy_shape(g_, fam, &w, &p, &h);
+    if (q) parts.push_back({fc.q[fam], q + off, w, p, h, HOST_F32, 1.0, 1.0});
+    if (al) parts.push_back({fc.al[fam], al + off, w, p, h, HOST_FF, sig, 1.0});
+    off += (size_t)natural_face_count(g_, fam);
   }
-  if (beta && e == cudaSuccess) {
-    const size_t nb = (size_t)g_.K * n0;
-    std::vector<float2> t(nb);
-    e = down(t.data(), fc.beta, nb * 8, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  for (int j = 0; beta && j < g_.K; ++j) {
     if (g_.D == 2) {
-      const float* p = reinterpret_cast<const float*>(t.data());
-      for (int j = 0; j < g_.K; ++j)
-        for (size_t i = 0; i < n0; ++i) {
-          const long long o = beta2_at(j, (long long)i, (long long)n0);
-          beta[j * n0 + i] = sig * ((double)p[o] + (double)p[o + 2]);
-        }
+      const long long o = beta2_at(j, 0, (long long)n0);
+      parts.push_back({reinterpret_cast<const float*>(fc.beta) + o / 4 * 4, beta + j * n0, n0, n0, 1,
+                       o % 4 ? HOST_LANE1 : HOST_LANE0, sig, 1.0});
     } else {
-      for (size_t i = 0; i < nb; ++i) beta[i] = sig * ((double)t[i].x + (double)t[i].y);
+      parts.push_back({fc.beta + j * n0, beta + j * n0, n0, n0, 1, HOST_FF, sig, 1.0});
     }
   }
+  const cudaError_t e = read_to_host(parts, s);
   if (e != cudaSuccess) { *err = std::string("read_state: ") + cudaGetErrorString(e); return DOT_ECUDA; }
   return DOT_OK;
 }
