@@ -25,9 +25,8 @@ struct SlotParam {
 struct MxFields {
   float* q[kMaxD + 1];     // q_0: T*P; q_d: (T+1)*P padded
   float2* al[kMaxD + 1];   // alpha / sigma (two-float), same shapes as q
-  float2* beta;            // beta / sigma (two-float), K * T * P; component planes for D = 3, for
-                           // D = 2 the pairs of beta2_at
-  float* z;                // K * T * P
+  float2* beta;            // beta / sigma (two-float), K * T * P, in the pairs of pair_of
+  float* z;                // K * T * P (D = 3), in the same pairs
   float2* phi;             // (T+1)*P two-float potential
   float* b;                // (T+1)*P right-hand side, high part; reused for the correction delta
   float* blo;              // (T+1)*P right-hand side, low part (b = b + blo as a two-float)
@@ -43,15 +42,34 @@ struct MxFields {
   const SlotParam* sp;     // G slot parameters
 };
 
-// D = 2: beta is stored as five planes of float4, one per pair of cone components
-// (0, 9), (1, 5), (2, 6), (3, 7), (4, 8) -- the x-face and y-face components of the
-// same kind side by side -- holding both high parts, then both low parts: the lane
-// pairs that the fused pass computes in, loaded and stored without rearranging.
-// Index of component j's high part at cone i (of n0) in floats; its low part is two
-// floats further.
-__host__ __device__ inline long long beta2_at(int j, long long i, long long n0) {
-  const int pair = j == 9 ? 0 : j <= 4 ? j : j - 4, lane = j == 9 || (j >= 5) ? 1 : 0;
-  return (pair * n0 + i) * 4 + lane;
+// beta is stored as K/2 planes of float4, one per pair of cone components, holding both
+// high parts, then both low parts; z as K/2 planes of float2.  Pairs: (0, K-1); the x-face
+// and y-face components of the same kind, (1, 5), (2, 6), (3, 7), (4, 8); for D = 3 also
+// (9, 10), (11, 12).  They are the lane pairs that the fused passes compute in, loaded and
+// stored without rearranging.
+__host__ __device__ inline void pair_of(int K, int j, int* pair, int* lane) {
+  if (j == 0 || j == K - 1) {
+    *pair = 0;
+    *lane = j != 0;
+  } else if (j <= 8) {
+    *pair = j <= 4 ? j : j - 4;
+    *lane = j > 4;
+  } else {
+    *pair = 5 + (j - 9) / 2;
+    *lane = (j - 9) % 2;
+  }
+}
+// Index (in floats) of component j's high part of beta at cone i of n0 (its low part is two
+// floats further), and of z.
+__host__ __device__ inline long long beta_at(int K, int j, long long i, long long n0) {
+  int p, l;
+  pair_of(K, j, &p, &l);
+  return (p * n0 + i) * 4 + l;
+}
+__host__ __device__ inline long long z_at(int K, int j, long long i, long long n0) {
+  int p, l;
+  pair_of(K, j, &p, &l);
+  return (p * n0 + i) * 2 + l;
 }
 
 constexpr int kBsumStride = 1024;   // doubles per slot in bsum: partial sums, then mean(b)
@@ -157,13 +175,12 @@ bool fused2d_supported(const Geo& g);
 long long fused2d_partials(const Geo& g, int G);
 void launch_fused2d(const Geo& g, int G, const MxFields& f, const MxFields& fn, double* socp_part,
                     cudaStream_t s, LaunchCounter lc);
-// Fused lines 3-6 for D = 3 (k_fused3d.cu) for every active slot: z and q_0, alpha_0
-// by one pass over the cones, then q_d, alpha_d, beta by a time-marching pass over
-// tiles of cells; reads q, alpha, beta of f, writes those of fn; f.z is scratch.
-// residual: also write the next iteration's lines 1-2 residual into f.r.
+// Fused lines 3-6 for D = 3 (k_fused3d.cu) for one solve: z and q_0, alpha_0 by one pass
+// over the cones, then q_d, alpha_d, beta and the next iteration's lines 1-2 residual (f.r)
+// by a pass over tiles of cells at each time node; reads q, alpha, beta of f, writes those
+// of fn; f.z is scratch.
 bool fused3d_supported(const Geo& g);
-void launch_fused3d(const Geo& g, int G, const MxFields& f, const MxFields& fn, bool residual, cudaStream_t s,
-                    LaunchCounter lc);
+void launch_fused3d(const Geo& g, const MxFields& f, const MxFields& fn, cudaStream_t s, LaunchCounter lc);
 // KKT partial-sum scratch (doubles) per slot.
 long long kkt_partials_len_mx(const Geo& g);
 

@@ -117,44 +117,6 @@ __device__ __forceinline__ bool ff_le(float2 a, float2 b) {
 
 __device__ __forceinline__ float ff_round(float2 a) { return a.x + a.y; }
 
-// Projection onto the second-order cone {y_0 >= |ybar|} (eq. (app-proj)) of a
-// two-float input.  The input of the ALM projection is dominated by -beta/sigma,
-// often 10^2 - 10^3 times the O(1) point it projects to, so the tests and the
-// boundary value (y_0 + |ybar|)/2 cancel: |ybar| and that sum are formed in
-// two-float arithmetic (~2^-44 relative).  The boundary direction ybar/|ybar| only
-// scales the O(1) result, so it is taken in FP32: every output component is then
-// within a few FP32 ulps of its own (O(1)) value, the precision it is stored in.
-// Case order: y if |ybar| <= y_0; 0 if |ybar| <= -y_0; else the boundary formula.
-template <int K>
-__device__ __forceinline__ void ff_proj_soc(float2* y) {
-  // |ybar|^2: exact squares of the high parts summed with TwoSum, the rounding
-  // errors and the cross terms 2 hi lo collected in one FP32 correction (all
-  // terms are non-negative, so the compensated sum is accurate to ~2^-44)
-  float sh = 0.f, sc = 0.f;
-#pragma unroll
-  for (int j = 1; j < K; ++j) {
-    const float h = y[j].x;
-    const float p = h * h;
-    const float e = fmaf(2.f * h, y[j].y, fmaf(h, h, -p));
-    const float2 t = two_sum(sh, p);
-    sh = t.x;
-    sc += t.y + e;
-  }
-  const float2 nb = ff_sqrt(quick_two_sum(sh, sc));
-  if (ff_le(nb, y[0])) return;
-  if (ff_le(nb, ff_neg(y[0]))) {
-#pragma unroll
-    for (int j = 0; j < K; ++j) y[j] = make_float2(0.f, 0.f);
-    return;
-  }
-  const float2 sum = ff_add(y[0], nb);
-  const float2 a = make_float2(0.5f * sum.x, 0.5f * sum.y);
-  const float scale = (a.x + a.y) / nb.x;
-  y[0] = a;
-#pragma unroll
-  for (int j = 1; j < K; ++j) y[j] = make_float2(scale * y[j].x, 0.f);
-}
-
 // ---- packed pairs ---------------------------------------------------------
 // sm_100-class GPUs execute add/sub/mul/fma on two FP32 lanes in one instruction
 // (.f32x2), each lane an ordinary IEEE round-to-nearest operation.  A float2 here
@@ -337,18 +299,23 @@ __device__ __forceinline__ void acc2_add_mul(ff2_acc& s, ff2_acc b, float2 x) {
   s.c = add2(s.c, add2(t.l, fma2(b.c, x, p.l)));
 }
 
-// Projection onto {y_0 >= |ybar|} (eq. (app-proj)) of a K = 10 cone held as five
-// lane pairs: P[0] = (y_0, y_9), P[1..4] = y_1 .. y_8 paired in any order.  The same
-// method as ff_proj_soc (two-float |ybar|, FP32 boundary direction), with |ybar|^2
-// summed in two lanes, the square root from rsqrt and the boundary scale from its
-// reciprocal instead of divisions.
-// The three cases are one scale each for the high and low parts, without branches:
-// zr = the result rounded to FP32, pairs as P; *z0 and the returned z_9 are those two
-// components as two-floats.
-__device__ __forceinline__ float2 ff2_project10(const ff2* P, float2* zr, float2* z0) {
+// Projection onto {y_0 >= |ybar|} (eq. (app-proj)) of a cone of K = 2 NP components held
+// as lane pairs: P[0] = (y_0, y_{K-1}), P[1 .. NP - 1] = the others paired in any order.
+// The input of the ALM projection is dominated by -beta/sigma, often 10^2 - 10^3 times
+// the O(1) point it projects to, so the tests and the boundary value (y_0 + |ybar|)/2
+// cancel: |ybar| and that sum are formed in two-float arithmetic (~2^-44 relative).  The
+// boundary direction ybar/|ybar| only scales the O(1) result, so it is taken in FP32:
+// every output component is then within a few FP32 ulps of its own (O(1)) value, the
+// precision it is stored in.  Case order: y if |ybar| <= y_0; 0 if |ybar| <= -y_0; else
+// the boundary formula.  |ybar|^2 is summed in two lanes, the square root comes from
+// rsqrt and the boundary scale from its reciprocal, without divisions.  The three cases are one scale each for the high
+// and low parts, without branches: zr = the result rounded to FP32, pairs as P; *z0 and
+// the returned z_{K-1} are those two components as two-floats.
+template <int NP>
+__device__ __forceinline__ float2 ff2_project(const ff2* P, float2* zr, float2* z0) {
   float2 sh = make_float2(0.f, 0.f), sc = make_float2(0.f, 0.f);
 #pragma unroll
-  for (int k = 1; k <= 4; ++k) {
+  for (int k = 1; k < NP; ++k) {
     const float2 h = P[k].h;
     const float2 p = mul2(h, h);
     const float2 e0 = make_float2(fmaf(h.x, h.x, -p.x), fmaf(h.y, h.y, -p.y));
@@ -362,7 +329,7 @@ __device__ __forceinline__ float2 ff2_project10(const ff2* P, float2* zr, float2
       sc = add2(sc, add2(t.l, e));
     }
   }
-  // y_9 and the two lanes
+  // y_{K-1} and the two lanes
   const float h9 = P[0].h.y;
   const float p9 = h9 * h9;
   const float e9 = fmaf(2.f * h9, P[0].l.y, fmaf(h9, h9, -p9));
@@ -381,7 +348,7 @@ __device__ __forceinline__ float2 ff2_project10(const ff2* P, float2* zr, float2
   *z0 = inside ? y0 : below ? make_float2(0.f, 0.f) : a;
   const float2 m2 = make_float2(m, m), s2 = make_float2(scale, scale);
 #pragma unroll
-  for (int k = 1; k <= 4; ++k) zr[k] = fma2(m2, P[k].l, mul2(s2, P[k].h));
+  for (int k = 1; k < NP; ++k) zr[k] = fma2(m2, P[k].l, mul2(s2, P[k].h));
   const float2 z9 = make_float2(scale * h9, m * P[0].l.y);
   zr[0] = make_float2(z0->x + z0->y, z9.x + z9.y);
   return z9;

@@ -246,7 +246,7 @@ __device__ __forceinline__ void segment(const Geo& g, const FusedArgs& a, unsign
         if (yh) qd.y = a.q[2][i + 2 * P];
       }
       float2 z0;
-      const float2 z9 = ff2_project10(z, zc, &z0);
+      const float2 z9 = ff2_project<5>(z, zc, &z0);
       sz1[tid] = zc[1];
       sz3[lev + tid] = zc[3];
       // q_0 (diagonal 3): rhs = A_0 phi + alpha_0/sigma + u_9 - u_0 with u = z + beta/sigma;

@@ -237,15 +237,11 @@ __global__ void k_rescale(Geo g, MxFields fb) {
 #pragma unroll
   for (int d = 0; d < D; ++d)
     for (long long i = i0; i < nn; i += stride) f.al[1 + d][i] = ff_mul(f.al[1 + d][i], sp.rescale);
-  if (D == 2) {
-    float4* b = reinterpret_cast<float4*>(f.beta);
-    for (long long i = i0; i < (long long)(g.K / 2) * n0; i += stride) {
-      const float4 v = b[i];
-      const float2 p = ff_mul(make_float2(v.x, v.z), sp.rescale), q = ff_mul(make_float2(v.y, v.w), sp.rescale);
-      b[i] = make_float4(p.x, q.x, p.y, q.y);
-    }
-  } else {
-    for (long long i = i0; i < (long long)g.K * n0; i += stride) f.beta[i] = ff_mul(f.beta[i], sp.rescale);
+  float4* b = reinterpret_cast<float4*>(f.beta);
+  for (long long i = i0; i < (long long)(g.K / 2) * n0; i += stride) {
+    const float4 v = b[i];
+    const float2 p = ff_mul(make_float2(v.x, v.z), sp.rescale), q = ff_mul(make_float2(v.y, v.w), sp.rescale);
+    b[i] = make_float4(p.x, q.x, p.y, q.y);
   }
 }
 
@@ -274,19 +270,19 @@ __global__ void k_combine(Geo g, MxFields fb, float2* __restrict__ out) {
     phi[i] = two_sum(phi1[i], delta[i]);
 }
 
-// beta / sigma of component j at cone i, and its high part alone.
+// beta / sigma of component j at cone i, its high part alone, and z.
 template <int D>
 __device__ __forceinline__ float2 beta_ff(const float2* beta, int j, int i, int n0) {
-  if (D == 2) {
-    const float* p = reinterpret_cast<const float*>(beta) + beta2_at(j, i, n0);
-    return make_float2(p[0], p[2]);
-  }
-  return beta[j * n0 + i];
+  const float* p = reinterpret_cast<const float*>(beta) + beta_at(4 * D + 2, j, i, n0);
+  return make_float2(p[0], p[2]);
 }
 template <int D>
 __device__ __forceinline__ float beta_hi(const float2* beta, int j, int i, int n0) {
-  if (D == 2) return reinterpret_cast<const float*>(beta)[beta2_at(j, i, n0)];
-  return beta[j * n0 + i].x;
+  return reinterpret_cast<const float*>(beta)[beta_at(4 * D + 2, j, i, n0)];
+}
+template <int D>
+__device__ __forceinline__ float z_of(const float* z, int j, int i, int n0) {
+  return z[z_at(4 * D + 2, j, i, n0)];
 }
 
 template <int D>
@@ -308,8 +304,8 @@ __device__ __forceinline__ void gather_Fq(const Geo& g, float* const* q, int i, 
 
 // ---- stopping measures: FP32 terms, per-thread FP32 sums, FP64 tree -----------
 //
-// Kinds of blocks run side by side -- cones, faces (D = 2: both axes of a node, which
-// share beta's pairs; D = 3: a kind per axis) and nodes -- each over its own sums.  A
+// Kinds of blocks run side by side -- cones, faces along x and y (which share beta's
+// pairs), for D = 3 faces along z, and nodes -- each over its own sums.  A
 // 32-lane FP64 instruction occupies an SM for 16 cycles, so nothing per element is FP64
 // but the two planes that carry c, a block adds up only the sums of its kind, and a
 // warp's tree halves the number of sums a lane carries at every exchange (16 additions
@@ -319,7 +315,7 @@ __device__ __forceinline__ void gather_Fq(const Geo& g, float* const* q, int i, 
 // CTAs per SM for D = 2 (three 241 us, five 237), three for D = 3 (four 643 us, five 618).
 
 constexpr int kKktBlocks = 152 * 3;   // most blocks per slot and kind
-__host__ __device__ constexpr int kkt_kinds(int D) { return D == 2 ? 3 : 5; }
+__host__ __device__ constexpr int kkt_kinds(int D) { return D == 2 ? 3 : 4; }
 
 // Partial sums of a slot: [R_NSLOTS][kinds * blocks].
 __host__ __device__ inline long long kkt_partials_len_slot(const Geo& g) {
@@ -404,14 +400,14 @@ __device__ __forceinline__ void kkt_cone(const Geo& g, const MxFields& f, float 
   acc[R_F] += fv * fv;
   const float s = f.somega ? f.somega[p] : s_default;
   if (use_z) {
-    float r = (f.z[i] - 1.f) + q0;
+    float r = (z_of<D>(f.z, 0, i, n0) - 1.f) + q0;
     acc[R_SOCP] += r * r;
 #pragma unroll
     for (int j = 1; j < K - 1; ++j) {
-      r = fmaf(-s, x[j], f.z[j * n0 + i]);
+      r = fmaf(-s, x[j], z_of<D>(f.z, j, i, n0));
       acc[R_SOCP] += r * r;
     }
-    r = (f.z[(K - 1) * n0 + i] - 1.f) - q0;
+    r = (z_of<D>(f.z, K - 1, i, n0) - 1.f) - q0;
     acc[R_SOCP] += r * r;
   }
   const float2 bK = beta_ff<D>(f.beta, K - 1, i, n0), b0 = beta_ff<D>(f.beta, 0, i, n0);
@@ -463,17 +459,20 @@ __device__ __forceinline__ void kkt_face(const Geo& g, const MxFields& f, float 
   acc[R_FBB] += fbb * fbb;
 }
 
-// The faces of axis AX of every node; D = 2: of both axes of a node together (they share
-// beta's pairs).
-template <int D, int AX>
+// The faces above every node along axes x and y (they share beta's pairs), or along z.
+template <int D, bool XY>
 __device__ __forceinline__ void kkt_face_loop(const Geo& g, const MxFields& f, float sg, int i0, int stride, float* acc,
                                               float2* dual) {
   const int P = (int)g.P, n = (g.T + 1) * P;
 #pragma unroll 1
   for (int i = i0; i < n; i += stride) {
     const int t = plane_of(g, i), p = i - t * P;
-    if (coord(g, p, AX) <= g.N[AX] - 2) kkt_face<D>(g, f, sg, AX, i, t, p, acc, dual);
-    if (D == 2 && coord(g, p, 1) <= g.N[1] - 2) kkt_face<D>(g, f, sg, 1, i, t, p, acc, dual);
+    if (XY) {
+      if (coord(g, p, 0) <= g.N[0] - 2) kkt_face<D>(g, f, sg, 0, i, t, p, acc, dual);
+      if (coord(g, p, 1) <= g.N[1] - 2) kkt_face<D>(g, f, sg, 1, i, t, p, acc, dual);
+    } else if (coord(g, p, D - 1) <= g.N[D - 1] - 2) {
+      kkt_face<D>(g, f, sg, D - 1, i, t, p, acc, dual);
+    }
   }
 }
 
@@ -526,9 +525,8 @@ __global__ void __launch_bounds__(kThreads, D == 2 ? 4 : 3) k_kkt(const __grid_c
     block_reduce_store(v, w, partials, rows, row);
   } else if (kind < kkt_kinds(D) - 1) {
     float2 dual = make_float2(0.f, 0.f);
-    if (kind == 1) kkt_face_loop<D, 0>(g, f, sg, i0, stride, acc, &dual);
-    else if (kind == 2) kkt_face_loop<D, 1>(g, f, sg, i0, stride, acc, &dual);
-    else kkt_face_loop<D, D - 1>(g, f, sg, i0, stride, acc, &dual);
+    if (kind == 1) kkt_face_loop<D, true>(g, f, sg, i0, stride, acc, &dual);
+    else kkt_face_loop<D, false>(g, f, sg, i0, stride, acc, &dual);
     constexpr int w[9] = {R_PRIM, R_APHI, R_Q, R_COMPD, R_ALPHAB, R_G, R_SOCD, R_FBB, R_DUALOBJ};
     double v[9];
 #pragma unroll

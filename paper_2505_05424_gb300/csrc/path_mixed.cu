@@ -407,7 +407,7 @@ void MixedBatch::iterate(cudaStream_t s, LaunchCounter lc) {
     if (r_valid_) launch_solve_residual_mx(g_, G_, fc, ps_, s, lc);
     else launch_assemble_solve_mx(g_, G_, fc, ps_, s, lc);
     // lines 3-6, and the next iteration's residual in f.r
-    launch_fused3d(g_, G_, fc, fn, true, s, lc);
+    launch_fused3d(g_, fc, fn, s, lc);
     r_valid_ = true;
     cur_ ^= 1;
   }
@@ -473,13 +473,9 @@ int MixedBatch::read_state(int b, double* q, double* al, double* beta, cudaStrea
     off += (size_t)natural_face_count(g_, fam);
   }
   for (int j = 0; beta && j < g_.K; ++j) {
-    if (g_.D == 2) {
-      const long long o = beta2_at(j, 0, (long long)n0);
-      parts.push_back({reinterpret_cast<const float*>(fc.beta) + o / 4 * 4, beta + j * n0, n0, n0, 1,
-                       o % 4 ? HOST_LANE1 : HOST_LANE0, sig, 1.0});
-    } else {
-      parts.push_back({fc.beta + j * n0, beta + j * n0, n0, n0, 1, HOST_FF, sig, 1.0});
-    }
+    const long long o = beta_at(g_.K, j, 0, (long long)n0);
+    parts.push_back({reinterpret_cast<const float*>(fc.beta) + o / 4 * 4, beta + j * n0, n0, n0, 1,
+                     o % 4 ? HOST_LANE1 : HOST_LANE0, sig, 1.0});
   }
   const cudaError_t e = read_to_host(parts, s);
   if (e != cudaSuccess) { *err = std::string("read_state: ") + cudaGetErrorString(e); return DOT_ECUDA; }
@@ -511,18 +507,14 @@ int MixedBatch::write_state(int b, const double* q, const double* al, const doub
   }
   const size_t nb = (size_t)g_.K * n0;
   std::vector<float2> tb(nb);
-  if (g_.D == 2) {
-    float* p = reinterpret_cast<float*>(tb.data());
-    for (int j = 0; j < g_.K; ++j)
-      for (size_t i = 0; i < n0; ++i) {
-        const float2 v = split_ff(beta[j * n0 + i] * is);
-        const long long o = beta2_at(j, (long long)i, (long long)n0);
-        p[o] = v.x;
-        p[o + 2] = v.y;
-      }
-  } else {
-    for (size_t i = 0; i < nb; ++i) tb[i] = split_ff(beta[i] * is);
-  }
+  float* pb = reinterpret_cast<float*>(tb.data());
+  for (int j = 0; j < g_.K; ++j)
+    for (size_t i = 0; i < n0; ++i) {
+      const float2 v = split_ff(beta[j * n0 + i] * is);
+      const long long o = beta_at(g_.K, j, (long long)i, (long long)n0);
+      pb[o] = v.x;
+      pb[o + 2] = v.y;
+    }
   if (e == cudaSuccess) e = up(fc.beta, tb.data(), nb * 8, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) { *err = std::string("write_state: ") + cudaGetErrorString(e); return DOT_ECUDA; }
