@@ -178,16 +178,15 @@ const char *dot_kernel_name(int id);
  * counterpart in the paper; it serves plugins of hosts that forbid allocation on
  * their worker threads, processes whose device memory is reserved by another
  * allocator, and loops with a fixed memory budget that must not risk an
- * allocation failing part way through).  It computes what dot_poisson computes for a DOT_MIXED
- * context -- phi = (A^*A)^dagger b by FP32/3xTF32 DCT solves with one refinement
- * step -- on caller-owned device buffers, and allocates nothing: all scratch
- * lives in one fixed __device__ array of the library (about 31 MB, held by every
- * GPU that loads the library until the process exits).
+ * allocation failing part way through).  It computes what dot_poisson computes for
+ * a DOT_MIXED context -- phi = (A^*A)^dagger b by FP32 solves with one refinement
+ * step -- on caller-owned device buffers, and allocates nothing: all scratch lives
+ * in one fixed __device__ array of the library (about 25 MB, held by every GPU that
+ * loads the library until the process exits).
  *   b    : device, FP32, [T+1][N_1]...[N_D]           (read only)
  *   phi  : device, 2 floats per node (hi, lo) in the same order; phi = hi + lo
  *   stream: cudaStream_t or NULL; the call synchronises it before returning.
- * Limits: D in {2, 3}, T+1 in [2, 160] (the time axis runs the SIMT time pass,
- * built for at most 160 time nodes, as in DOT_MIXED contexts), every N_d in
+ * Limits: D in {2, 3}, T+1 in [2, 160] (as DOT_MIXED contexts), every N_d in
  * [2, 256], (T+1) N_1...N_D <= 2^20 nodes; larger grids return DOT_EINVAL with a message from
  * dot_noalloc_last_error().  The first call on a device fetches the array's
  * device address and should come before any stream capture.  Every call shares

@@ -20,6 +20,7 @@ template <> struct Vec2<double> { using type = double2; };
 // factors and the inverse input factors (cos, sin)(pi k / 2N) with the orthonormal
 // scaling folded in.
 std::vector<double> fft_tables_host(int N);
+void fft_tables_fill(int N, float* out);   // the same into 6 N floats
 inline size_t fft_table_pairs(int N) { return (size_t)3 * N; }
 
 template <class R>

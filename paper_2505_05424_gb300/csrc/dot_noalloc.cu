@@ -7,10 +7,14 @@
 // budget that must not risk an allocation failing part way through a run.
 // dot_poisson_f32_noalloc serves
 // them: the caller passes the right-hand side and the output buffer, and every
-// scratch buffer the solve needs (four node-sized FP32 fields, the FP64 partial
-// sums of the zero mode, the DCT tables and the pipeline error flag) lives in one
-// file-scope __device__ array of fixed size, which every GPU that loads this
-// library holds until the process exits.
+// scratch buffer the solve needs (six node-sized FP32 fields, the FP64 partial sums of
+// the zero mode, the transform tables) lives in one file-scope __device__ array of
+// fixed size, which every GPU that loads this library holds until the process exits.
+//
+// Both solves of the refinement run the fast transforms (k_fft.cu), whose tables are
+// O(N) per axis and go up in one copy with the eigenvalues: dense tables (O(N^2)
+// cosines on the host and sixteen copies per call) took 0.25 ms of a call on
+// 64 x 48 x 16 and 2.1 ms on 256^2 x 15.
 //
 // The array is shared by every call: a call overwrites what the previous one
 // left there, and two calls whose work overlaps on the GPU (different streams, or
@@ -32,26 +36,26 @@ namespace {
 
 constexpr long long kMaxNodes = 1LL << 20;  // (T+1) * N_1 * ... * N_D
 constexpr int kMaxAxis = 256;               // largest node count along one spatial axis
-// Here the time axis runs the SIMT time pass of the mixed path (no padded time
-// tables), which is built for at most 160 time nodes, as DOT_MIXED contexts are.
-constexpr int kMaxTimeNodes = 160;
+constexpr int kMaxTimeNodes = 160;          // as DOT_MIXED contexts
+
+// What a call uploads: per axis the transform tables and the eigenvalues, one active slot.
+struct Upload {
+  float tab[kMaxD][6 * kMaxAxis];
+  float lam[kMaxD][kMaxAxis];
+  SlotParam sp;
+};
 
 // Layout of the scratch array (256-byte aligned pieces, sizes in bytes).
 constexpr size_t kField = (size_t)kMaxNodes * sizeof(float);
-constexpr size_t kTable = (size_t)kMaxAxis * kMaxAxis * sizeof(float);
-constexpr size_t kLam = (size_t)kMaxAxis * sizeof(float);
 constexpr size_t kOffB = 0;
 constexpr size_t kOffBlo = kOffB + kField;
 constexpr size_t kOffPhi1 = kOffBlo + kField;
 constexpr size_t kOffR = kOffPhi1 + kField;
 constexpr size_t kOffW1 = kOffR + kField;
 constexpr size_t kOffW2 = kOffW1 + kField;
-constexpr size_t kOffTables = kOffW2 + kField;                           // (kMaxD+1) axes x 6 tables
-constexpr size_t kOffLam = kOffTables + (size_t)(kMaxD + 1) * 6 * kTable; // (kMaxD+1) axes
-constexpr size_t kOffSum = kOffLam + (size_t)(kMaxD + 1) * kLam;
-constexpr size_t kOffErr = kOffSum + kBsumStride * sizeof(double);  // partial sums of b, then mean(b)
-constexpr size_t kOffParam = kOffErr + 256;                            // one SlotParam (active)
-constexpr size_t kScratchBytes = kOffParam + 256;
+constexpr size_t kOffUp = kOffW2 + kField;
+constexpr size_t kOffSum = kOffUp + (sizeof(Upload) + 255) / 256 * 256;   // partial sums of b, then mean(b)
+constexpr size_t kScratchBytes = kOffSum + kBsumStride * sizeof(double);
 
 static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 
@@ -60,9 +64,7 @@ static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 std::mutex g_mu;
 void* g_dev_ptr[64] = {nullptr};
 
-// Host staging of the DCT tables (static: this path allocates nothing).
-float g_host_tab[(kMaxD + 1) * 6][kMaxAxis * kMaxAxis];
-float g_host_lam[kMaxD + 1][kMaxAxis];
+Upload g_up;   // host staging (static: this path allocates nothing)
 
 // error text in a fixed buffer (formatting it allocates nothing)
 thread_local char g_err[256];
@@ -70,15 +72,6 @@ thread_local char g_err[256];
 int fail(int code, const char* m, const char* detail = "") {
   std::snprintf(g_err, sizeof(g_err), "%s%s", m, detail);
   return code;
-}
-
-float tf32_round(float x) {
-  uint32_t u;
-  std::memcpy(&u, &x, 4);
-  u = (u + 0x1000u) & 0xFFFFE000u;
-  float r;
-  std::memcpy(&r, &u, 4);
-  return r;
 }
 
 }  // namespace
@@ -129,65 +122,30 @@ extern "C" int dot_poisson_f32_noalloc(const dot_grid* grid, const float* b, flo
   f.bsum = (double*)(base + kOffSum);
   MxPoisson ps;
   std::memset(&ps, 0, sizeof(ps));
-  ps.w1 = (float*)(base + kOffW1);
-  ps.w2 = (float*)(base + kOffW2);
-  ps.err = (int*)(base + kOffErr);
-  ps.use_tc = true;
-  f.sp = (const SlotParam*)(base + kOffParam);
-
-  // DCT tables of this grid (orthonormal DCT-II, its transpose and their TF32 splits)
-  for (int a = 0; a <= g.D; ++a) {
-    const int M = a == 0 ? g.T + 1 : g.N[a - 1];
+  Upload* up = (Upload*)(base + kOffUp);
+  f.sp = &up->sp;
+  ps.fast.w1 = (float*)(base + kOffW1);
+  ps.fast.w2 = (float*)(base + kOffW2);
+  ps.use_fast = true;
+  for (int d = 0; d < g.D; ++d) {
+    const int M = g.N[d];
     const double pi = 3.14159265358979323846;
-    const double h = a == 0 ? 1.0 / g.T : 1.0 / g.N[a - 1];
-    float* t[6];
-    for (int j = 0; j < 6; ++j) t[j] = g_host_tab[a * 6 + j];
+    fft_tables_fill(M, g_up.tab[d]);
     for (int k = 0; k < M; ++k) {
-      const double sk = k == 0 ? std::sqrt(1.0 / M) : std::sqrt(2.0 / M);
-      for (int n = 0; n < M; ++n) {
-        const double c = sk * std::cos(pi * k * (n + 0.5) / M);
-        const float hi = tf32_round((float)c);
-        const float lo = (float)(c - (double)hi);
-        t[0][k * M + n] = (float)c;
-        t[1][n * M + k] = (float)c;
-        t[2][k * M + n] = hi;
-        t[3][k * M + n] = lo;
-        t[4][n * M + k] = hi;
-        t[5][n * M + k] = lo;
-      }
       const double sv = std::sin(pi * k / (2.0 * M));
-      g_host_lam[a][k] = (float)(4.0 / (h * h) * sv * sv);
+      g_up.lam[d][k] = (float)(4.0 * M * M * sv * sv);
     }
-    float* dst[6];
-    for (int j = 0; j < 6; ++j) {
-      dst[j] = (float*)(base + kOffTables + (size_t)(a * 6 + j) * kTable);
-      e = cudaMemcpyAsync(dst[j], t[j], (size_t)M * M * sizeof(float), cudaMemcpyHostToDevice, s);
-      if (e != cudaSuccess) return fail(DOT_ECUDA, "table upload: ", cudaGetErrorString(e));
-    }
-    float* ldst = (float*)(base + kOffLam + (size_t)a * kLam);
-    e = cudaMemcpyAsync(ldst, g_host_lam[a], (size_t)M * sizeof(float), cudaMemcpyHostToDevice, s);
-    if (e != cudaSuccess) return fail(DOT_ECUDA, "table upload: ", cudaGetErrorString(e));
-    ps.C[a] = dst[0];
-    ps.CT[a] = dst[1];
-    ps.Chi[a] = dst[2];
-    ps.Clo[a] = dst[3];
-    ps.CThi[a] = dst[4];
-    ps.CTlo[a] = dst[5];
-    ps.lam[a] = ldst;
+    ps.fast.tab[d] = (const float2*)up->tab[d];
+    ps.fast.lam[d] = up->lam[d];
   }
-  // the right-hand side is copied in (the solve overwrites it with the correction);
-  // its low part and the error flag must start at zero
-  SlotParam one;
-  std::memset(&one, 0, sizeof(one));
-  one.rescale = make_float2(1.f, 0.f);
-  one.active = 1;
-  static SlotParam kOne;
-  kOne = one;
-  e = cudaMemcpyAsync(f.b, b, (size_t)nn * sizeof(float), cudaMemcpyDeviceToDevice, s);
+  std::memset(&g_up.sp, 0, sizeof(g_up.sp));
+  g_up.sp.rescale = make_float2(1.f, 0.f);
+  g_up.sp.active = 1;
+  // the right-hand side is copied in (the solve overwrites it with the correction); its low
+  // part starts at zero
+  e = cudaMemcpyAsync(up, &g_up, sizeof(g_up), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(f.b, b, (size_t)nn * sizeof(float), cudaMemcpyDeviceToDevice, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(f.blo, 0, (size_t)nn * sizeof(float), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(ps.err, 0, sizeof(int), s);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(base + kOffParam, &kOne, sizeof(kOne), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return fail(DOT_ECUDA, "scratch set-up: ", cudaGetErrorString(e));
   long launches = 0;
   LaunchCounter lc{&launches};
@@ -195,10 +153,7 @@ extern "C" int dot_poisson_f32_noalloc(const dot_grid* grid, const float* b, flo
   launch_poisson_refined_mx(g, 1, f, ps, reinterpret_cast<float2*>(phi), false, s, lc);
   e = cudaGetLastError();
   if (e != cudaSuccess) return fail(DOT_ECUDA, "launch: ", cudaGetErrorString(e));
-  int flag = 0;
-  e = cudaMemcpyAsync(&flag, ps.err, sizeof(int), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return fail(DOT_ECUDA, "poisson: ", cudaGetErrorString(e));
-  if (flag) return fail(DOT_ECUDA, "a tensor-core pipeline wait timed out (kernel returned early)");
   return DOT_OK;
 }

@@ -43,22 +43,32 @@
 
 namespace dot {
 
-std::vector<double> fft_tables_host(int N) {
+namespace {
+
+template <class R>
+void fill_tables(int N, R* t) {
   const double pi = 3.14159265358979323846;
-  std::vector<double> t((size_t)6 * N);
   for (int j = 0; j < N; ++j) {
-    const double w = 2.0 * pi * j / N, h = pi * j / (2.0 * N);
+    const double w = 2.0 * pi * j / N, h = pi * j / (2.0 * N), ch = std::cos(h), sh = std::sin(h);
     const double fo = (j == 0 ? std::sqrt(1.0 / N) : std::sqrt(2.0 / N)) / 2.0;
     const double in = j == 0 ? std::sqrt(1.0 / N) : std::sqrt(1.0 / (2.0 * N));
-    t[2 * j] = std::cos(w);
-    t[2 * j + 1] = -std::sin(w);
-    t[2 * (N + j)] = fo * std::cos(h);
-    t[2 * (N + j) + 1] = fo * std::sin(h);
-    t[2 * (2 * N + j)] = in * std::cos(h);
-    t[2 * (2 * N + j) + 1] = in * std::sin(h);
+    t[2 * j] = (R)std::cos(w);
+    t[2 * j + 1] = (R)-std::sin(w);
+    t[2 * (N + j)] = (R)(fo * ch);
+    t[2 * (N + j) + 1] = (R)(fo * sh);
+    t[2 * (2 * N + j)] = (R)(in * ch);
+    t[2 * (2 * N + j) + 1] = (R)(in * sh);
   }
+}
+
+}  // namespace
+
+std::vector<double> fft_tables_host(int N) {
+  std::vector<double> t((size_t)6 * N);
+  fill_tables(N, t.data());
   return t;
 }
+void fft_tables_fill(int N, float* out) { fill_tables(N, out); }
 
 namespace {
 

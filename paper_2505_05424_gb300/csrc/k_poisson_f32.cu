@@ -13,7 +13,9 @@
 // time axis runs as two passes (DCT-II with the eigenvalue scaling in its
 // epilogue, then DCT-III), and a batch of G solves of one grid is transformed in
 // the same passes (the group index is carried outermost through every layout).
-// SIMT flow (one solve; axes the tensor-core pass cannot take): the spatial passes
+// Grids with an axis that the tensor-core pass cannot take run the fast transforms
+// (k_fft.cu), as the iterations do.
+// SIMT flow (one solve; axes beyond both, more than 5,632 points): the spatial passes
 // run on the kernel below, in FP32 with the same output layouts, and the time axis
 // is one fused pass per column of spatial frequencies: DCT-II, scale, DCT-III.
 #include <cstring>
@@ -387,6 +389,10 @@ bool poisson_tc(const Geo& g, int G, const MxPoisson& ps, const float* src, floa
 bool launch_poisson_mx(const Geo& g, int G, const MxPoisson& ps, const float* src, float* dst, cudaStream_t s,
                        LaunchCounter lc, float2* accum) {
   if (poisson_tc_flow(g, ps) && poisson_tc(g, G, ps, src, dst, s, lc, accum)) return accum != nullptr;
+  if (ps.use_fast) {
+    launch_fast_poisson(g, G, ps.fast, src, dst, nullptr, s, lc);
+    return false;
+  }
   // SIMT flow (one solve)
   const long long n = (long long)(g.T + 1) * g.P;
   float* w[2] = {ps.w1, ps.w2};
