@@ -13,8 +13,9 @@
 //   B. updates q_d, alpha_d of its two faces on time node t, as the two lanes of packed
 //      two-float arithmetic, from its own z and beta and its two neighbours', and
 //      publishes q and w = q - alpha/sigma - A phi of them;
-//   C. (owners) updates beta of the cone at t - 1, which reads q^{k+1} on the faces of
-//      nodes t - 1 and t (kept in registers from step to step), and writes the next
+//   C. (owners) updates the components of beta whose update reads q^{k+1} on the faces of
+//      node t -- 1, 2, 5, 6 of the cone at t and 3, 4, 7, 8 of the cone at t - 1, the ones
+//      those faces collected (0 and 9 follow q_0 in step A) -- and writes the next
 //      iteration's residual at node t from the faces' w.
 // A thread copies its column's beta one cone time ahead into its own shared-memory
 // slots (cp.async, any N_y), where step A, the faces below it and step C read it.  z
@@ -24,14 +25,16 @@
 // two-float face right-hand sides and multiplier updates (ffloat.cuh).
 //
 // Bound by instruction issue and by the latency of a time step (two barriers, a
-// dependent chain of some 100 FP operations): on 256^2 x 64 157 M warp instructions,
-// 49% issue, 0.58 of the HBM bandwidth on its 1,026 MB, 257 us per launch.  The form
-// before it (a thread per halo cone, faces dealt out in rounds, beta by TMA in
-// component planes, 80 registers at two CTAs per SM, fixed 16-time chunks): 245 M
-// instructions, 357 us; and for odd N_y, where it could not use TMA, 262 us on
-// 150 x 117 x 37 against 64 now.  Measured on the way: this mapping at two CTAs of 8
-// rows and 80 registers 429 us (spills), one CTA of 12 rows and 128 registers 293; equal
-// shares of work for every SM and beta in lane pairs 267.
+// dependent chain of some 100 FP operations): on 256^2 x 64 about 150 M warp
+// instructions, 49% issue, 0.6 of the HBM bandwidth on its 1,026 MB, 251 us per launch;
+// 128^2 x 32 47.5 us, 32^2 x 16 10.4 us.  The form before it (a thread per halo cone,
+// faces dealt out in rounds, beta by TMA in component planes, 80 registers at two CTAs per
+// SM, fixed 16-time chunks): 245 M instructions, 357, 62 and 19.6 us; and for odd N_y,
+// where it could not use TMA, 262 us on 150 x 117 x 37 against 60 now.  Measured on the
+// way: this mapping at two CTAs of 8 rows and 80 registers 429 us (spills), one CTA of 12
+// rows and 128 registers 293; equal shares of work for every SM and beta in lane pairs
+// 267; a segment owning whole cones, whose last update needs one projection and one face
+// step beyond it, 257 (128^2 x 32: 53.5).
 #include <cmath>
 
 #include "dot_internal.cuh"
@@ -77,7 +80,7 @@ struct FusedArgs {
   const float* somega;
   int G;               // slots
   int ntx, nty;        // tiles along x and y
-  int unit, nunit;     // cone times per work unit, units per tile
+  int unit, nunit;     // time nodes per work unit, units per tile
   const SlotParam* sp;
   double* socp_part;   // per work unit: sum of |z - B F q^{k+1} - d|^2
   // the next iteration's lines 1-2 residual
@@ -99,7 +102,7 @@ __device__ __forceinline__ float4 f4_of(ff2 b) { return make_float4(b.h.x, b.h.y
 
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
 
-// One segment: cone times [ta, tb) of one tile of one slot.  *pend: the work unit of
+// One segment: time nodes [ta, tb) of one tile of one slot.  *pend: the work unit of
 // the segment before whose sums wait in wsum (null: none).  Element indices stay below
 // 2^31 over all slots of a batch (dot_server.cu bounds the batch).
 template <int TX, bool MASKED>
@@ -153,7 +156,7 @@ __device__ __forceinline__ void segment(const Geo& g, const FusedArgs& a, unsign
   }
 
   const int tstart = ta > 0 ? ta - 1 : 0;
-  const int tlast = min(tb, T - 1);         // last cone time this segment projects
+  const int tlast = min(tb - 1, T - 1);     // last cone time this segment projects
   // element of the column on time plane t: of node fields; cone fields and beta's pair 0
   // at a fixed distance
   int i = slot * (n0 + P) + tstart * P + x * N1 + y;
@@ -201,25 +204,25 @@ __device__ __forceinline__ void segment(const Geo& g, const FusedArgs& a, unsign
       if (yh) qd.y = a.q[2][i + P];
     }
     ph_t = a.phi[i];
-    ph_n = a.phi[i + P];                    // tstart <= T - 1
-    if (owner) al0 = a.al[0][i + ocone];
+    if (tstart < T) ph_n = a.phi[i + P];
+    if (owner && tstart <= tlast) al0 = a.al[0][i + ocone];
     if (tstart >= ta) {
       if (fx) a1 = a.al[1][i];
       if (fy) a2 = a.al[2][i];
     }
   }
 
-  float2 zc[5], zp[5];                      // FP32 z of the cone at t and t - 1: (0, 9), (1, 5), ..., (4, 8)
+  float2 zc[5];                             // FP32 z of the cone at t: (0, 9), (1, 5), ..., (4, 8)
 #pragma unroll
-  for (int k = 0; k < 5; ++k) zc[k] = zp[k] = z2;
-  float q0c = 0.f, q0p = 0.f;
+  for (int k = 0; k < 5; ++k) zc[k] = z2;
+  float2 zp3 = z2, zp4 = z2;                // (3, 7) and (4, 8) of the cone at t - 1
   float2 w0c = z2, w0p = z2;                // alpha_0/sigma + A_0 phi - q_0 of cones t and t - 1 (unnormalised)
-  float2 qlp = z2, qop = z2;                // q^{k+1} of the faces below and of the own faces on node t - 1
   float2 socp = z2;
-  int left = a.unit;                        // cone times to the end of the work unit
+  const float2 ts2 = f2(ts, ts);
+  int left = a.unit;                        // time nodes to the end of the work unit
   double* entry = socp_tile + ta / a.unit;
 
-  for (int t = tstart; t <= tb; ++t, i += P) {
+  for (int t = tstart; t < tb; ++t, i += P) {
     const int lev = (t & 1) * kThreads;
     if (t + 1 <= tlast) fetch(st_n, i + obeta + P);
     asm volatile("cp.async.commit_group;" ::: "memory");
@@ -251,7 +254,7 @@ __device__ __forceinline__ void segment(const Geo& g, const FusedArgs& a, unsign
       sz3[lev + tid] = zc[3];
       // q_0 (diagonal 3): rhs = A_0 phi + alpha_0/sigma + u_9 - u_0 with u = z + beta/sigma;
       // the cone before the segment (t = ta - 1) is updated for the residual only
-      if (owner && t < tb) {
+      if (owner) {
         const float2 gp = ff_grad(ph_t, ph_n, ih0);
         const ff2 u = ff2_add(ff2_pack(z0, z9), ff2_of(bt[0]));
         ff_acc acc = acc_init(gp);
@@ -264,11 +267,13 @@ __device__ __forceinline__ void segment(const Geo& g, const FusedArgs& a, unsign
         if (t >= ta) {
           a.qn[0][i + ocone] = qn;
           a.aln[0][i + ocone] = aln;
+          const float2 inc = add2(sub2(zc[0], f2(1.f, 1.f)), f2(qn, -qn));
+          socp = fma2(inc, inc, socp);
+          a.betan[i + obeta] = f4_of(ff2_add_f(ff2_of(bt[0]), mul2(ts2, inc)));
         }
-        q0c = qn;
         const float2 e = two_sum(aln.x, gm);
         w0c = f2(e.x, e.y + aln.y);
-        if (t + 1 < tb) al0 = a.al[0][i + ocone + P];
+        if (t + 1 <= tlast) al0 = a.al[0][i + ocone + P];
       }
     }
     sph[tid] = ph_t;
@@ -281,7 +286,6 @@ __device__ __forceinline__ void segment(const Geo& g, const FusedArgs& a, unsign
       }
       *pend = nullptr;
     }
-    const bool write_node = t >= ta && (t < tb || t == T);
     float2 qo = z2;
     ff2 wo{z2, z2};
     // ---------------- B: the column's faces on time node t ----------------
@@ -311,7 +315,7 @@ __device__ __forceinline__ void segment(const Geo& g, const FusedArgs& a, unsign
         acc2_add(ao, ff2_of(bslot[(st_p * (K2 / 2) + 4) * kThreads]));
         const int lp = kThreads - lev;
         zn = add2(zn, f2(sz3[lp + hx].x, sz3[lp + hy].y));
-        zo = add2(zo, zp[4]);
+        zo = add2(zo, zp4);
       }
       // (the same operations with and without a mask: a solve served among masked ones
       // takes the masked kernel, with every weight 1)
@@ -330,12 +334,12 @@ __device__ __forceinline__ void segment(const Geo& g, const FusedArgs& a, unsign
       const ff2 pr = two_prod2(q1, den);
       qo = fma2(add2(sub2(sub2(acc.h, pr.h), pr.l), acc.c), rd, q1);
       const float2 gm = add2(sub2(gh, qo), gl);
-      const ff2 aln = ff2_add_f(al, mul2(f2(ts, ts), gm));
+      const ff2 aln = ff2_add_f(al, mul2(ts2, gm));
       wo = two_sum2(aln.h, gm);             // alpha/sigma + A phi - q (unnormalised)
       wo.l = add2(wo.l, aln.l);
       if (!fx) { qo.x = 0.f; wo.h.x = 0.f; wo.l.x = 0.f; }
       if (!fy) { qo.y = 0.f; wo.h.y = 0.f; wo.l.y = 0.f; }
-      if (write_node && owner) {
+      if (owner) {
         if (fx) {
           a.qn[1][i] = qo.x;
           a.aln[1][i] = ff2_lane0(aln);
@@ -350,35 +354,34 @@ __device__ __forceinline__ void segment(const Geo& g, const FusedArgs& a, unsign
     sw[tid] = f4_of(wo);
     // the next time's potential and alpha / sigma of the faces
     ph_t = ph_n;
-    if (t < tb) {
+    if (t + 1 < tb) {
       if (cone_ok && t + 2 <= T) ph_n = a.phi[i + 2 * P];
       if (fx) a1 = a.al[1][i + P];
       if (fy) a2 = a.al[2][i + P];
     }
     __syncthreads();
-    if (own_ok) {
-      const float2 ql = f2(sq[lx].x, sq[ly].y);   // faces below, node t
-      // ---------------- C: beta of the cone at t - 1 ----------------
-      if (t > ta) {
-        const float4* bt = bslot + st_p * (K2 / 2) * kThreads;
-        float4* bn = a.betan + (i + obeta - P);
-        const float2 ns2 = f2(-s, -s), ts2 = f2(ts, ts);
-        float2 inc[5];
-        inc[0] = add2(sub2(zp[0], f2(1.f, 1.f)), f2(q0p, -q0p));
-        inc[1] = fma2(ns2, qlp, zp[1]);
-        inc[2] = fma2(ns2, qop, zp[2]);
-        inc[3] = fma2(ns2, ql, zp[3]);
-        inc[4] = fma2(ns2, qo, zp[4]);
-#pragma unroll
-        for (int k = 0; k < 5; ++k) {
-          socp = fma2(inc[k], inc[k], socp);
-          bn[(long long)k * n0] = f4_of(ff2_add_f(ff2_of(bt[k * kThreads]), mul2(ts2, inc[k])));
-        }
+    if (own_ok && t >= ta) {
+      // ---------------- C: beta and the residual at node t ----------------
+      const float2 ql = f2(sq[lx].x, sq[ly].y);   // faces below
+      const float2 ns2 = f2(-s, -s);
+      auto upd = [&](const float4* bt, float4* bn, int k, float2 q, float2 z) {
+        const float2 inc = fma2(ns2, q, z);
+        socp = fma2(inc, inc, socp);
+        bn[(long long)k * n0] = f4_of(ff2_add_f(ff2_of(bt[k * kThreads]), mul2(ts2, inc)));
+      };
+      if (t < T) {
+        const float4* bt = bslot + st_c * (K2 / 2) * kThreads;
+        upd(bt, a.betan + (i + obeta), 1, ql, zc[1]);
+        upd(bt, a.betan + (i + obeta), 2, qo, zc[2]);
       }
-      qlp = ql;
+      if (t >= 1) {
+        const float4* bt = bslot + st_p * (K2 / 2) * kThreads;
+        upd(bt, a.betan + (i + obeta - P), 3, ql, zp3);
+        upd(bt, a.betan + (i + obeta - P), 4, qo, zp4);
+      }
       // the next iteration's residual at node t: A^* w - c/sigma with w = q - alpha/sigma -
       // A phi of the node's faces (sw and w0 hold -w, zero at the walls)
-      if (write_node) {
+      {
         const float* wx = reinterpret_cast<const float*>(sw + lx);
         const float* wy = reinterpret_cast<const float*>(sw + ly) + 1;
         const ff2 dw = two_diff2(wo.h, f2(wx[0], wy[0]));
@@ -400,8 +403,8 @@ __device__ __forceinline__ void segment(const Geo& g, const FusedArgs& a, unsign
         a.r[i] = acc.h + acc.c;
       }
     }
-    // the sum of squared beta increments of a work unit that ends with cone t - 1
-    if (t > ta && (--left == 0 || t == T)) {
+    // the sum of squared beta increments of a work unit that ends with node t
+    if (t >= ta && (--left == 0 || t == T)) {
       if (owner) {
         double v = (double)socp.x + (double)socp.y;
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -411,11 +414,9 @@ __device__ __forceinline__ void segment(const Geo& g, const FusedArgs& a, unsign
       *pend = entry++;
       left = a.unit;
     }
-    qop = qo;
-    q0p = q0c;
     w0p = w0c;
-#pragma unroll
-    for (int k = 0; k < 5; ++k) zp[k] = zc[k];
+    zp3 = zc[3];
+    zp4 = zc[4];
     const int s0 = st_p;
     st_p = st_c;
     st_c = st_n;
@@ -427,11 +428,10 @@ __device__ __forceinline__ void segment(const Geo& g, const FusedArgs& a, unsign
   }
 }
 
-// Work units -- a slot's tile and a run of `unit` cone times -- in the order (active
+// Work units -- a slot's tile and a run of `unit` time nodes -- in the order (active
 // slot, tile, time), cut into one contiguous run per CTA: every SM gets the same
-// number of cone times whatever the grid, and a CTA crosses from one tile to the next
-// at most once more than its share needs.  Each segment projects two cone times more
-// than it owns.
+// number of nodes whatever the grid, and a CTA crosses from one tile to the next at most
+// once more than its share needs.  Each segment projects one cone time more than it owns.
 template <int TX, bool MASKED>
 __global__ void __launch_bounds__(Tile<TX>::kThreads, 1) k_fused2d(const __grid_constant__ Geo g,
                                                                   const __grid_constant__ FusedArgs a) {
@@ -462,7 +462,7 @@ __global__ void __launch_bounds__(Tile<TX>::kThreads, 1) k_fused2d(const __grid_
     const int s = tl / ntile, tile = tl - s * ntile;
     const int ty = tile / a.ntx, tx = tile - ty * a.ntx;
     const int slot = act[s];
-    segment<TX, MASKED>(g, a, sm, wsum, slot, tx * TX, ty * TY, u0 * a.unit, min(g.T, u1 * a.unit),
+    segment<TX, MASKED>(g, a, sm, wsum, slot, tx * TX, ty * TY, u0 * a.unit, min(g.T + 1, u1 * a.unit),
                         a.socp_part + ((long long)slot * ntile + tile) * nunit, &pend);
     k += u1 - u0;
   }
@@ -478,26 +478,26 @@ int ntiles(const Geo& g, int tx) { return ((g.N[0] + tx - 1) / tx) * ((g.N[1] + 
 
 // Tile rows.  13 is the most (16 warps at 128 registers fill an SM) and has the
 // smallest halo; smaller tiles give small grids more CTAs and shorter time steps.
-// A CTA's pass takes its share of the cone times plus the two around each segment, at
-// a time per step that grows with the rows, so the choice is the least of that product
-// (with 1 + 0.2 rows for the step, the fit of: 32^2 x 16 11.7 us with 4 rows, 13.7 with
-// 8, 16.2 with 13; 64^2 x 32 25.1, 23.0, 24.8; 96^2 x 16 27.3, 24.8, 25.0; 128^2 x 32
-// 64.7, 53.9, 53.7; 150 x 117 x 37 78.3, 66.0, 63.6).
+// A CTA's pass takes its share of the time nodes plus the cone time before each segment,
+// at a time per step that grows with the rows, so the choice is the least of that product
+// (with 1 + 0.2 rows for the step, the fit of: 32^2 x 16 10.3 us with 4 rows, 11.8 with
+// 8, 13.3 with 13; 64^2 x 32 22.5, 20.3, 22.6; 96^2 x 16 24.7, 22.0, 22.8; 128^2 x 32
+// 64.0, 47.6, 47.4; 150 x 117 x 37 77.6, 59.4, 59.9).
 int rows_of(const Geo& g, int G) {
   const int rows[3] = {13, 8, 4};
   int best = 13;
   double t = 1e300;
   for (int r : rows) {
-    const long long w = (long long)G * ntiles(g, r) * g.T;
-    const double e = (double)((w + kSMs - 1) / kSMs + 2) * (1.0 + 0.2 * r);
+    const long long w = (long long)G * ntiles(g, r) * (g.T + 1);
+    const double e = (double)((w + kSMs - 1) / kSMs + 1) * (1.0 + 0.2 * r);
     if (e < t) { t = e; best = r; }
   }
   return best;
 }
 
-// Cone times per work unit: about sixteen units per SM, at most eight.
+// Time nodes per work unit: about sixteen units per SM, at most eight.
 int unit_of(const Geo& g, int G) {
-  const long long u = (long long)G * ntiles(g, rows_of(g, G)) * g.T / (kSMs * 16);
+  const long long u = (long long)G * ntiles(g, rows_of(g, G)) * (g.T + 1) / (kSMs * 16);
   return (int)(u < 1 ? 1 : u > 8 ? 8 : u);
 }
 
@@ -514,7 +514,7 @@ bool fused2d_supported(const Geo& g) { return g.D == 2; }
 
 long long fused2d_partials(const Geo& g, int G) {
   const int u = unit_of(g, G);
-  return (long long)ntiles(g, rows_of(g, G)) * ((g.T + u - 1) / u);
+  return (long long)ntiles(g, rows_of(g, G)) * ((g.T + u) / u);
 }
 
 void launch_fused2d(const Geo& g, int G, const MxFields& f, const MxFields& fn, double* socp_part, cudaStream_t s,
@@ -535,7 +535,7 @@ void launch_fused2d(const Geo& g, int G, const MxFields& f, const MxFields& fn, 
   a.ntx = (g.N[0] + tx - 1) / tx;
   a.nty = (g.N[1] + TY - 1) / TY;
   a.unit = unit_of(g, G);
-  a.nunit = (g.T + a.unit - 1) / a.unit;
+  a.nunit = (g.T + a.unit) / a.unit;
   a.sp = f.sp;
   a.socp_part = socp_part;
   a.r = f.r;
