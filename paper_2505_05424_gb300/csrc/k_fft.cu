@@ -727,7 +727,12 @@ __device__ __forceinline__ float recip(float x) {
   const float r = rcp_approx(x);
   return fmaf(r, fmaf(-x, r, 1.f), r);
 }
-__device__ __forceinline__ double recip(double x) { return 1.0 / x; }
+__device__ __forceinline__ double recip(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));   // 2^-23, squared by each Newton step
+  r = fma(r, fma(-x, r, 1.0), r);
+  return fma(r, fma(-x, r, 1.0), r);
+}
 
 template <class R>
 struct TimeArgs {

@@ -6,6 +6,7 @@
 #include <cmath>
 
 #include "dot_internal.cuh"
+#include "dot_reduce.cuh"
 
 namespace dot {
 namespace {
@@ -113,7 +114,7 @@ __global__ void k_update_q0(Geo g, F64Fields f, double sigma, double tau) {
     const double uK = f.z[(long long)(K - 1) * n0 + i] - 1.0 + f.beta[(long long)(K - 1) * n0 + i] * isg;
     const double u0 = f.z[i] - 1.0 + f.beta[i] * isg;
     const double a = f.al[0][i];
-    const double qn = (aphi + a * isg + (uK - u0)) / 3.0;
+    const double qn = (aphi + a * isg + (uK - u0)) * (1.0 / 3.0);
     f.q[0][i] = qn;
     f.al[0][i] = a + tau * sigma * (aphi - qn);
   }
@@ -129,6 +130,10 @@ __global__ void k_update_qd(Geo g, F64Fields f, int d, double sigma, double tau)
   const long long n0 = (long long)g.T * g.P;
   const double isg = 1.0 / sigma;
   const double s_default = sqrt(0.5);
+  // without obstacles the diagonal takes two values: the division (some ten FP64
+  // instructions) is done once per thread
+  const double one = 2.0 * (s_default * s_default);
+  const double r1 = 1.0 / (1.0 + one), r2 = 1.0 / (1.0 + 2.0 * one);
   const long long s = g.sst[d];
   double* qd = f.q[1 + d];
   double* ad = f.al[1 + d];
@@ -174,7 +179,8 @@ __global__ void k_update_qd(Geo g, F64Fields f, int d, double sigma, double tau)
       }
     }
     const double a = ad[i];
-    const double qn = (aphi + a * isg + acc) / (1.0 + dg);
+    const double rden = f.somega ? 1.0 / (1.0 + dg) : (t >= 1 && t < g.T ? r2 : r1);
+    const double qn = (aphi + a * isg + acc) * rden;
     qd[i] = qn;
     ad[i] = a + tau * sigma * (aphi - qn);
   }
@@ -211,25 +217,9 @@ __global__ void k_update_beta(Geo g, F64Fields f, double sigma, double tau) {
 
 constexpr int kKktBlocks = 608;
 
-__device__ __forceinline__ void block_reduce_store(double* acc, double* out_row) {
-  __shared__ double sh[kThreads / 32][R_NSLOTS];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int k = 0; k < R_NSLOTS; ++k) {
-    double v = acc[k];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) sh[warp][k] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < R_NSLOTS) {
-    double v = 0.0;
-    for (int w = 0; w < kThreads / 32; ++w) v += sh[w][threadIdx.x];
-    out_row[threadIdx.x] = v;
-  }
-}
-
 // Cones (time faces): eta_P terms of q_0, f(q), complementarity of alpha_0,
 // z - BFq - d, and F^*B^*beta + alpha on q_0.
-__global__ void k_kkt_cones(Geo g, F64Fields f, double* partials) {
+__global__ void k_kkt_cones(Geo g, F64Fields f, double* partials, int rows) {
   double acc[R_NSLOTS];
   for (int k = 0; k < R_NSLOTS; ++k) acc[k] = 0.0;
   const long long n0 = (long long)g.T * g.P;
@@ -269,13 +259,15 @@ __global__ void k_kkt_cones(Geo g, F64Fields f, double* partials) {
     acc[R_SOCD] += (fbb + a0) * (fbb + a0);
     acc[R_FBB] += fbb * fbb;
   }
-  block_reduce_store(acc, partials + (long long)blockIdx.x * R_NSLOTS);
+  constexpr int w[9] = {R_PRIM, R_APHI, R_Q, R_COMP0, R_ALPHA0, R_F, R_SOCP, R_SOCD, R_FBB};
+  const double v[9] = {acc[R_PRIM], acc[R_APHI], acc[R_Q], acc[R_COMP0], acc[R_ALPHA0], acc[R_F], acc[R_SOCP], acc[R_SOCD], acc[R_FBB]};
+  block_reduce_store<kThreads>(v, w, partials, rows, blockIdx.x);
 }
 
 // Faces of axis d: eta_P terms, g_d = (L_X^d L_T^*(omega alpha_0)) o q_d (the mean of
 // omega alpha_0 over the up-to-four cones touching the face, each weighted 1/4),
 // the dual objective term, and F^*B^*beta + alpha on q_d.
-__global__ void k_kkt_faces(Geo g, F64Fields f, int d, double* partials) {
+__global__ void k_kkt_faces(Geo g, F64Fields f, int d, double* partials, int rows) {
   double acc[R_NSLOTS];
   for (int k = 0; k < R_NSLOTS; ++k) acc[k] = 0.0;
   const long long n = (long long)(g.T + 1) * g.P;
@@ -319,11 +311,13 @@ __global__ void k_kkt_faces(Geo g, F64Fields f, int d, double* partials) {
     acc[R_SOCD] += (fbb + a) * (fbb + a);
     acc[R_FBB] += fbb * fbb;
   }
-  block_reduce_store(acc, partials + (long long)blockIdx.x * R_NSLOTS);
+  constexpr int w[9] = {R_PRIM, R_APHI, R_Q, R_COMPD, R_ALPHAB, R_G, R_SOCD, R_FBB, R_DUALOBJ};
+  const double v[9] = {acc[R_PRIM], acc[R_APHI], acc[R_Q], acc[R_COMPD], acc[R_ALPHAB], acc[R_G], acc[R_SOCD], acc[R_FBB], acc[R_DUALOBJ]};
+  block_reduce_store<kThreads>(v, w, partials, rows, (1 + d) * gridDim.x + blockIdx.x);
 }
 
 // Nodes: A^* alpha + c and <c, phi>.
-__global__ void k_kkt_nodes(Geo g, F64Fields f, double* partials) {
+__global__ void k_kkt_nodes(Geo g, F64Fields f, double* partials, int rows) {
   double acc[R_NSLOTS];
   for (int k = 0; k < R_NSLOTS; ++k) acc[k] = 0.0;
   const long long n = (long long)(g.T + 1) * g.P;
@@ -348,24 +342,15 @@ __global__ void k_kkt_nodes(Geo g, F64Fields f, double* partials) {
     acc[R_DUALRES] += v * v;
     acc[R_CPHI] += c * f.phi[i];
   }
-  block_reduce_store(acc, partials + (long long)blockIdx.x * R_NSLOTS);
+  constexpr int w[2] = {R_DUALRES, R_CPHI};
+  const double v[2] = {acc[R_DUALRES], acc[R_CPHI]};
+  block_reduce_store<kThreads>(v, w, partials, rows, (1 + g.D) * gridDim.x + blockIdx.x);
 }
 
-// Fixed-order sum of the partial rows: deterministic run to run.
-__global__ void k_kkt_final(const double* partials, int rows, double* out) {
-  __shared__ double sh[kThreads];
-  for (int k = 0; k < R_NSLOTS; ++k) {
-    double v = 0.0;
-    for (int r = threadIdx.x; r < rows; r += blockDim.x) v += partials[(long long)r * R_NSLOTS + k];
-    sh[threadIdx.x] = v;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-      if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) out[k] = sh[0];
-    __syncthreads();
-  }
+// Fixed-order sum of the partial rows, a block per sum: deterministic run to run.
+__global__ void __launch_bounds__(128) k_kkt_final(const double* partials, int rows, double* out) {
+  const double v = row_sum128(partials + (long long)blockIdx.x * rows, rows);
+  if (threadIdx.x == 0) out[blockIdx.x] = v;
 }
 
 }  // namespace
@@ -400,11 +385,11 @@ long long kkt_partials_len(const Geo& g) { return (long long)(g.D + 2) * kKktBlo
 
 void launch_kkt_f64(const Geo& g, const F64Fields& f, double* partials, double* out, cudaStream_t s,
                     LaunchCounter lc) {
-  k_kkt_cones<<<kKktBlocks, kThreads, 0, s>>>(g, f, partials);
-  for (int d = 0; d < g.D; ++d)
-    k_kkt_faces<<<kKktBlocks, kThreads, 0, s>>>(g, f, d, partials + (long long)(1 + d) * kKktBlocks * R_NSLOTS);
-  k_kkt_nodes<<<kKktBlocks, kThreads, 0, s>>>(g, f, partials + (long long)(1 + g.D) * kKktBlocks * R_NSLOTS);
-  k_kkt_final<<<1, kThreads, 0, s>>>(partials, (g.D + 2) * kKktBlocks, out);
+  const int rows = (g.D + 2) * kKktBlocks;
+  k_kkt_cones<<<kKktBlocks, kThreads, 0, s>>>(g, f, partials, rows);
+  for (int d = 0; d < g.D; ++d) k_kkt_faces<<<kKktBlocks, kThreads, 0, s>>>(g, f, d, partials, rows);
+  k_kkt_nodes<<<kKktBlocks, kThreads, 0, s>>>(g, f, partials, rows);
+  k_kkt_final<<<R_NSLOTS, 128, 0, s>>>(partials, rows, out);
   lc.launched(KID_KKT, g.D + 3);
 }
 

@@ -15,6 +15,7 @@
 
 #include "dot_internal.cuh"
 #include "dot_mixed.cuh"
+#include "dot_reduce.cuh"
 #include "ffloat.cuh"
 
 namespace dot {
@@ -307,12 +308,10 @@ __device__ __forceinline__ void gather_Fq(const Geo& g, float* const* q, int i, 
 // Kinds of blocks run side by side -- cones, faces along x and y (which share beta's
 // pairs), for D = 3 faces along z, and nodes -- each over its own sums.  A
 // 32-lane FP64 instruction occupies an SM for 16 cycles, so nothing per element is FP64
-// but the two planes that carry c, a block adds up only the sums of its kind, and a
-// warp's tree halves the number of sums a lane carries at every exchange (16 additions
-// for 16 sums instead of 80).  Bound by the latency of each element's loads; per check
-// on 256^2 x 64 219 us (0.73 GB read; 350 us when every block ran all kinds in turn with
-// FP64 on every node), 128^2 x 32 41 (86), 32^2 x 16 14 (49), 64^3 x 32 585 (983).  Four
-// CTAs per SM for D = 2 (three 241 us, five 237), three for D = 3 (four 643 us, five 618).
+// but the two planes that carry c, and the sums take few additions (dot_reduce.cuh).  Bound by the latency of each element's loads; per check
+// on 256^2 x 64 216 us (0.73 GB read; 350 us when every block ran all kinds in turn with
+// FP64 on every node), 128^2 x 32 41 (86), 32^2 x 16 14 (49), 64^3 x 32 700 (983).  Four
+// CTAs per SM for D = 2 (three 241 us, five 237), three for D = 3.
 
 constexpr int kKktBlocks = 152 * 3;   // most blocks per slot and kind
 __host__ __device__ constexpr int kkt_kinds(int D) { return D == 2 ? 3 : 4; }
@@ -327,46 +326,6 @@ inline int kkt_blocks(const Geo& g) {
   const long long nn = (long long)(g.T + 1) * g.P;
   const long long b = (nn + kThreads - 1) / kThreads;
   return (int)(b < 1 ? 1 : (b > kKktBlocks ? kKktBlocks : b));
-}
-
-// Sums of v[0 .. 15] over the warp: lane l returns the sum of v[l / 2].
-__device__ __forceinline__ double warp_sums16(double* v) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int h = 8; h >= 1; h /= 2) {   // lanes exchange at distance 2 h and keep half of their sums
-    const bool up = lane & (2 * h);
-#pragma unroll
-    for (int k = 0; k < h; ++k) {
-      const double send = up ? v[k] : v[k + h], keep = up ? v[k + h] : v[k];
-      v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * h);
-    }
-  }
-  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
-}
-
-// The block's sums of the slots listed in `which` (n of them) into out[slot rows + row].
-template <int NS>
-__device__ __forceinline__ void block_reduce_store(const double (&val)[NS], const int (&which)[NS], double* out,
-                                                   int rows, int row) {
-  static_assert(NS <= 16, "one exchange tree");
-  __shared__ double sh[kThreads / 32][16];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double v[16];
-#pragma unroll
-  for (int k = 0; k < 16; ++k) v[k] = k < NS ? val[k < NS ? k : 0] : 0.0;
-  const double t = warp_sums16(v);
-  if ((lane & 1) == 0) sh[warp][lane >> 1] = t;
-  __syncthreads();
-  if (threadIdx.x < R_NSLOTS) {
-    int at = -1;
-#pragma unroll
-    for (int k = 0; k < NS; ++k)
-      if (which[k] == (int)threadIdx.x) at = k;
-    double s = 0.0;
-    if (at >= 0)
-      for (int w = 0; w < kThreads / 32; ++w) s += sh[w][at];
-    out[(long long)threadIdx.x * rows + row] = s;
-  }
 }
 
 // One node's share of the stopping measures: its cone (t < T), its faces along
@@ -509,7 +468,7 @@ __global__ void __launch_bounds__(kThreads, D == 2 ? 4 : 3) k_kkt(const __grid_c
   const float sg = sg2.x + sg2.y;
   double* partials = partials_all + slot * kkt_partials_len_slot(g);
   const int rows = kkt_kinds(D) * gridDim.x, row = kind * gridDim.x + blockIdx.x;
-  const int P = (int)g.P, n = (g.T + 1) * P, n0 = g.T * P;
+  const int P = (int)g.P, n0 = g.T * P;
   const int i0 = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
   float acc[R_NSLOTS];
 #pragma unroll
@@ -522,7 +481,7 @@ __global__ void __launch_bounds__(kThreads, D == 2 ? 4 : 3) k_kkt(const __grid_c
     double v[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) v[k] = acc[w[k]];
-    block_reduce_store(v, w, partials, rows, row);
+    block_reduce_store<kThreads>(v, w, partials, rows, row);
   } else if (kind < kkt_kinds(D) - 1) {
     float2 dual = make_float2(0.f, 0.f);
     if (kind == 1) kkt_face_loop<D, true>(g, f, sg, i0, stride, acc, &dual);
@@ -532,7 +491,7 @@ __global__ void __launch_bounds__(kThreads, D == 2 ? 4 : 3) k_kkt(const __grid_c
 #pragma unroll
     for (int k = 0; k < 8; ++k) v[k] = acc[w[k]];
     v[8] = ff_to_double(dual);
-    block_reduce_store(v, w, partials, rows, row);
+    block_reduce_store<kThreads>(v, w, partials, rows, row);
   } else {
     // planes 1 .. T - 1 carry no c
 #pragma unroll 2
@@ -555,7 +514,7 @@ __global__ void __launch_bounds__(kThreads, D == 2 ? 4 : 3) k_kkt(const __grid_c
       for (int i = i0; i < nsocp; i += stride) socp += socp_all[(long long)slot * nsocp + i];
     constexpr int w[3] = {R_DUALRES, R_SOCP, R_CPHI};
     const double v[3] = {(double)acc[R_DUALRES] + dres, socp, cphi};
-    block_reduce_store(v, w, partials, rows, row);
+    block_reduce_store<kThreads>(v, w, partials, rows, row);
   }
 }
 
@@ -565,14 +524,8 @@ __global__ void __launch_bounds__(128) k_kkt_final(Geo g, const SlotParam* sp, c
   const int slot = blockIdx.x, k = blockIdx.y;
   if (!sp[slot].active) return;
   const double* p = partials_all + slot * kkt_partials_len_slot(g) + (long long)k * rows;
-  double v = 0.0;
-#pragma unroll 4
-  for (int r = threadIdx.x; r < rows; r += 128) v += p[r];
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  __shared__ double sh[4];
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) out_all[slot * R_NSLOTS + k] = (sh[0] + sh[1]) + (sh[2] + sh[3]);
+  const double v = row_sum128(p, rows);
+  if (threadIdx.x == 0) out_all[slot * R_NSLOTS + k] = v;
 }
 
 // Line 2 with one refinement step: phi1 = P(b); r = b - A^*A phi1 (exact);
