@@ -52,7 +52,7 @@ constexpr size_t kOffBlo = kOffB + kField;
 constexpr size_t kOffPhi1 = kOffBlo + kField;
 constexpr size_t kOffR = kOffPhi1 + kField;
 constexpr size_t kOffW1 = kOffR + kField;
-constexpr size_t kOffW2 = kOffW1 + kField;
+constexpr size_t kOffW2 = kOffW1 + kField;   // (on small grids with an odd N_y w1 runs up to (T+1) N_x floats into w2)
 constexpr size_t kOffUp = kOffW2 + kField;
 constexpr size_t kOffSum = kOffUp + (sizeof(Upload) + 255) / 256 * 256;   // partial sums of b, then mean(b)
 constexpr size_t kScratchBytes = kOffSum + kBsumStride * sizeof(double);

@@ -25,7 +25,7 @@
 // passes along time.  256^2 x 64, per iteration: 4 x 16.3 + 18.5 us (tensor cores
 // 4 x 25.4 + 2 x 23.6); 1024^2 x 32: 4 x 115 + 62 (4 x 396 + 2 x 162); 64^3 x 32:
 // 6 x 20.2 + 20.7 (6 x 30 + 2 x 54); 150 x 117 x 37, where the dense transform ran on
-// the FP32 units: 4 x 12.5 + 10 (4 x 22 + 19).  A cold solve's error is 2 to 5 times
+// the FP32 units: 2 x 14.8 + 20.7 (k_xtx; 4 x 22 + 19).  A cold solve's error is 2 to 5 times
 // smaller than the 3xTF32 one's.
 //
 // FP64: GB300 issues two FP64 lanes per SM and clock, so the count of operations is the
@@ -74,6 +74,7 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kMaxStages = 16;
+constexpr int kMaxSmem = 220 * 1024;
 
 struct FftPlan {
   int N, nst;
@@ -119,6 +120,10 @@ struct FftArgs {
   long long nseq;         // sequences (inner == 1)
   const SlotParam* sp;
   long long slot_pairs;   // pairs per slot (sp != nullptr)
+  // inner == 1: the frequency side is not the field's layout but W[slot][k / 2][row][k % 2],
+  // the layout of k_xtx (forward: of dst, inverse: of src); rows of a slot
+  int rot, slot_rows;
+  FastDiv fslot;          // division by the pairs of a slot
   FftPlan plan;
 };
 
@@ -199,14 +204,40 @@ __device__ __forceinline__ void dft(V* x) {
   }
 }
 
+// The pairs of sequences a CTA holds, stored pair by pair at each position with an odd
+// pitch: a number known at compile time, or any.
+template <int NP>
+struct FixedPairs {
+  static constexpr int kThreads = 256;
+  __device__ __forceinline__ int count() const { return NP; }
+  __device__ __forceinline__ int pitch() const { return NP + 1; }
+  __device__ __forceinline__ int split(int e, int* pr) const {   // e = rest * count + pair
+    *pr = e % NP;
+    return e / NP;
+  }
+};
+struct AnyPairs {
+  static constexpr int kThreads = 512;
+  int n;
+  FastDiv f;
+  __device__ __forceinline__ int count() const { return n; }
+  __device__ __forceinline__ int pitch() const { return n | 1; }
+  __device__ __forceinline__ int split(int e, int* pr) const {
+    const int b = (int)fdiv((unsigned)e, f);
+    *pr = e - b * n;
+    return b;
+  }
+};
+
 // One Stockham stage of radix RAD with stride s: butterfly b = p s + q reads elements
 // b + (N / RAD) j and writes q + s (RAD p + k), times exp(-2 pi i s p k / N).
-template <int RAD, int NP, bool INV, class V>
-__device__ __forceinline__ void stage(const V* src, V* dst, const V* tw, int N, int s, FastDiv fs) {
-  constexpr int kPitch = NP + 1;
+template <int RAD, bool INV, class Q, class V>
+__device__ __forceinline__ void stage(const Q& np, const V* src, V* dst, const V* tw, int N, int s, FastDiv fs) {
+  const int kPitch = np.pitch();
   const int nb = N / RAD;
-  for (int e = threadIdx.x; e < nb * NP; e += kThreads) {
-    const int pr = e % NP, b = e / NP;
+  for (int e = threadIdx.x; e < nb * np.count(); e += Q::kThreads) {
+    int pr;
+    const int b = np.split(e, &pr);
     const int p = (int)fdiv((unsigned)b, fs), q = b - p * s;
     V x[RAD];
 #pragma unroll
@@ -225,13 +256,14 @@ __device__ __forceinline__ void stage(const V* src, V* dst, const V* tw, int N, 
 
 // A stage of any odd radix r: outputs k and r - k share their sums over the conjugate
 // input pairs, sum_j (x_j + x_{r-j}) cos and (x_j - x_{r-j}) sin.
-template <int NP, bool INV, class V>
-__device__ __forceinline__ void stage_any(const V* src, V* dst, const V* tw, int N, int r, int s, FastDiv fs,
-                                          FastDiv fr) {
-  constexpr int kPitch = NP + 1;
+template <bool INV, class Q, class V>
+__device__ __forceinline__ void stage_any(const Q& np, const V* src, V* dst, const V* tw, int N, int r, int s,
+                                          FastDiv fs, FastDiv fr) {
+  const int kPitch = np.pitch();
   const int nb = N / r, hk = (r + 1) / 2;
-  for (int e = threadIdx.x; e < nb * hk * NP; e += kThreads) {
-    const int pr = e % NP, bk = e / NP;
+  for (int e = threadIdx.x; e < nb * hk * np.count(); e += Q::kThreads) {
+    int pr;
+    const int bk = np.split(e, &pr);
     const int k = (int)fdiv((unsigned)bk, fr), b = bk - k * nb;
     const int p = (int)fdiv((unsigned)b, fs), q = b - p * s;
     const V* x = src + b * kPitch + pr;
@@ -260,18 +292,18 @@ __device__ __forceinline__ void stage_any(const V* src, V* dst, const V* tw, int
 }
 
 // All stages; returns the buffer that holds the result.
-template <int NP, bool INV, class V>
-__device__ __forceinline__ V* transform(V* a, V* b, const V* tw, const FftPlan& pl) {
+template <bool INV, class Q, class V>
+__device__ __forceinline__ V* transform(const Q& np, V* a, V* b, const V* tw, const FftPlan& pl) {
   int s = 1;
   for (int i = 0; i < pl.nst; ++i) {
     const int r = pl.rad[i];
     switch (r) {
-      case 8: stage<8, NP, INV>(a, b, tw, pl.N, s, pl.fs[i]); break;
-      case 4: stage<4, NP, INV>(a, b, tw, pl.N, s, pl.fs[i]); break;
-      case 2: stage<2, NP, INV>(a, b, tw, pl.N, s, pl.fs[i]); break;
-      case 3: stage<3, NP, INV>(a, b, tw, pl.N, s, pl.fs[i]); break;
-      case 5: stage<5, NP, INV>(a, b, tw, pl.N, s, pl.fs[i]); break;
-      default: stage_any<NP, INV>(a, b, tw, pl.N, r, s, pl.fs[i], pl.fr[i]); break;
+      case 8: stage<8, INV>(np, a, b, tw, pl.N, s, pl.fs[i]); break;
+      case 4: stage<4, INV>(np, a, b, tw, pl.N, s, pl.fs[i]); break;
+      case 2: stage<2, INV>(np, a, b, tw, pl.N, s, pl.fs[i]); break;
+      case 3: stage<3, INV>(np, a, b, tw, pl.N, s, pl.fs[i]); break;
+      case 5: stage<5, INV>(np, a, b, tw, pl.N, s, pl.fs[i]); break;
+      default: stage_any<INV>(np, a, b, tw, pl.N, r, s, pl.fs[i], pl.fr[i]); break;
     }
     __syncthreads();
     V* t = a;
@@ -328,6 +360,37 @@ __device__ __forceinline__ V zk(V w, V xk, V xm) {
 template <class V>
 __device__ __forceinline__ V xk_of(V w, V z, V y) {
   return mk<V>(w.x * (z.x + y.x) + w.y * (z.y - y.y), w.x * (z.y + y.y) - w.y * (z.x - y.x));
+}
+
+// Element (pair kp of frequencies) of the first row of row pair pg in W.
+template <class R>
+__device__ __forceinline__ long long rot_at(const FftArgs<R>& a, long long pg, int kp) {
+  const int z = (int)fdiv((unsigned)pg, a.fslot);
+  const long long row = 2 * (pg - (long long)z * a.fslot.d);
+  return ((long long)z * ((a.plan.N + 1) / 2) + kp) * a.slot_rows + row;
+}
+
+// Frequencies 2 kp, 2 kp + 1 of row pair pg: out of Z (forward) into W, or from W (inverse)
+// into the raw spectrum B.
+template <class R, class V>
+__device__ __forceinline__ void rot_store(const FftArgs<R>& a, long long pg, int kp, const V* rotf, const V* Z, int pitch,
+                                          int pr) {
+  const int N = a.plan.N, k = 2 * kp;
+  const V x = xk_of(rotf[k], Z[k * pitch + pr], Z[(k ? N - k : 0) * pitch + pr]);
+  V y = mk<V>((R)0, (R)0);
+  if (k + 1 < N) y = xk_of(rotf[k + 1], Z[(k + 1) * pitch + pr], Z[(N - k - 1) * pitch + pr]);
+  if (2 * pg >= a.nseq) return;
+  V* w = reinterpret_cast<V*>(a.dst) + rot_at(a, pg, kp);
+  w[0] = mk<V>(x.x, y.x);
+  if (2 * pg + 1 < a.nseq) w[1] = mk<V>(x.y, y.y);
+}
+template <class R, class V>
+__device__ __forceinline__ void rot_load(const FftArgs<R>& a, long long pg, int kp, V* va, V* vb) {
+  *va = *vb = mk<V>((R)0, (R)0);
+  if (2 * pg >= a.nseq) return;
+  const V* w = reinterpret_cast<const V*>(a.src) + rot_at(a, pg, kp);
+  *va = __ldg(w);
+  if (2 * pg + 1 < a.nseq) *vb = __ldg(w + 1);
 }
 
 // Whether any slot of the pairs [p0, p0 + np) holds a solve.
@@ -406,7 +469,7 @@ __global__ void __launch_bounds__(kThreads) k_dct_any(const __grid_constant__ Ff
       }
     }
     __syncthreads();
-    const V* Z = transform<NP, INV>(A, B, tw, a.plan);
+    const V* Z = transform<INV>(FixedPairs<NP>(), A, B, tw, a.plan);
     if (!c.ok) return;
     if (!INV) {
 #pragma unroll 2
@@ -422,14 +485,26 @@ __global__ void __launch_bounds__(kThreads) k_dct_any(const __grid_constant__ Ff
     }
   } else {
     // pairs of contiguous rows: neighbouring threads take neighbouring elements
+    const int nk = (N + 1) / 2;
+    if (INV && a.rot) {
 #pragma unroll 4
-    for (int e = threadIdx.x; e < NP * N; e += kThreads) {
-      const int pr = (int)fdiv((unsigned)e, a.plan.fN), j = e - pr * N;
-      const long long row = 2 * (p0 + pr);
-      const R* s = a.src + row * N + j;
-      const V v = mk<V>(row < a.nseq ? __ldg(s) : (R)0, row + 1 < a.nseq ? __ldg(s + N) : (R)0);
-      if (INV) B[j * kPitch + pr] = v;
-      else A[((j & 1) ? N - 1 - (j >> 1) : j >> 1) * kPitch + pr] = v;
+      for (int e = threadIdx.x; e < NP * nk; e += kThreads) {
+        const int pr = e % NP, kp = e / NP;
+        V va, vb;
+        rot_load(a, p0 + pr, kp, &va, &vb);
+        B[2 * kp * kPitch + pr] = mk<V>(va.x, vb.x);
+        if (2 * kp + 1 < N) B[(2 * kp + 1) * kPitch + pr] = mk<V>(va.y, vb.y);
+      }
+    } else {
+#pragma unroll 4
+      for (int e = threadIdx.x; e < NP * N; e += kThreads) {
+        const int pr = (int)fdiv((unsigned)e, a.plan.fN), j = e - pr * N;
+        const long long row = 2 * (p0 + pr);
+        const R* s = a.src + row * N + j;
+        const V v = mk<V>(row < a.nseq ? __ldg(s) : (R)0, row + 1 < a.nseq ? __ldg(s + N) : (R)0);
+        if (INV) B[j * kPitch + pr] = v;
+        else A[((j & 1) ? N - 1 - (j >> 1) : j >> 1) * kPitch + pr] = v;
+      }
     }
     __syncthreads();
     if (INV) {
@@ -441,7 +516,11 @@ __global__ void __launch_bounds__(kThreads) k_dct_any(const __grid_constant__ Ff
       }
       __syncthreads();
     }
-    const V* Z = transform<NP, INV>(A, B, tw, a.plan);
+    const V* Z = transform<INV>(FixedPairs<NP>(), A, B, tw, a.plan);
+    if (!INV && a.rot) {
+      for (int e = threadIdx.x; e < NP * nk; e += kThreads) rot_store(a, p0 + e % NP, e / NP, rotf, Z, kPitch, e % NP);
+      return;
+    }
     const int np = (int)min((long long)NP, a.npair - p0);
 #pragma unroll 4
     for (int e = threadIdx.x; e < np * N; e += kThreads) {
@@ -628,6 +707,17 @@ __global__ void __launch_bounds__(Pow2<N, NP>::kThreads) k_dct_pow2(const __grid
     // pairs of contiguous rows, four neighbouring elements of both per thread and step
     constexpr int kQ = N / 4, kIt = 4;                 // kT kIt chunks in all
     static_assert(kT * kIt == NP * kQ, "four chunks per thread");
+    if (INV && a.rot) {
+      V wa[8], wb[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) rot_load(a, p0 + pr, b + u * kNb, &wa[u], &wb[u]);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int k = 2 * (b + u * kNb);
+        A[k * kPitch + pr] = mk<V>(wa[u].x, wb[u].x);
+        A[(k + 1) * kPitch + pr] = mk<V>(wa[u].y, wb[u].y);
+      }
+    } else {
     R va[kIt][4], vb[kIt][4];
 #pragma unroll
     for (int u = 0; u < kIt; ++u) {
@@ -653,6 +743,7 @@ __global__ void __launch_bounds__(Pow2<N, NP>::kThreads) k_dct_pow2(const __grid
         for (int q = 0; q < 4; ++q) A[(j + q) * kPitch + r] = mk<V>(va[u][q], vb[u][q]);
       }
     }
+    }
     __syncthreads();
     if constexpr (INV) {
 #pragma unroll
@@ -665,6 +756,11 @@ __global__ void __launch_bounds__(Pow2<N, NP>::kThreads) k_dct_pow2(const __grid
       __syncthreads();
     }
     p2_stages<N, NP, 1, INV, false>(x, A, tw, b, pr);
+    if (!INV && a.rot) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) rot_store(a, p0 + pr, b + u * kNb, rotf, A, kPitch, pr);
+      return;
+    }
     if constexpr (INV && sizeof(R) == 4) {
       if (a.accum) {
 #pragma unroll
@@ -858,7 +954,116 @@ __global__ void __launch_bounds__(THREADS) k_time_solve(const __grid_constant__ 
   }
 }
 
-constexpr int kMaxSmem = 220 * 1024;
+// ---- small grids (D = 2): the x transforms and the time solve in one block ------------
+//
+// On small grids a pass is a launch and one trip to memory and back for a few microseconds
+// of work.  For a pair of y frequencies everything along x and time is independent of
+// the others, so a block takes W[slot][kp] = (T + 1) x N_x pairs -- which the y pass wrote
+// side by side -- and runs the x transform, the time solve of its 2 N_x columns and the
+// x transform back in shared memory: three launches per solve instead of five.  Bound by
+// launch, barriers and the serial time recurrence (128^2 x 32: 17 us).
+struct XtxArgs {
+  float2* w;              // in place
+  const float2* tab;      // axis x
+  const float* lam[2];    // eigenvalues along x and y
+  float a;                // 1 / h_0^2
+  int M, N1, rows;        // time nodes, points along y, rows of a slot
+  FastDiv fN0;
+  AnyPairs np;            // M pairs
+  FftPlan plan;           // axis x
+  const SlotParam* sp;
+};
+
+__global__ void __launch_bounds__(AnyPairs::kThreads) k_xtx(const __grid_constant__ XtxArgs a) {
+  using V = float2;
+  constexpr int kT = AnyPairs::kThreads;
+  extern __shared__ __align__(16) unsigned char fsm[];
+  const int slot = blockIdx.y, kp = blockIdx.x;
+  if (a.sp && !a.sp[slot].active) return;
+  const int M = a.M, N = a.plan.N, pitch = a.np.pitch();
+  V* A = reinterpret_cast<V*>(fsm);
+  V* B = A + N * pitch;
+  V* tw = B + N * pitch;
+  V* W = a.w + ((long long)slot * gridDim.x + kp) * a.rows;
+  for (int j = threadIdx.x; j < N; j += kT) tw[j] = __ldg(a.tab + j);
+#pragma unroll 4
+  for (int e = threadIdx.x; e < M * N; e += kT) {
+    const int t = (int)fdiv((unsigned)e, a.fN0), x = e - t * N;
+    A[((x & 1) ? N - 1 - (x >> 1) : x >> 1) * pitch + t] = W[e];
+  }
+  __syncthreads();
+  V* Z = transform<false>(a.np, A, B, tw, a.plan);
+  V* Y = Z == A ? B : A;   // the free buffer
+  const V* rf = a.tab + N;
+  const int half = (N / 2 + 1) * M;
+  for (int e = threadIdx.x; e < half; e += kT) {   // in place: a thread owns its k, N - k
+    int t;
+    const int k = a.np.split(e, &t), m = k ? N - k : 0;
+    const V z = Z[k * pitch + t], y = Z[m * pitch + t];
+    Z[k * pitch + t] = xk_of(__ldg(rf + k), z, y);
+    if (k && m != k) Z[m * pitch + t] = xk_of(__ldg(rf + m), y, z);
+  }
+  __syncthreads();
+  // the columns (k_x, lane): pivots' reciprocals in the free buffer, at the column's places
+  const float c = a.a;
+  if (kp == 0 && threadIdx.x >= kT - 32) {
+    float* z = reinterpret_cast<float*>(Z);
+    zero_column(z, reinterpret_cast<float*>(Y), M, 2LL, 1.0 / (double)c);
+    __syncwarp();
+    for (int t = threadIdx.x & 31; t < M; t += 32) z[2 * t] = reinterpret_cast<float*>(Y)[2 * t];
+  }
+  for (int e = threadIdx.x; e < 2 * N; e += kT) {
+    const int k = e >> 1, l = e & 1, ky = 2 * kp + l;
+    if (ky >= a.N1 || (k == 0 && ky == 0)) continue;
+    const float lam = __ldg(a.lam[0] + k) + __ldg(a.lam[1] + ky);
+    float* y = reinterpret_cast<float*>(Z + k * pitch) + l;
+    float* rr = reinterpret_cast<float*>(Y + k * pitch) + l;
+    float s = lam, r = recip(c + s), yp = y[0];
+    rr[0] = r;
+    for (int t = 1; t < M; ++t) {
+      const float ar = c * r;
+      s = lam + ar * s;
+      r = recip(t < M - 1 ? c + s : s);
+      yp = y[2 * t] + ar * yp;
+      y[2 * t] = yp;
+      rr[2 * t] = r;
+    }
+    float xp = yp * r;
+    y[2 * (M - 1)] = xp;
+#pragma unroll 4
+    for (int t = M - 2; t >= 0; --t) {
+      xp = (y[2 * t] + c * xp) * rr[2 * t];
+      y[2 * t] = xp;
+    }
+  }
+  __syncthreads();
+  const V* ri = a.tab + 2 * N;
+  for (int e = threadIdx.x; e < half; e += kT) {
+    int t;
+    const int k = a.np.split(e, &t), m = N - k;
+    const V xk = Z[k * pitch + t], xm = k ? Z[m * pitch + t] : make_float2(0.f, 0.f);
+    Z[k * pitch + t] = zk(__ldg(ri + k), xk, xm);
+    if (k && m != k) Z[m * pitch + t] = zk(__ldg(ri + m), xm, xk);
+  }
+  __syncthreads();
+  const V* X = transform<true>(a.np, Z, Y, tw, a.plan);
+#pragma unroll 4
+  for (int e = threadIdx.x; e < M * N; e += kT) {
+    const int t = (int)fdiv((unsigned)e, a.fN0), x = e - t * N;
+    W[e] = X[((x & 1) ? N - 1 - (x >> 1) : x >> 1) * pitch + t];
+  }
+}
+
+size_t xtx_smem(const Geo& g) { return ((size_t)2 * g.N[0] * ((g.T + 1) | 1) + g.N[0]) * sizeof(float2); }
+// Small grids by their own size (not the batch's, whose members' results may not depend
+// on it), up to the size where the passes of their own are as fast.  An iteration,
+// with and without: 32^2 x 16 23.8 and 26.5 us, 64^2 x 32 37.9 and 41.5, 128^2 x 32 84.5 and
+// 87.2, 150 x 117 x 37 103.0 and 105.4, 256^2 x 9 92.6 and 98.9, 512^2 x 8 243.6 and 250.7,
+// 256^2 x 32 (8,448 pairs per block) 200.6 and 202.6.
+bool use_xtx(const Geo& g) {
+  return g.D == 2 && (long long)(g.T + 1) * g.N[0] <= 8704 && xtx_smem(g) <= (size_t)kMaxSmem;
+}
+
 template <class R> constexpr int time_threads() { return sizeof(R) == 4 ? 128 : 64; }
 
 template <class R>
@@ -914,7 +1119,7 @@ bool try_pow2(const FftArgs<R>& a, cudaStream_t s) {
 // One axis of G solves.  Pairs per CTA: 16 (8 in FP64: 128-byte segments of a strided
 // axis), fewer while that leaves SMs without a CTA or does not fit shared memory.
 template <class R, bool INV>
-void fft_axis(const Geo& g, int G, int axis, const FastPoisson<R>& fp, const R* src, R* dst, float2* accum,
+void fft_axis(const Geo& g, int G, int axis, const FastPoisson<R>& fp, const R* src, R* dst, float2* accum, bool rot,
               cudaStream_t s, LaunchCounter lc) {
   FftArgs<R> a;
   std::memset(&a, 0, sizeof(a));
@@ -930,6 +1135,9 @@ void fft_axis(const Geo& g, int G, int axis, const FastPoisson<R>& fp, const R* 
   a.npair = a.inner > 1 ? total / ((long long)N * a.inner) * a.pin : (a.nseq + 1) / 2;
   a.fpi = make_fastdiv((unsigned)a.pin);
   a.plan = make_plan(N);
+  a.rot = rot;
+  a.slot_rows = (int)(a.nseq / G);
+  a.fslot = make_fastdiv((unsigned)((a.slot_rows + 1) / 2));
   a.sp = G > 1 ? fp.sp : nullptr;
   a.slot_pairs = G > 1 ? a.npair / G : a.npair;
   if (try_pow2<R, INV>(a, s)) {
@@ -952,11 +1160,37 @@ void fft_axis(const Geo& g, int G, int axis, const FastPoisson<R>& fp, const R* 
 template <class R>
 void fast_poisson(const Geo& g, int G, const FastPoisson<R>& fp, const R* src, R* dst, float2* accum, cudaStream_t s,
                   LaunchCounter lc) {
+  if constexpr (sizeof(R) == 4) {
+    if (use_xtx(g)) {
+      fft_axis<R, false>(g, G, 1, fp, src, fp.w1, nullptr, true, s, lc);
+      XtxArgs x;
+      std::memset(&x, 0, sizeof(x));
+      x.w = reinterpret_cast<float2*>(fp.w1);
+      x.tab = fp.tab[0];
+      x.lam[0] = fp.lam[0];
+      x.lam[1] = fp.lam[1];
+      x.a = (float)(g.invh[0] * g.invh[0]);
+      x.M = g.T + 1;
+      x.N1 = g.N[1];
+      x.rows = x.M * g.N[0];
+      x.fN0 = make_fastdiv((unsigned)g.N[0]);
+      x.np.n = x.M;
+      x.np.f = make_fastdiv((unsigned)x.M);
+      x.plan = make_plan(g.N[0]);
+      x.sp = G > 1 ? fp.sp : nullptr;
+      static std::atomic<unsigned long long> done{0};
+      smem_optin((const void*)k_xtx, kMaxSmem, &done);
+      k_xtx<<<dim3((g.N[1] + 1) / 2, G), AnyPairs::kThreads, xtx_smem(g), s>>>(x);
+      lc.launched(KID_SCALE);
+      fft_axis<R, true>(g, G, 1, fp, fp.w1, dst, accum, true, s, lc);
+      return;
+    }
+  }
   R* w[2] = {fp.w1, fp.w2};
   const R* cur = src;
   int nx = 0;
   for (int d = g.D - 1; d >= 0; --d) {
-    fft_axis<R, false>(g, G, d, fp, cur, w[nx], nullptr, s, lc);
+    fft_axis<R, false>(g, G, d, fp, cur, w[nx], nullptr, false, s, lc);
     cur = w[nx];
     nx ^= 1;
   }
@@ -978,7 +1212,7 @@ void fast_poisson(const Geo& g, int G, const FastPoisson<R>& fp, const R* src, R
   nx ^= 1;
   for (int d = 0; d < g.D; ++d) {
     const bool last = d == g.D - 1;
-    fft_axis<R, true>(g, G, d, fp, cur, last ? dst : w[nx], last ? accum : nullptr, s, lc);
+    fft_axis<R, true>(g, G, d, fp, cur, last ? dst : w[nx], last ? accum : nullptr, false, s, lc);
     cur = w[nx];
     nx ^= 1;
   }

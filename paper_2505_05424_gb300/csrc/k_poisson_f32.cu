@@ -277,7 +277,10 @@ bool poisson_tc_flow(const Geo& g, const MxPoisson& ps) {
 size_t poisson_scratch_elems(const Geo& g) {
   const size_t nn = (size_t)(g.T + 1) * g.P;
   const size_t padded = (size_t)g.P * time_ld(g);
-  return nn > padded ? nn : padded;
+  // pairs of y frequencies (k_fft.cu: k_xtx); an odd N_y leaves half a pair unused
+  const size_t pairs = g.D == 2 ? (size_t)(g.T + 1) * g.N[0] * ((g.N[1] + 1) / 2 * 2) : 0;
+  const size_t n = nn > padded ? nn : padded;
+  return n > pairs ? n : pairs;
 }
 
 namespace {

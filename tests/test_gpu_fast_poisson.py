@@ -46,6 +46,20 @@ def test_fp64_poisson(T, N):
 def test_fp32_iteration(T, N):
     """The FP32 form inside one iteration of the mixed path, at the mixed path's one-step
     bound."""
+    one_iteration(T, N)
+
+
+# the kernel of small grids (x transforms and time solve in one block): its smallest, the
+# largest by (T + 1) N_x and the next, odd N_y (half a pair), prime and even T + 1, the
+# longest time axis, and short ones whose x axis just fits and does not fit its memory
+@pytest.mark.parametrize("T,N", [(1, [2, 2]), (1, [3, 5]), (16, [512, 5]), (16, [513, 4]), (37, [229, 7]),
+                                 (159, [54, 31]), (40, [31, 2]), (1, [4020, 3]), (1, [4032, 2])])
+def test_fp32_iteration_small(T, N):
+    """As above."""
+    one_iteration(T, N)
+
+
+def one_iteration(T, N):
     rng = np.random.default_rng(70 + T + sum(N))
     D, P = len(N), int(np.prod(N))
     r0, r1 = rng.random(P) + 0.05, rng.random(P) + 0.05
