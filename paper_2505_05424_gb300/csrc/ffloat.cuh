@@ -76,40 +76,6 @@ __device__ __forceinline__ float2 ff_mul(float2 a, float2 b) {
   return quick_two_sum(p, e);
 }
 
-// ff^2
-__device__ __forceinline__ float2 ff_sqr(float2 a) {
-  const float p = a.x * a.x;
-  float e = fmaf(a.x, a.x, -p);
-  e = fmaf(2.f * a.x, a.y, e);
-  return quick_two_sum(p, e);
-}
-
-// sqrt of a non-negative ff: FP32 root plus one Newton correction
-__device__ __forceinline__ float2 ff_sqrt(float2 a) {
-  if (!(a.x > 0.f)) return make_float2(0.f, 0.f);
-  const float s = sqrtf(a.x);
-  const float2 s2 = two_prod(s, s);
-  const float r = ((a.x - s2.x) - s2.y) + a.y;   // a - s^2, small
-  return quick_two_sum(s, r / (2.f * s));
-}
-
-// ff / ff (b != 0): FP32 quotient plus one correction
-__device__ __forceinline__ float2 ff_div(float2 a, float2 b) {
-  const float q1 = a.x / b.x;
-  const float2 p = ff_mul(make_float2(q1, 0.f), b);
-  const float2 r = ff_add(a, ff_neg(p));
-  const float q2 = r.x / b.x;
-  return quick_two_sum(q1, q2);
-}
-
-// ff / float
-__device__ __forceinline__ float2 ff_div_f(float2 a, float b) {
-  const float q1 = a.x / b;
-  const float2 p = two_prod(q1, b);
-  const float r = ((a.x - p.x) - p.y) + a.y;
-  return quick_two_sum(q1, r / b);
-}
-
 // a <= b for ff values
 __device__ __forceinline__ bool ff_le(float2 a, float2 b) {
   return a.x < b.x || (a.x == b.x && a.y <= b.y);
@@ -197,9 +163,6 @@ __device__ __forceinline__ ff2 two_prod2(float2 a, float2 b) {
   const float2 p = mul2(a, b);
   return ff2{p, make_float2(fmaf(a.x, b.x, -p.x), fmaf(a.y, b.y, -p.y))};
 }
-__device__ __forceinline__ ff2 ff2_neg(ff2 a) {
-  return ff2{make_float2(-a.h.x, -a.h.y), make_float2(-a.l.x, -a.l.y)};
-}
 // the two lanes of an ff2 as scalar two-floats, and back
 __device__ __forceinline__ float2 ff2_lane0(ff2 a) { return make_float2(a.h.x, a.l.x); }
 __device__ __forceinline__ float2 ff2_lane1(ff2 a) { return make_float2(a.h.y, a.l.y); }
@@ -210,7 +173,7 @@ __device__ __forceinline__ ff2 ff2_pack(float2 a, float2 b) {
 // ---- cheaper forms used by the fused cone kernel ----------------------------
 
 // ff / float given r ~ 1/b (a few ulps suffice): FP32 quotient a.x * r plus one
-// correction from the exact remainder, as ff_div_f without its two divisions.
+// correction from the exact remainder.
 __device__ __forceinline__ float2 ff_div_f_r(float2 a, float b, float r) {
   const float q1 = a.x * r;
   const float2 p = two_prod(q1, b);
