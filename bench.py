@@ -207,7 +207,7 @@ def algorithmic_bytes(name: str, D: int, T: int, N: int, prec: str) -> float:
 # the named workload, with the SHA-256 prefix of the kernel source it was taken on:
 # the figure is reported only while that source is unchanged (else traffic = null).
 NCU_TRAFFIC = {("fused_cone_update", "mix256", "mixed"):
-               (603.940096e6 + 472.039424e6, "k_fused2d.cu", "1800e29b4d940626")}
+               (542.629888e6 + 459.951872e6, "k_fused2d.cu", "97325e93ce221f64")}
 
 
 def stored_traffic(kernel: str, workload: str, prec: str):
@@ -350,23 +350,14 @@ def run_ours(args):
     dname, (dms, dn) = dom[0], dom[1]
     per_launch_ms = dms / max(dn, 1)
     abytes = algorithmic_bytes(dname, spec.D, spec.T, spec.N, args.prec)
-    if dname in ("dct_axis", "dct_tcgen05"):
-        M = spec.N
-        flops = 2.0 * M * (spec.T + 1) * spec.N ** spec.D * (3 if dname == "dct_tcgen05" else 1)
-        tf32_peak = peaks.get("bf16_tflops_sustained", 1700.0) * (1.1 / 2.25)
-        achieved = flops / (per_launch_ms / 1e3) / 1e12
-        roof = {"bound": "tensor", "achieved": achieved, "peak": tf32_peak, "unit": "TFLOP/s",
-                "frac": achieved / tf32_peak, "traffic": None, "kernel": dname,
-                "peak_source": f"{peak_src} bf16 sustained x tf32/bf16 nominal ratio 1.1/2.25"}
-    else:
-        achieved = abytes / (per_launch_ms / 1e3) / 1e9
-        hbm = peaks.get("hbm_gbs", 6800.0)
-        traffic, traffic_src = stored_traffic(dname, wl, args.prec)
-        roof = {"bound": "hbm", "achieved": round(achieved, 1), "peak": hbm, "unit": "GB/s",
-                "frac": round(achieved / hbm, 4), "traffic": traffic, "traffic_source": traffic_src,
-                "kernel": dname,
-                "per_launch_ms": round(per_launch_ms, 5), "algorithmic_bytes": abytes,
-                "peak_source": f"{peak_src} (of measured copy bandwidth)" if peak_src == "measured" else peak_src}
+    achieved = abytes / (per_launch_ms / 1e3) / 1e9
+    hbm = peaks.get("hbm_gbs", 6800.0)
+    traffic, traffic_src = stored_traffic(dname, wl, args.prec)
+    roof = {"bound": "hbm", "achieved": round(achieved, 1), "peak": hbm, "unit": "GB/s",
+            "frac": round(achieved / hbm, 4), "traffic": traffic, "traffic_source": traffic_src,
+            "kernel": dname,
+            "per_launch_ms": round(per_launch_ms, 5), "algorithmic_bytes": abytes,
+            "peak_source": f"{peak_src} (of measured copy bandwidth)" if peak_src == "measured" else peak_src}
 
     kernels = {k: {"ms_total": round(v[0], 3), "launches": v[1],
                    "ms_per_launch": round(v[0] / max(v[1], 1), 5),

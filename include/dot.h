@@ -55,9 +55,9 @@ typedef struct {
 
 typedef enum {
   DOT_FP64 = 0,   /* every field and every operation in FP64 (the reference path) */
-  DOT_MIXED = 1   /* FP32 stencils/projection, 3xTF32 DCT GEMMs on the tensor cores,
-                     two-float (48-bit) multipliers and potential, FP64 reductions,
-                     one refinement step of the Poisson solve per iteration */
+  DOT_MIXED = 1   /* FP32 stencils/projection and fast cosine transforms, two-float
+                     (48-bit) multipliers and potential, FP64 reductions; each iteration's
+                     Poisson solve corrects the exact residual of the last potential */
 } dot_precision;
 
 typedef struct {

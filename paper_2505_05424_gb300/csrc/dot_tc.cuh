@@ -1,4 +1,4 @@
-// dot_tc.cuh -- tensor-core (tcgen05) DCT pass of the mixed-path Poisson solve.
+// dot_tc.cuh -- tensor-core (tcgen05) DCT pass of dot_poisson on a mixed context.
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>

@@ -1,4 +1,4 @@
-// k_dct_tc.cu -- one DCT pass of the mixed-path Poisson solve on the 5th-generation
+// k_dct_tc.cu -- one DCT pass of the mixed Poisson operator (dot_poisson) on the 5th-generation
 // tensor cores (tcgen05, TMEM accumulators, TMA operand staging), in 3xTF32
 // split precision with FP32 accumulation.
 //

@@ -25,8 +25,8 @@
 // two-float face right-hand sides and multiplier updates (ffloat.cuh).
 //
 // Bound by instruction issue and by the latency of a time step (two barriers, a
-// dependent chain of some 100 FP operations): on 256^2 x 64 about 150 M warp
-// instructions, 49% issue, 0.6 of the HBM bandwidth on its 1,026 MB, 251 us per launch;
+// dependent chain of some 100 FP operations): on 256^2 x 64 136 M warp
+// instructions, 46% issue, 0.6 of the HBM bandwidth on its 1,026 MB, 251 us per launch;
 // 128^2 x 32 47.5 us, 32^2 x 16 10.4 us.  The form before it (a thread per halo cone,
 // faces dealt out in rounds, beta by TMA in component planes, 80 registers at two CTAs per
 // SM, fixed 16-time chunks): 245 M instructions, 357, 62 and 19.6 us; and for odd N_y,

@@ -1,5 +1,6 @@
-// k_poisson_f32.cu -- the mixed-path Poisson solve A^*A phi = b on rge(A^*)
-// (Sec. 4, phi-subproblem of Algorithm 2): orthonormal DCT-II along every axis,
+// k_poisson_f32.cu -- the mixed-path Poisson operator A^*A phi = b on rge(A^*) with dense
+// transforms (Sec. 4, phi-subproblem of Algorithm 2; dot_poisson.  The iterations run
+// k_fft.cu where the axes fit it): orthonormal DCT-II along every axis,
 // division by the Neumann eigenvalues with the zero mode set to 0, DCT-III back.
 //
 // Data flow ("rotated" passes): every spatial pass transforms the innermost axis

@@ -1,10 +1,10 @@
 // k_poisson_f64.cu -- dense FP64 Poisson solve A^*A phi = b on rge(A^*) (Sec. 4: the
 // phi-subproblem of Algorithm 2), for the grids whose axes do not fit the fast solve's
-// shared memory (k_fft.cu: a spatial axis beyond 2,816 points or T beyond 219).  A^*A is the Neumann Laplacian of the node
-// grid; the orthonormal DCT-II along every axis diagonalises it with eigenvalues
+// shared memory (k_fft.cu: a spatial axis beyond 2,816 points or T beyond 219).  A^*A is the Neumann
+// Laplacian of the node grid; the orthonormal DCT-II along every axis diagonalises it with eigenvalues
 // sum_a (4/h_a^2) sin^2(pi k_a / (2 M_a)).  Each per-axis transform is a dense
 // GEMM  Y[o][k][i] = sum_m C[k][m] X[o][m][i]  run on the FP64 tensor path
-// (mma.sync m8n8k4 .f64, which GB300 executes about 4x faster than FP64 FMA).
+// (mma.sync m8n8k4 .f64).
 #include "dot_internal.cuh"
 
 namespace dot {
