@@ -165,15 +165,16 @@ void launch_assemble_solve_mx(const Geo& g, int G, const MxFields& f, const MxPo
 // (nullable): per-block sums of |z - BFq - d|^2 written by the fused kernel,
 // nsocp per slot; when given, they replace the z-based term.
 void launch_kkt_mx(const Geo& g, int G, const MxFields& f, double* partials, double* out,
-                   const double* socp_part, int nsocp, cudaStream_t s, LaunchCounter lc);
+                   const float2* socp_part, int nsocp, cudaStream_t s, LaunchCounter lc);
 
 // Fused lines 3-6 for D = 2 (k_fused2d.cu) for every active slot: reads q, alpha,
 // beta of f, writes those of fn and the next iteration's lines 1-2 residual into f.r
 // (see launch_solve_residual_mx); phi, somega, sp from f.  socp_part:
-// fused2d_partials(g, G) doubles per slot (the tiling depends on the batch size).
+// fused2d_partials(g) entries per slot (the tiling depends on the batch size, these sums
+// and their order do not).
 bool fused2d_supported(const Geo& g);
-long long fused2d_partials(const Geo& g, int G);
-void launch_fused2d(const Geo& g, int G, const MxFields& f, const MxFields& fn, double* socp_part,
+long long fused2d_partials(const Geo& g);
+void launch_fused2d(const Geo& g, int G, const MxFields& f, const MxFields& fn, float2* socp_part,
                     cudaStream_t s, LaunchCounter lc);
 // Fused lines 3-6 for D = 3 (k_fused3d.cu) for one solve: z and q_0, alpha_0 by one pass
 // over the cones, then q_d, alpha_d, beta and the next iteration's lines 1-2 residual (f.r)

@@ -81,8 +81,9 @@ struct FusedArgs {
   int G;               // slots
   int ntx, nty;        // tiles along x and y
   int unit, nunit;     // time nodes per work unit, units per tile
+  int run;             // time nodes per partial sum (divides unit)
   const SlotParam* sp;
-  double* socp_part;   // per work unit: sum of |z - B F q^{k+1} - d|^2
+  float2* socp_part;   // [slot][run][y tile][x]: sums of |z - B F q^{k+1} - d|^2 over 32 cells of a row
   // the next iteration's lines 1-2 residual
   // r = A^*(q^{k+1} - alpha^{k+1}/sigma) - c/sigma - A^*A phi^{k+1} at every node
   float* r;
@@ -102,12 +103,25 @@ __device__ __forceinline__ float4 f4_of(ff2 b) { return make_float4(b.h.x, b.h.y
 
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
 
-// One segment: time nodes [ta, tb) of one tile of one slot.  *pend: the work unit of
-// the segment before whose sums wait in wsum (null: none).  Element indices stay below
+// Sum of a two-float over the warp, unnormalised.  (A 32-lane FP64 addition occupies an SM
+// for 16 cycles; with FP64 shuffles here 300 iterations on 128^2 x 32 take 28.7 ms, not 26.4,
+// and 32 served 64^2 x 32 solves 114 ms, not 107.)
+__device__ __forceinline__ float2 warp_sum_ff(float2 v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float2 u = f2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
+    const float2 e = two_sum(v.x, u.x);
+    v = f2(e.x, e.y + (v.y + u.y));
+  }
+  return v;
+}
+
+// One segment: time nodes [ta, tb) of one tile of one slot.  socp_tile: the slot's partial
+// sums of the tile's rows over the first run of time nodes.  Element indices stay below
 // 2^31 over all slots of a batch (dot_server.cu bounds the batch).
 template <int TX, bool MASKED>
-__device__ __forceinline__ void segment(const Geo& g, const FusedArgs& a, unsigned char* sm, double* wsum, int slot,
-                                        int x0, int y0, int ta, int tb, double* socp_tile, double** pend) {
+__device__ __forceinline__ void segment(const Geo& g, const FusedArgs& a, unsigned char* sm, int slot, int x0, int y0,
+                                        int ta, int tb, float2* socp_tile) {
   using L = Tile<TX>;
   constexpr int kThreads = L::kThreads;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -219,8 +233,8 @@ __device__ __forceinline__ void segment(const Geo& g, const FusedArgs& a, unsign
   float2 w0c = z2, w0p = z2;                // alpha_0/sigma + A_0 phi - q_0 of cones t and t - 1 (unnormalised)
   float2 socp = z2;
   const float2 ts2 = f2(ts, ts);
-  int left = a.unit;                        // time nodes to the end of the work unit
-  double* entry = socp_tile + ta / a.unit;
+  int left = a.run;                         // time nodes to the end of the partial sum
+  float2* entry = socp_tile + (long long)(ta / a.run) * a.nty * N0 + warp;
 
   for (int t = tstart; t < tb; ++t, i += P) {
     const int lev = (t & 1) * kThreads;
@@ -278,14 +292,6 @@ __device__ __forceinline__ void segment(const Geo& g, const FusedArgs& a, unsign
     }
     sph[tid] = ph_t;
     __syncthreads();
-    if (*pend) {                            // the unit that ended at the last step
-      if (tid == 0) {
-        double b = 0.0;
-        for (int w = 0; w < TX; ++w) b += wsum[w];
-        **pend = b;
-      }
-      *pend = nullptr;
-    }
     float2 qo = z2;
     ff2 wo{z2, z2};
     // ---------------- B: the column's faces on time node t ----------------
@@ -403,16 +409,15 @@ __device__ __forceinline__ void segment(const Geo& g, const FusedArgs& a, unsign
         a.r[i] = acc.h + acc.c;
       }
     }
-    // the sum of squared beta increments of a work unit that ends with node t
+    // the squared beta increments of a row's 32 cells over a run that ends with node t
     if (t >= ta && (--left == 0 || t == T)) {
       if (owner) {
-        double v = (double)socp.x + (double)socp.y;
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) wsum[warp] = v;
+        const float2 v = warp_sum_ff(two_sum(socp.x, socp.y));
+        if (lane == 0 && x < N0) *entry = v;
         socp = z2;
       }
-      *pend = entry++;
-      left = a.unit;
+      entry += (long long)a.nty * N0;
+      left = a.run;
     }
     w0p = w0c;
     zp3 = zc[3];
@@ -436,7 +441,6 @@ template <int TX, bool MASKED>
 __global__ void __launch_bounds__(Tile<TX>::kThreads, 1) k_fused2d(const __grid_constant__ Geo g,
                                                                   const __grid_constant__ FusedArgs a) {
   extern __shared__ __align__(16) unsigned char sm[];
-  __shared__ double wsum[TX];
   __shared__ short act[256];
   __shared__ int nact_s;
   const int tid = threadIdx.x;
@@ -451,26 +455,19 @@ __global__ void __launch_bounds__(Tile<TX>::kThreads, 1) k_fused2d(const __grid_
     if (tid == 0) nact_s = n;
   }
   __syncthreads();
-  const int ntile = a.ntx * a.nty, nunit = a.nunit;
+  const int ntile = a.ntx * a.nty, nunit = a.nunit, nrun = (g.T + a.run) / a.run;
   const long long total = (long long)nact_s * ntile * nunit;
   long long k = total * blockIdx.x / gridDim.x;
   const long long kend = total * (blockIdx.x + 1) / gridDim.x;
-  double* pend = nullptr;
   while (k < kend) {
     const int tl = (int)(k / nunit), u0 = (int)(k - (long long)tl * nunit);
     const int u1 = (int)min((long long)nunit, u0 + (kend - k));
     const int s = tl / ntile, tile = tl - s * ntile;
     const int ty = tile / a.ntx, tx = tile - ty * a.ntx;
     const int slot = act[s];
-    segment<TX, MASKED>(g, a, sm, wsum, slot, tx * TX, ty * TY, u0 * a.unit, min(g.T + 1, u1 * a.unit),
-                        a.socp_part + ((long long)slot * ntile + tile) * nunit, &pend);
+    segment<TX, MASKED>(g, a, sm, slot, tx * TX, ty * TY, u0 * a.unit, min(g.T + 1, u1 * a.unit),
+                        a.socp_part + ((long long)slot * nrun * a.nty + ty) * g.N[0] + tx * TX);
     k += u1 - u0;
-  }
-  __syncthreads();
-  if (pend && tid == 0) {
-    double b = 0.0;
-    for (int w = 0; w < TX; ++w) b += wsum[w];
-    *pend = b;
   }
 }
 
@@ -495,10 +492,23 @@ int rows_of(const Geo& g, int G) {
   return best;
 }
 
-// Time nodes per work unit: about sixteen units per SM, at most eight.
-int unit_of(const Geo& g, int G) {
+// Time nodes to hand out at once: about sixteen units per SM, at most eight.
+int share_of(const Geo& g, int G) {
   const long long u = (long long)G * ntiles(g, rows_of(g, G)) * (g.T + 1) / (kSMs * 16);
   return (int)(u < 1 ? 1 : u > 8 ? 8 : u);
+}
+
+// Time nodes per partial sum of the squared beta increments: FP32 over a run of one
+// cell's nodes, two-float over a row's 32 cells, FP64 from there.  Of the grid alone, as the order of these sums may not
+// depend on the batch: they enter the penalty rule, and a served solve takes the steps of
+// a solve alone.
+int run_of(const Geo& g) { return share_of(g, 1); }
+int runs(const Geo& g) { return (g.T + run_of(g)) / run_of(g); }
+
+// Time nodes per work unit: whole runs.
+int unit_of(const Geo& g, int G) {
+  const int r = run_of(g), u = share_of(g, G) / r * r;
+  return u > r ? u : r;
 }
 
 template <int TX, bool MASKED>
@@ -512,12 +522,9 @@ void launch(const Geo& g, const FusedArgs& a, int nb, cudaStream_t s) {
 
 bool fused2d_supported(const Geo& g) { return g.D == 2; }
 
-long long fused2d_partials(const Geo& g, int G) {
-  const int u = unit_of(g, G);
-  return (long long)ntiles(g, rows_of(g, G)) * ((g.T + u) / u);
-}
+long long fused2d_partials(const Geo& g) { return (long long)runs(g) * ((g.N[1] + TY - 1) / TY) * g.N[0]; }
 
-void launch_fused2d(const Geo& g, int G, const MxFields& f, const MxFields& fn, double* socp_part, cudaStream_t s,
+void launch_fused2d(const Geo& g, int G, const MxFields& f, const MxFields& fn, float2* socp_part, cudaStream_t s,
                     LaunchCounter lc) {
   FusedArgs a;
   for (int d = 0; d < 3; ++d) {
@@ -536,6 +543,7 @@ void launch_fused2d(const Geo& g, int G, const MxFields& f, const MxFields& fn, 
   a.nty = (g.N[1] + TY - 1) / TY;
   a.unit = unit_of(g, G);
   a.nunit = (g.T + a.unit) / a.unit;
+  a.run = run_of(g);
   a.sp = f.sp;
   a.socp_part = socp_part;
   a.r = f.r;

@@ -460,7 +460,7 @@ __device__ __forceinline__ float2 kkt_div(const Geo& g, const MxFields& f, float
 template <int D>
 __global__ void __launch_bounds__(kThreads, D == 2 ? 4 : 3) k_kkt(const __grid_constant__ Geo g,
                                                      const __grid_constant__ MxFields fb, double* partials_all,
-                                                     const double* socp_all, int nsocp) {
+                                                     const float2* socp_all, int nsocp) {
   const int slot = blockIdx.y, kind = blockIdx.z;
   if (!fb.sp[slot].active) return;
   const MxFields f = slot_view(fb, g, slot);
@@ -511,7 +511,7 @@ __global__ void __launch_bounds__(kThreads, D == 2 ? 4 : 3) k_kkt(const __grid_c
       cphi += c * ff_to_double(f.phi[t * P + p]);
     }
     if (socp_all)
-      for (int i = i0; i < nsocp; i += stride) socp += socp_all[(long long)slot * nsocp + i];
+      for (int i = i0; i < nsocp; i += stride) socp += ff_to_double(socp_all[(long long)slot * nsocp + i]);
     constexpr int w[3] = {R_DUALRES, R_SOCP, R_CPHI};
     const double v[3] = {(double)acc[R_DUALRES] + dres, socp, cphi};
     block_reduce_store<kThreads>(v, w, partials, rows, row);
@@ -574,7 +574,7 @@ void assemble_solve_tmpl(const Geo& g, int G, const MxFields& f, const MxPoisson
 
 template <int D>
 void launch_kkt_tmpl(const Geo& g, int G, const MxFields& f, double* partials, double* out,
-                     const double* socp_part, int nsocp, cudaStream_t s, LaunchCounter lc) {
+                     const float2* socp_part, int nsocp, cudaStream_t s, LaunchCounter lc) {
   const int kb = kkt_blocks(g);
   k_kkt<D><<<dim3(kb, G, kkt_kinds(D)), kThreads, 0, s>>>(g, f, partials, socp_part, nsocp);
   k_kkt_final<<<dim3(G, R_NSLOTS), 128, 0, s>>>(g, f.sp, partials, kkt_kinds(D) * kb, out);
@@ -608,7 +608,7 @@ void launch_assemble_solve_mx(const Geo& g, int G, const MxFields& f, const MxPo
 }
 
 void launch_kkt_mx(const Geo& g, int G, const MxFields& f, double* partials, double* out,
-                   const double* socp_part, int nsocp, cudaStream_t s, LaunchCounter lc) {
+                   const float2* socp_part, int nsocp, cudaStream_t s, LaunchCounter lc) {
   if (g.D == 2) launch_kkt_tmpl<2>(g, G, f, partials, out, socp_part, nsocp, s, lc);
   else launch_kkt_tmpl<3>(g, G, f, partials, out, socp_part, nsocp, s, lc);
 }

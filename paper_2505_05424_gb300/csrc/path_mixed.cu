@@ -16,7 +16,7 @@ namespace dot {
 struct MixedBatch::Buffers {
   MxFields f;        // set 0 of (q, alpha, beta) + the shared fields
   MxFields f2;       // set 1 of (q, alpha, beta) (fused D = 2 path), shared fields as f
-  double* socp;      // fused-kernel partial sums of |z - BFq - d|^2, per slot
+  float2* socp;      // fused-kernel partial sums of |z - BFq - d|^2, per slot
   float2* phi_op;
   float2* c0;
   float2* c1;
@@ -61,7 +61,7 @@ void carve(const Geo& g, int G, bool masks, Carver& cv, MixedBatch::Buffers* B) 
   }
   if (fused2d_supported(g)) {
     B->f.z = nullptr;                       // z never leaves the fused kernel
-    B->socp = cv.take<double>(Gs * fused2d_partials(g, G));
+    B->socp = cv.take<float2>(Gs * fused2d_partials(g));
   } else {
     B->f.z = cv.take<float>(Gs * g.K * n0);
     B->socp = nullptr;
@@ -288,7 +288,7 @@ cudaError_t MixedBatch::zero_slot(int b, cudaStream_t s) {
   }
   if (e == cudaSuccess && B.f.z) e = cudaMemsetAsync(B.f.z + b * g_.K * n0, 0, (size_t)g_.K * n0 * 4, s);
   if (e == cudaSuccess && B.socp)
-    e = cudaMemsetAsync(B.socp + b * fused2d_partials(g_, G_), 0, (size_t)fused2d_partials(g_, G_) * sizeof(double), s);
+    e = cudaMemsetAsync(B.socp + b * fused2d_partials(g_), 0, (size_t)fused2d_partials(g_) * sizeof(float2), s);
   return e;
 }
 
@@ -418,7 +418,7 @@ void MixedBatch::kkt(cudaStream_t s, LaunchCounter lc) {
   // every slot whose assemble flag is set (and reuses f.r for the others)
   r_valid_ = false;
   launch_kkt_mx(g_, G_, cur(), B_->partials, B_->red, fused_ ? B_->socp : nullptr,
-                fused_ ? (int)fused2d_partials(g_, G_) : 0, s, lc);
+                fused_ ? (int)fused2d_partials(g_) : 0, s, lc);
 }
 
 namespace {
