@@ -11,6 +11,7 @@
 #include <string>
 #include <vector>
 
+#include "dot_hostcopy.cuh"
 #include "dot_mixed.cuh"
 #include "dot_paths.cuh"
 
@@ -93,6 +94,7 @@ class MixedBatch {
   std::vector<SlotParam> hp_;
   std::vector<double> hs_;   // sigma per slot (host)
   std::vector<std::vector<float>> hT_, hF_;
+  HostStage stage_;
 
   const MxFields& cur() const;
   const MxFields& other() const;

@@ -59,6 +59,11 @@ __host__ __device__ inline void pair_of(int K, int j, int* pair, int* lane) {
     *lane = (j - 9) % 2;
   }
 }
+// The components of a pair, lane 0 first.
+inline void pair_members(int K, int pair, int* j0, int* j1) {
+  *j0 = pair <= 4 ? pair : 9 + 2 * (pair - 5);
+  *j1 = pair == 0 ? K - 1 : pair <= 4 ? pair + 4 : *j0 + 1;
+}
 // Index (in floats) of component j's high part of beta at cone i of n0 (its low part is two
 // floats further), and of z.
 __host__ __device__ inline long long beta_at(int K, int j, long long i, long long n0) {

@@ -119,6 +119,7 @@ class PathF64 : public Path {
       B_.dct.C[a] = B_.Cbuf[a];
       B_.dct.lam[a] = B_.lbuf[a];
     }
+    stage_.reserve(((size_t)g_.T + (size_t)(g_.D + 1) * (g_.T + 1)) * P * sizeof(double), HOST_F64);   // the fields
     fast_ = fast_poisson_supported(g_, sizeof(double));
     std::memset(&fp_, 0, sizeof(fp_));
     fp_.w1 = B_.f.w1;
@@ -159,7 +160,7 @@ class PathF64 : public Path {
       m += natural_face_count(g_, fam);
     }
     if (phi) parts.push_back({B_.f.phi, phi, nn, nn, 1, HOST_F64, 1.0, 1.0});
-    const cudaError_t e = read_to_host(parts, s);
+    const cudaError_t e = read_to_host(parts, stage_, s);
     if (e != cudaSuccess) { *err = std::string("read_fields: ") + cudaGetErrorString(e); return DOT_ECUDA; }
     return DOT_OK;
   }
@@ -260,6 +261,7 @@ class PathF64 : public Path {
   std::vector<double> hom_, hsom_;
   std::vector<std::vector<double>> hC_, hl_, hf_;
   FastPoisson<double> fp_;
+  HostStage stage_;
   bool fast_ = false;
 };
 

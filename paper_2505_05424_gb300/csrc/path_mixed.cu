@@ -9,7 +9,6 @@
 #include <cstring>
 
 #include "dot_batch.cuh"
-#include "dot_hostcopy.cuh"
 
 namespace dot {
 
@@ -190,6 +189,7 @@ int MixedBatch::init(char* ws, size_t bytes, cudaStream_t s, std::string* err) {
     f->somega = slot_masks_ ? B.somega : nullptr;
     f->sp = B.params;
   }
+  stage_.reserve(((size_t)g_.T + (size_t)(g_.D + 1) * (g_.T + 1)) * g_.P * 8, HOST_FF);   // the fields
   red_ = B.red;
   err_ = B.err;
   dparams_ = B.params;
@@ -452,7 +452,7 @@ int MixedBatch::read_fields(int b, double* rho, double* m, double* phi, cudaStre
     m += natural_face_count(g_, fam);
   }
   if (phi) parts.push_back({fc.phi, phi, nn, nn, 1, HOST_FF, 1.0, 1.0});
-  const cudaError_t e = read_to_host(parts, s);
+  const cudaError_t e = read_to_host(parts, stage_, s);
   if (e != cudaSuccess) { *err = std::string("read_fields: ") + cudaGetErrorString(e); return DOT_ECUDA; }
   return DOT_OK;
 }
@@ -472,12 +472,8 @@ int MixedBatch::read_state(int b, double* q, double* al, double* beta, cudaStrea
     if (al) parts.push_back({fc.al[fam], al + off, w, p, h, HOST_FF, sig, 1.0});
     off += (size_t)natural_face_count(g_, fam);
   }
-  for (int j = 0; beta && j < g_.K; ++j) {
-    const long long o = beta_at(g_.K, j, 0, (long long)n0);
-    parts.push_back({reinterpret_cast<const float*>(fc.beta) + o / 4 * 4, beta + j * n0, n0, n0, 1,
-                     o % 4 ? HOST_LANE1 : HOST_LANE0, sig, 1.0});
-  }
-  const cudaError_t e = read_to_host(parts, s);
+  if (beta) parts.push_back({fc.beta, beta, n0, n0, (size_t)g_.K / 2, HOST_PAIRS, sig, 1.0});
+  const cudaError_t e = read_to_host(parts, stage_, s);
   if (e != cudaSuccess) { *err = std::string("read_state: ") + cudaGetErrorString(e); return DOT_ECUDA; }
   return DOT_OK;
 }
