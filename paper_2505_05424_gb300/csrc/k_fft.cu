@@ -255,44 +255,76 @@ __device__ __forceinline__ void stage(const Q& np, const V* src, V* dst, const V
 }
 
 // A stage of any odd radix r: outputs k and r - k share their sums over the conjugate
-// input pairs, sum_j (x_j + x_{r-j}) cos and (x_j - x_{r-j}) sin.
-template <bool INV, class Q, class V>
-__device__ __forceinline__ void stage_any(const Q& np, const V* src, V* dst, const V* tw, int N, int r, int s,
-                                          FastDiv fs, FastDiv fr) {
+// input pairs, sum_j (x_j + x_{r-j}) cos and (x_j - x_{r-j}) sin.  The pairs are formed in
+// their places first; a thread then runs over them for KB values of k, so that a pair is
+// read once for KB outputs and their conjugates.
+template <int KB, bool INV, class Q, class V>
+__device__ __forceinline__ void stage_any(const Q& np, V* src, V* dst, const V* tw, int N, int r, int s, FastDiv fs,
+                                          FastDiv fr) {
   const int kPitch = np.pitch();
-  const int nb = N / r, hk = (r + 1) / 2;
-  for (int e = threadIdx.x; e < nb * hk * np.count(); e += Q::kThreads) {
+  const int nb = N / r, hk = (r + 1) / 2, step = nb * kPitch;
+  for (int e = threadIdx.x; e < nb * (hk - 1) * np.count(); e += Q::kThreads) {
+    int pr;
+    const int bj = np.split(e, &pr);
+    const int j = (int)fdiv((unsigned)bj, fr), b = bj - j * nb;
+    V* p = src + (b + nb * (j + 1)) * kPitch + pr;
+    V* q = src + (b + nb * (r - 1 - j)) * kPitch + pr;
+    const V a = *p, c = *q;
+    *p = cadd(a, c);
+    *q = rot<!INV>(csub(a, c));   // i (x_j - x_{r-j}) forward: times sin it adds to the sum
+  }
+  __syncthreads();
+  const int nk = (hk + KB - 1) / KB;
+  for (int e = threadIdx.x; e < nb * nk * np.count(); e += Q::kThreads) {
     int pr;
     const int bk = np.split(e, &pr);
-    const int k = (int)fdiv((unsigned)bk, fr), b = bk - k * nb;
+    const int kb = (int)fdiv((unsigned)bk, fr), b = bk - kb * nb;
     const int p = (int)fdiv((unsigned)b, fs), q = b - p * s;
     const V* x = src + b * kPitch + pr;
-    V* o = dst + (q + s * r * p) * kPitch + pr;
-    V re = x[0], im = mk<V>(re.x - re.x, re.y - re.y);
-    int m = 0;   // j k mod r
-    for (int j = 1; j < hk; ++j) {
-      m += k;
-      if (m >= r) m -= r;
-      const V w = tw[m * nb];
-      const V a = x[nb * j * kPitch], c = x[nb * (r - j) * kPitch];
-      const V sm = cadd(a, c), df = csub(a, c);
-      re = mk<V>(re.x + sm.x * w.x, re.y + sm.y * w.x);
-      // i w.y df, w.y = -sin (forward)
-      im = INV ? mk<V>(im.x + df.y * w.y, im.y - df.x * w.y) : mk<V>(im.x - df.y * w.y, im.y + df.x * w.y);
+    const V *xs = x, *xd = x + r * step;
+    V re[KB], im[KB];
+    int m[KB], dm[KB];                     // j k mod r, in units of N / r
+    re[0] = x[0];
+    im[0] = mk<V>(re[0].x - re[0].x, re[0].y - re[0].y);
+#pragma unroll
+    for (int i = 0; i < KB; ++i) {
+      re[i] = re[0];
+      im[i] = im[0];
+      m[i] = 0;
+      dm[i] = min(kb * KB + i, hk - 1) * nb;
     }
-    V y = cadd(re, im);
-    if (k && nb > s) y = cmulw<INV>(y, tw[s * p * k]);
-    o[s * k * kPitch] = y;
-    if (k) {
-      V z = csub(re, im);
-      if (nb > s) z = cmulw<INV>(z, tw[s * p * (r - k)]);
-      o[s * (r - k) * kPitch] = z;
+    for (int j = 1; j < hk; ++j) {
+      xs += step;
+      xd -= step;
+      const V sm = *xs, df = *xd;
+#pragma unroll
+      for (int i = 0; i < KB; ++i) {
+        m[i] += dm[i];
+        if (m[i] >= N) m[i] -= N;
+        const V w = tw[m[i]];
+        re[i] = mk<V>(re[i].x + sm.x * w.x, re[i].y + sm.y * w.x);
+        im[i] = mk<V>(im[i].x + df.x * w.y, im[i].y + df.y * w.y);   // w.y = -sin (forward)
+      }
+    }
+    V* o = dst + (q + s * r * p) * kPitch + pr;
+#pragma unroll
+    for (int i = 0; i < KB; ++i) {
+      const int k = kb * KB + i;
+      if (k >= hk) break;
+      V y = cadd(re[i], im[i]);
+      if (k && nb > s) y = cmulw<INV>(y, tw[s * p * k]);
+      o[s * k * kPitch] = y;
+      if (k) {
+        V z = csub(re[i], im[i]);
+        if (nb > s) z = cmulw<INV>(z, tw[s * p * (r - k)]);
+        o[s * (r - k) * kPitch] = z;
+      }
     }
   }
 }
 
 // All stages; returns the buffer that holds the result.
-template <bool INV, class Q, class V>
+template <bool INV, int KB = 2, class Q, class V>
 __device__ __forceinline__ V* transform(const Q& np, V* a, V* b, const V* tw, const FftPlan& pl) {
   int s = 1;
   for (int i = 0; i < pl.nst; ++i) {
@@ -303,7 +335,7 @@ __device__ __forceinline__ V* transform(const Q& np, V* a, V* b, const V* tw, co
       case 2: stage<2, INV>(np, a, b, tw, pl.N, s, pl.fs[i]); break;
       case 3: stage<3, INV>(np, a, b, tw, pl.N, s, pl.fs[i]); break;
       case 5: stage<5, INV>(np, a, b, tw, pl.N, s, pl.fs[i]); break;
-      default: stage_any<INV>(np, a, b, tw, pl.N, r, s, pl.fs[i], pl.fr[i]); break;
+      default: stage_any<KB, INV>(np, a, b, tw, pl.N, r, s, pl.fs[i], pl.fr[i]); break;
     }
     __syncthreads();
     V* t = a;
@@ -436,8 +468,9 @@ struct Columns {
   }
 };
 
-// The DCT-II (INV false) or DCT-III of NP pairs of sequences of any length.
-template <class R, int NP, bool INV>
+// The DCT-II (INV false) or DCT-III of NP pairs of sequences of any length; KB as in
+// stage_any.
+template <class R, int NP, bool INV, int KB>
 __global__ void __launch_bounds__(kThreads) k_dct_any(const __grid_constant__ FftArgs<R> a) {
   using V = typename Vec2<R>::type;
   constexpr int kPitch = NP + 1;
@@ -469,7 +502,7 @@ __global__ void __launch_bounds__(kThreads) k_dct_any(const __grid_constant__ Ff
       }
     }
     __syncthreads();
-    const V* Z = transform<INV>(FixedPairs<NP>(), A, B, tw, a.plan);
+    const V* Z = transform<INV, KB>(FixedPairs<NP>(), A, B, tw, a.plan);
     if (!c.ok) return;
     if (!INV) {
 #pragma unroll 2
@@ -516,7 +549,7 @@ __global__ void __launch_bounds__(kThreads) k_dct_any(const __grid_constant__ Ff
       }
       __syncthreads();
     }
-    const V* Z = transform<INV>(FixedPairs<NP>(), A, B, tw, a.plan);
+    const V* Z = transform<INV, KB>(FixedPairs<NP>(), A, B, tw, a.plan);
     if (!INV && a.rot) {
       for (int e = threadIdx.x; e < NP * nk; e += kThreads) rot_store(a, p0 + e % NP, e / NP, rotf, Z, kPitch, e % NP);
       return;
@@ -1069,11 +1102,28 @@ template <class R> constexpr int time_threads() { return sizeof(R) == 4 ? 128 : 
 template <class R>
 size_t fft_smem(int N, int NP) { return (size_t)(2 * N * (NP + 1) + N) * 2 * sizeof(R); }
 
+template <class R, int NP, bool INV, int KB>
+void launch_np_kb(const FftArgs<R>& a, cudaStream_t s) {
+  static std::atomic<unsigned long long> done{0};
+  smem_optin((const void*)k_dct_any<R, NP, INV, KB>, kMaxSmem, &done);
+  k_dct_any<R, NP, INV, KB><<<(unsigned)((a.npair + NP - 1) / NP), kThreads, fft_smem<R>(a.plan.N, NP), s>>>(a);
+}
+// Outputs per thread of a stage with an odd radix r: four in FP32 from r = 64, where every
+// thread then has work, else two; in a kernel of their own, as four take registers that
+// cost every other axis CTAs.  An iteration with two and with four: 508^2 x 32 1,156 and
+// 1,054 us, 1004^2 x 32 5,473 and 4,819 (one output at a time, its pairs formed anew: 1,398
+// and 7,297; before the fast transforms 1,174 and 5,112), 61^3 x 16 719 and 760,
+// 127^2 x 32 109 and 120; FP64 2801 x 2 x 2 3,956 and 4,490.
 template <class R, int NP, bool INV>
 void launch_np(const FftArgs<R>& a, cudaStream_t s) {
-  static std::atomic<unsigned long long> done{0};
-  smem_optin((const void*)k_dct_any<R, NP, INV>, kMaxSmem, &done);
-  k_dct_any<R, NP, INV><<<(unsigned)((a.npair + NP - 1) / NP), kThreads, fft_smem<R>(a.plan.N, NP), s>>>(a);
+  const int r = a.plan.rad[a.plan.nst - 1];   // the largest odd prime factor, if there is one
+  if constexpr (sizeof(R) == 4) {
+    if (r >= 64 && a.plan.N / r * ((r + 7) / 8) * NP >= kThreads) {
+      launch_np_kb<R, NP, INV, 4>(a, s);
+      return;
+    }
+  }
+  launch_np_kb<R, NP, INV, 2>(a, s);
 }
 
 template <class R, int N, int NP, bool INV, bool ROWS>
