@@ -271,9 +271,10 @@ __device__ __forceinline__ void acc2_add_mul(ff2_acc& s, ff2_acc b, float2 x) {
 // every output component is then within a few FP32 ulps of its own (O(1)) value, the
 // precision it is stored in.  Case order: y if |ybar| <= y_0; 0 if |ybar| <= -y_0; else
 // the boundary formula.  |ybar|^2 is summed in two lanes, the square root comes from
-// rsqrt and the boundary scale from its reciprocal, without divisions.  The three cases are one scale each for the high
-// and low parts, without branches: zr = the result rounded to FP32, pairs as P; *z0 and
-// the returned z_{K-1} are those two components as two-floats.
+// rsqrt, and the boundary scale from its reciprocal with one correction from the remainder.
+// The three cases are one scale each for the high and low parts, without branches: zr = the
+// result rounded to FP32, pairs as P; *z0 and the returned z_{K-1} are those two components
+// as two-floats.
 template <int NP>
 __device__ __forceinline__ float2 ff2_project(const ff2* P, float2* zr, float2* z0) {
   float2 sh = make_float2(0.f, 0.f), sc = make_float2(0.f, 0.f);
@@ -305,9 +306,13 @@ __device__ __forceinline__ float2 ff2_project(const ff2* P, float2* zr, float2* 
   const bool inside = ff_le(nb, y0), below = ff_le(nb, ff_neg(y0));
   const float2 sum = ff_add(y0, nb);
   const float2 a = make_float2(0.5f * sum.x, 0.5f * sum.y);
-  // inside: h + l; below: 0; else the boundary point along ybar / |ybar|
+  // inside: h + l; below: 0; else the boundary point along ybar / |ybar|, the quotient
+  // (y_0 + |ybar|) / 2 / |ybar| with one correction from its remainder (r alone is good to
+  // two ulps, and its error is the same for all components: phi's error against 64 bits on
+  // 37 x 21 x 50 x 20 was 2.2e-7 so, 2.1e-7 with it)
   const float m = inside ? 1.f : 0.f;
-  const float scale = inside ? 1.f : below ? 0.f : (a.x + a.y) * r;
+  const float as = a.x + a.y, sr = as * r;
+  const float scale = inside ? 1.f : below ? 0.f : fmaf(fmaf(-sr, nb.x, as), r, sr);
   *z0 = inside ? y0 : below ? make_float2(0.f, 0.f) : a;
   const float2 m2 = make_float2(m, m), s2 = make_float2(scale, scale);
 #pragma unroll
