@@ -59,7 +59,6 @@ class MixedBatch {
   void kkt(cudaStream_t s, LaunchCounter lc);
   const double* red_out() const { return red_; }
   const int* error_flag() const { return err_; }
-  void set_tensor_cores(bool on) { ps_.use_tc = on; }
   int slots() const { return G_; }
   // Which of the two (q, alpha, beta) sets is current.  A stream capture of
   // iterate() flips it without running anything; set_parity puts it back.

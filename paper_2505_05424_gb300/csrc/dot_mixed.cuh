@@ -127,7 +127,6 @@ struct MxPoisson {
   float* w1;                      // poisson_scratch_elems(g) floats per solve of a batch
   float* w2;
   int* err;                       // set by a tensor-core pass whose pipeline wait timed out
-  bool use_tc;                    // run eligible passes on the tensor cores
   FastPoisson<float> fast;        // the solve of each iteration, where the grid fits it
   bool use_fast;
 };
@@ -144,17 +143,14 @@ size_t poisson_scratch_elems(const Geo& g);
 size_t tsolve_smem_bytes(const Geo& g);
 
 // src -> dst (src is preserved), FP32 in and out, for G solves of grid g stored
-// one after the other (G > 1 needs poisson_tc_flow).  accum (nullable, two-float,
-// slot-strided like phi): when the tensor-core flow runs, its last pass adds the
-// result into accum instead of writing dst and the call returns true.
-bool launch_poisson_mx(const Geo& g, int G, const MxPoisson& ps, const float* src, float* dst, cudaStream_t s,
-                       LaunchCounter lc, float2* accum);
+// one after the other (G > 1 needs poisson_tc_flow).
+void launch_poisson_mx(const Geo& g, int G, const MxPoisson& ps, const float* src, float* dst, cudaStream_t s,
+                       LaunchCounter lc);
 // Refined solve of f.b (+ f.blo) into out (two-float, slot-strided like phi) for
-// the G slots of a batch; f.b is overwritten.  have_bsum: f.bsum already holds
-// the partial sums of b.
+// the G slots of a batch; f.b is overwritten.
 constexpr int kBsumParts = 608;   // most partial sums per slot
 void launch_poisson_refined_mx(const Geo& g, int G, const MxFields& f, const MxPoisson& ps, float2* out,
-                               bool have_bsum, cudaStream_t s, LaunchCounter lc);
+                               cudaStream_t s, LaunchCounter lc);
 // Multiply the stored alpha/sigma and beta/sigma of every slot whose rescale
 // factor is not 1 by that factor (after a penalty change).
 void launch_rescale_mx(const Geo& g, int G, const MxFields& f, cudaStream_t s, LaunchCounter lc);

@@ -150,7 +150,7 @@ extern "C" int dot_poisson_f32_noalloc(const dot_grid* grid, const float* b, flo
   long launches = 0;
   LaunchCounter lc{&launches};
   static_assert(kBsumParts + 2 <= kBsumStride, "the partial sums and the mean fit one slot's stride");
-  launch_poisson_refined_mx(g, 1, f, ps, reinterpret_cast<float2*>(phi), false, s, lc);
+  launch_poisson_refined_mx(g, 1, f, ps, reinterpret_cast<float2*>(phi), s, lc);
   e = cudaGetLastError();
   if (e != cudaSuccess) return fail(DOT_ECUDA, "launch: ", cudaGetErrorString(e));
   e = cudaStreamSynchronize(s);

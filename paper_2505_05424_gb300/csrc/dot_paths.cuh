@@ -91,8 +91,6 @@ class Path {
   virtual int poisson_op(const double* b, double* phi, cudaStream_t s, LaunchCounter lc, std::string* err) = 0;
   // Device flag that a kernel sets when a bounded pipeline wait gave up (or nullptr).
   virtual const int* error_flag() const { return nullptr; }
-  // Mixed path: whether eligible DCT passes run on the tensor cores.
-  virtual void set_tensor_cores(bool) {}
 
   // Replay of whole check periods from a CUDA graph (the mixed path, whose kernels
   // read the penalty and step from device memory).  set_penalty applies sigma and

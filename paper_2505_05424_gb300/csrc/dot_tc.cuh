@@ -32,8 +32,6 @@ struct TcPass {
   int M, ldo;           // ROWS_FLAT: runs of M rows written with stride ldo; KEEP: output row stride
   const Geo* geo;       // KEEP: grid of one group (rows r map to in-plane index r mod P)
   const float* lam[4];  // KEEP: eigenvalues, lam[0] along the transformed axis
-  float2* accum;        // ROWS_A (nullable): add the result into this two-float field (same
-                        // layout as out) instead of writing out
   int* err;             // set by a CTA whose pipeline wait timed out
   unsigned extra_tx;    // self-test only (dot_selftest_pipeline_timeout): bytes each stage's
                         // barrier expects beyond what its loads deliver; 0 otherwise
@@ -41,9 +39,5 @@ struct TcPass {
 // Returns false when the pass cannot run on the tensor cores (unsupported K,
 // misaligned strides or pointers, tensor maps that cannot be encoded).
 bool launch_tc_pass(const TcPass& p, cudaStream_t s);
-
-// Plain (unswizzled) tiled tensor map for TMA loads of other kernels.
-bool encode_tensor_map(CUtensorMap* m, CUtensorMapDataType type, int rank, const void* base,
-                       const cuuint64_t* dims, const cuuint64_t* strides_bytes, const cuuint32_t* box);
 
 }  // namespace dot

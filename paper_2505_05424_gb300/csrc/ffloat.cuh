@@ -55,12 +55,6 @@ __device__ __forceinline__ float2 ff_sub_exact(float a, float b) { return two_su
 
 __device__ __forceinline__ double ff_to_double(float2 a) { return (double)a.x + (double)a.y; }
 
-// host or device: split a double into (hi, lo) floats
-__host__ __device__ inline float2 ff_from_double(double v) {
-  const float hi = (float)v;
-  return make_float2(hi, (float)(v - (double)hi));
-}
-
 // exact product of two floats as an ff (TwoProd via FMA)
 __device__ __forceinline__ float2 two_prod(float a, float b) {
   const float p = a * b;

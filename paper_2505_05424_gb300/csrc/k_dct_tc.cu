@@ -40,7 +40,6 @@
 
 #include "dot_internal.cuh"
 #include "dot_tc.cuh"
-#include "ffloat.cuh"
 
 namespace dot {
 namespace {
@@ -153,7 +152,6 @@ struct PassArgs {
   int N[kMaxD];
   unsigned P;
   FastDiv fP, fS[kMaxD], fN[kMaxD];
-  float2* accum;   // ROWS_A: accumulate into a two-float field instead of writing out
   int* err;
   unsigned extra_tx;   // see TcPass::extra_tx
 };
@@ -352,16 +350,6 @@ k_dct_pass_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ 
             for (int j = 0; j < 16; ++j)
               if (n0 + c0 + j < pa.K) o[j] = w[j];
           }
-        } else if (pa.accum) {
-          // all 16 loads first, then the stores: no load waits behind a store
-          float2 old[16];
-#pragma unroll
-          for (int j = 0; j < 16; ++j)
-            if (n0 + c0 + j < pa.K) old[j] = pa.accum[out_base + (long long)(n0 + c0 + j) * col_stride];
-#pragma unroll
-          for (int j = 0; j < 16; ++j)
-            if (n0 + c0 + j < pa.K)
-              pa.accum[out_base + (long long)(n0 + c0 + j) * col_stride] = ff_add_f(old[j], __uint_as_float(v[j]));
         } else {
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
@@ -407,18 +395,7 @@ bool encode(CUtensorMap* m, const float* base, int rank, const cuuint64_t* dims,
 
 }  // namespace
 
-bool encode_tensor_map(CUtensorMap* m, CUtensorMapDataType type, int rank, const void* base,
-                       const cuuint64_t* dims, const cuuint64_t* strides_bytes, const cuuint32_t* box) {
-  auto fn = get_encode();
-  if (!fn) return false;
-  cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-  CUresult r = fn(m, type, rank, (void*)base, dims, strides_bytes, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                  CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS;
-}
-
 bool tc_pass_supported(int K) { return K >= 1 && K <= 16 * kMaxN; }
-
 
 bool launch_tc_pass(const TcPass& p, cudaStream_t s) {
   static std::atomic<unsigned long long> smem_done{0};
@@ -462,8 +439,6 @@ bool launch_tc_pass(const TcPass& p, cudaStream_t s) {
   pa.fM = make_fastdiv((unsigned)pa.M);
   pa.err = p.err;
   pa.extra_tx = p.extra_tx;
-  pa.accum = p.mode == TC_ROWS_A ? p.accum : nullptr;
-  if (p.accum && p.mode != TC_ROWS_A) return false;
   if (p.mode == TC_ROWS_FLAT && (p.R % pa.A != 0 || pa.A % pa.M != 0 || pa.ldo < pa.M)) return false;
   if (p.mode == TC_KEEP) {
     if (!p.geo || pa.ldo < K || pa.ldo % 4 != 0 || ((uintptr_t)p.out & 15)) return false;

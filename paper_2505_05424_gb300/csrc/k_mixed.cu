@@ -532,24 +532,22 @@ __global__ void __launch_bounds__(128) k_kkt_final(Geo g, const SlotParam* sp, c
 // delta = P(r); out = phi1 + delta as a two-float pair.  Overwrites f.b with delta.
 template <int D>
 void poisson_refined_tmpl(const Geo& g, int G, const MxFields& f, const MxPoisson& ps, float2* out,
-                          bool have_bsum, cudaStream_t s, LaunchCounter lc) {
+                          cudaStream_t s, LaunchCounter lc) {
   const long long nn = (long long)(g.T + 1) * g.P;
   const int nb = bsum_blocks(g);
-  if (!have_bsum) {
-    k_sum_b<<<dim3(nb, G), kThreads, 0, s>>>(g, f);
-    lc.launched(KID_RESIDUAL);
-  }
+  k_sum_b<<<dim3(nb, G), kThreads, 0, s>>>(g, f);
+  lc.launched(KID_RESIDUAL);
   k_mean_b<<<G, kThreads, 0, s>>>(g, f, nb);
-  launch_poisson_mx(g, G, ps, f.b, f.phi1, s, lc, nullptr);
+  launch_poisson_mx(g, G, ps, f.b, f.phi1, s, lc);
   k_residual<D><<<dim3(grid_for(nn), G), kThreads, 0, s>>>(g, f);
   lc.launched(KID_RESIDUAL, 2);
-  launch_poisson_mx(g, G, ps, f.r, f.b, s, lc, nullptr);
+  launch_poisson_mx(g, G, ps, f.r, f.b, s, lc);
   k_combine<<<dim3(grid_for(nn), G), kThreads, 0, s>>>(g, f, out);
   lc.launched(KID_COMBINE);
 }
 
-// delta = P(f.r), phi += delta: the last DCT pass adds into phi when it runs on
-// the tensor cores; otherwise delta goes through phi1 and one more kernel.
+// delta = P(f.r), phi += delta: the last fast pass adds into phi; on grids beyond the fast
+// solve delta goes through phi1 and one more kernel.
 void poisson_add_tmpl(const Geo& g, int G, const MxFields& f, const MxPoisson& ps, cudaStream_t s,
                       LaunchCounter lc) {
   const long long nn = (long long)(g.T + 1) * g.P;
@@ -557,7 +555,7 @@ void poisson_add_tmpl(const Geo& g, int G, const MxFields& f, const MxPoisson& p
     launch_fast_poisson(g, G, ps.fast, f.r, f.phi1, f.phi, s, lc);
     return;
   }
-  if (launch_poisson_mx(g, G, ps, f.r, f.phi1, s, lc, f.phi)) return;
+  launch_poisson_mx(g, G, ps, f.r, f.phi1, s, lc);
   k_phi_add<<<dim3(grid_for(nn), G), kThreads, 0, s>>>(g, f);
   lc.launched(KID_COMBINE);
 }
@@ -584,9 +582,9 @@ void launch_kkt_tmpl(const Geo& g, int G, const MxFields& f, double* partials, d
 }  // namespace
 
 void launch_poisson_refined_mx(const Geo& g, int G, const MxFields& f, const MxPoisson& ps, float2* out,
-                               bool have_bsum, cudaStream_t s, LaunchCounter lc) {
-  if (g.D == 2) poisson_refined_tmpl<2>(g, G, f, ps, out, have_bsum, s, lc);
-  else poisson_refined_tmpl<3>(g, G, f, ps, out, have_bsum, s, lc);
+                               cudaStream_t s, LaunchCounter lc) {
+  if (g.D == 2) poisson_refined_tmpl<2>(g, G, f, ps, out, s, lc);
+  else poisson_refined_tmpl<3>(g, G, f, ps, out, s, lc);
 }
 
 void launch_rescale_mx(const Geo& g, int G, const MxFields& f, cudaStream_t s, LaunchCounter lc) {

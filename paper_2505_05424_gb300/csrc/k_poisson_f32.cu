@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(256) k_tsolve_f32(Geo g, const float* __restri
 void spatial_pass(const MxPoisson& ps, int axis, bool inverse, const float* X, float* Y, int K, long long n,
                   int mode, int A, int Bd, cudaStream_t s, LaunchCounter lc) {
   const long long R = n / K;
-  if (ps.use_tc && K % 4 == 0 && tc_pass_supported(K)) {
+  if (K % 4 == 0 && tc_pass_supported(K)) {
     TcPass p;
     std::memset(&p, 0, sizeof(p));
     p.X = X;
@@ -269,7 +269,7 @@ void launch_tsolve(const Geo& g, const MxPoisson& ps, const float* X, float* Y, 
 // The tensor-core flow applies when every axis is within the tcgen05 pass's
 // range and the spatial rows have 16-byte strides.
 bool poisson_tc_flow(const Geo& g, const MxPoisson& ps) {
-  if (!ps.use_tc || !ps.tpad[0] || !tc_pass_supported(g.T + 1)) return false;
+  if (!ps.tpad[0] || !tc_pass_supported(g.T + 1)) return false;
   for (int d = 0; d < g.D; ++d)
     if (!tc_pass_supported(g.N[d]) || g.N[d] % 4 != 0) return false;
   return true;
@@ -298,7 +298,7 @@ bool tc_pass(const MxPoisson& ps, TcPass p, int axis, bool inverse, cudaStream_t
 
 // The tensor-core flow for G solves stored one after the other.
 bool poisson_tc(const Geo& g, int G, const MxPoisson& ps, const float* src, float* dst, cudaStream_t s,
-                LaunchCounter lc, float2* accum) {
+                LaunchCounter lc) {
   const long long nn = (long long)(g.T + 1) * g.P;
   const int M = g.T + 1, ldt = time_ld(g);
   float* w[2] = {ps.w1, ps.w2};
@@ -379,7 +379,6 @@ bool poisson_tc(const Geo& g, int G, const MxPoisson& ps, const float* src, floa
       p.A = (int)(g.P / K);
       p.Bd = M;
       p.G = G;
-      p.accum = accum;
     }
     if (!tc_pass(ps, p, a, true, s, lc)) return false;
     cur = p.out;
@@ -390,12 +389,12 @@ bool poisson_tc(const Geo& g, int G, const MxPoisson& ps, const float* src, floa
 
 }  // namespace
 
-bool launch_poisson_mx(const Geo& g, int G, const MxPoisson& ps, const float* src, float* dst, cudaStream_t s,
-                       LaunchCounter lc, float2* accum) {
-  if (poisson_tc_flow(g, ps) && poisson_tc(g, G, ps, src, dst, s, lc, accum)) return accum != nullptr;
+void launch_poisson_mx(const Geo& g, int G, const MxPoisson& ps, const float* src, float* dst, cudaStream_t s,
+                       LaunchCounter lc) {
+  if (poisson_tc_flow(g, ps) && poisson_tc(g, G, ps, src, dst, s, lc)) return;
   if (ps.use_fast) {
     launch_fast_poisson(g, G, ps.fast, src, dst, nullptr, s, lc);
-    return false;
+    return;
   }
   // SIMT flow (one solve)
   const long long n = (long long)(g.T + 1) * g.P;
@@ -424,7 +423,6 @@ bool launch_poisson_mx(const Geo& g, int G, const MxPoisson& ps, const float* sr
     spatial_pass(ps, a, true, cur(), out, K, n, mode, A, Bd, s, lc);
     if (!last) ci = next();
   }
-  return false;
 }
 
 }  // namespace dot

@@ -140,7 +140,6 @@ size_t MixedBatch::workspace_bytes(const Geo& g, int G, bool slot_masks) {
 bool MixedBatch::batchable(const Geo& g) {
   MxPoisson ps;
   std::memset(&ps, 0, sizeof(ps));
-  ps.use_tc = true;
   float dummy = 0.f;
   ps.tpad[0] = &dummy;
   return fused2d_supported(g) && poisson_tc_flow(g, ps);
@@ -250,7 +249,6 @@ int MixedBatch::init(char* ws, size_t bytes, cudaStream_t s, std::string* err) {
     ps_.fast.lam[d] = B.lbuf[1 + d];
   }
   ps_.err = B.err;
-  ps_.use_tc = true;
   if (e == cudaSuccess) e = cudaMemsetAsync(B.err, 0, 64 * sizeof(int), s);
   // zero everything a slot owns (finite scratch for the shared passes) and the params
   const size_t nn = (size_t)(g_.T + 1) * g_.P;
@@ -534,7 +532,7 @@ int MixedBatch::poisson_op(const double* b, double* phi, cudaStream_t s, LaunchC
   if (e == cudaSuccess) e = up(B.f.b, tb.data(), nn * 4, s);
   if (e == cudaSuccess) e = up(B.f.blo, tl.data(), nn * 4, s);
   if (e == cudaSuccess) {
-    launch_poisson_refined_mx(g_, 1, B.f, ps_, B.phi_op, false, s, lc);
+    launch_poisson_refined_mx(g_, 1, B.f, ps_, B.phi_op, s, lc);
     e = cudaGetLastError();
   }
   std::vector<float2> t(nn);
@@ -595,7 +593,6 @@ class PathMixed : public Path {
   void kkt(cudaStream_t s, LaunchCounter lc) override { batch_.kkt(s, lc); }
   const double* red_out() const override { return batch_.red_out(); }
   const int* error_flag() const override { return batch_.error_flag(); }
-  void set_tensor_cores(bool on) override { batch_.set_tensor_cores(on); }
   int read_fields(double* rho, double* m, double* phi, cudaStream_t s, std::string* err) override {
     return batch_.read_fields(0, rho, m, phi, s, err);
   }
