@@ -255,25 +255,30 @@ __device__ __forceinline__ void stage(const Q& np, const V* src, V* dst, const V
 }
 
 // A stage of any odd radix r: outputs k and r - k share their sums over the conjugate
-// input pairs, sum_j (x_j + x_{r-j}) cos and (x_j - x_{r-j}) sin.  The pairs are formed in
-// their places first; a thread then runs over them for KB values of k, so that a pair is
-// read once for KB outputs and their conjugates.
+// input pairs, sum_j (x_j + x_{r-j}) cos and (x_j - x_{r-j}) sin.  KB > 1: the pairs are
+// formed in their places first, and a thread runs over them for KB values of k, so that a
+// pair is read once for KB outputs and their conjugates.  KB = 1: a thread forms them
+// itself, for axes too short to give every thread more than one output.
 template <int KB, bool INV, class Q, class V>
 __device__ __forceinline__ void stage_any(const Q& np, V* src, V* dst, const V* tw, int N, int r, int s, FastDiv fs,
                                           FastDiv fr) {
   const int kPitch = np.pitch();
   const int nb = N / r, hk = (r + 1) / 2, step = nb * kPitch;
-  for (int e = threadIdx.x; e < nb * (hk - 1) * np.count(); e += Q::kThreads) {
-    int pr;
-    const int bj = np.split(e, &pr);
-    const int j = (int)fdiv((unsigned)bj, fr), b = bj - j * nb;
-    V* p = src + (b + nb * (j + 1)) * kPitch + pr;
-    V* q = src + (b + nb * (r - 1 - j)) * kPitch + pr;
-    const V a = *p, c = *q;
-    *p = cadd(a, c);
-    *q = rot<!INV>(csub(a, c));   // i (x_j - x_{r-j}) forward: times sin it adds to the sum
+  // x_j + x_{r-j}, and i (x_j - x_{r-j}) (forward), which times sin adds to the sum
+  auto pair = [](V* a, V* c) {
+    const V x = *a, y = *c;
+    *a = cadd(x, y);
+    *c = rot<!INV>(csub(x, y));
+  };
+  if constexpr (KB > 1) {
+    for (int e = threadIdx.x; e < nb * (hk - 1) * np.count(); e += Q::kThreads) {
+      int pr;
+      const int bj = np.split(e, &pr);
+      const int j = (int)fdiv((unsigned)bj, fr), b = bj - j * nb;
+      pair(src + (b + nb * (j + 1)) * kPitch + pr, src + (b + nb * (r - 1 - j)) * kPitch + pr);
+    }
+    __syncthreads();
   }
-  __syncthreads();
   const int nk = (hk + KB - 1) / KB;
   for (int e = threadIdx.x; e < nb * nk * np.count(); e += Q::kThreads) {
     int pr;
@@ -293,10 +298,12 @@ __device__ __forceinline__ void stage_any(const Q& np, V* src, V* dst, const V* 
       m[i] = 0;
       dm[i] = min(kb * KB + i, hk - 1) * nb;
     }
+#pragma unroll 4
     for (int j = 1; j < hk; ++j) {
       xs += step;
       xd -= step;
-      const V sm = *xs, df = *xd;
+      V sm = *xs, df = *xd;
+      if constexpr (KB == 1) pair(&sm, &df);
 #pragma unroll
       for (int i = 0; i < KB; ++i) {
         m[i] += dm[i];
@@ -324,7 +331,7 @@ __device__ __forceinline__ void stage_any(const Q& np, V* src, V* dst, const V* 
 }
 
 // All stages; returns the buffer that holds the result.
-template <bool INV, int KB = 2, class Q, class V>
+template <bool INV, int KB, class Q, class V>
 __device__ __forceinline__ V* transform(const Q& np, V* a, V* b, const V* tw, const FftPlan& pl) {
   int s = 1;
   for (int i = 0; i < pl.nst; ++i) {
@@ -1007,6 +1014,7 @@ struct XtxArgs {
   const SlotParam* sp;
 };
 
+template <int KB>
 __global__ void __launch_bounds__(AnyPairs::kThreads) k_xtx(const __grid_constant__ XtxArgs a) {
   using V = float2;
   constexpr int kT = AnyPairs::kThreads;
@@ -1025,7 +1033,7 @@ __global__ void __launch_bounds__(AnyPairs::kThreads) k_xtx(const __grid_constan
     A[((x & 1) ? N - 1 - (x >> 1) : x >> 1) * pitch + t] = W[e];
   }
   __syncthreads();
-  V* Z = transform<false>(a.np, A, B, tw, a.plan);
+  V* Z = transform<false, KB>(a.np, A, B, tw, a.plan);
   V* Y = Z == A ? B : A;   // the free buffer
   const V* rf = a.tab + N;
   const int half = (N / 2 + 1) * M;
@@ -1079,7 +1087,7 @@ __global__ void __launch_bounds__(AnyPairs::kThreads) k_xtx(const __grid_constan
     if (k && m != k) Z[m * pitch + t] = zk(__ldg(ri + m), xm, xk);
   }
   __syncthreads();
-  const V* X = transform<true>(a.np, Z, Y, tw, a.plan);
+  const V* X = transform<true, KB>(a.np, Z, Y, tw, a.plan);
 #pragma unroll 4
   for (int e = threadIdx.x; e < M * N; e += kT) {
     const int t = (int)fdiv((unsigned)e, a.fN0), x = e - t * N;
@@ -1097,6 +1105,19 @@ bool use_xtx(const Geo& g) {
   return g.D == 2 && (long long)(g.T + 1) * g.N[0] <= 8704 && xtx_smem(g) <= (size_t)kMaxSmem;
 }
 
+template <int KB>
+void launch_xtx(const XtxArgs& x, dim3 blocks, size_t smem, cudaStream_t s) {
+  static std::atomic<unsigned long long> done{0};
+  smem_optin((const void*)k_xtx<KB>, kMaxSmem, &done);
+  k_xtx<KB><<<blocks, AnyPairs::kThreads, smem, s>>>(x);
+}
+// Two outputs per thread of a large odd radix where the block's rounds of such items take
+// less than its rounds of single ones.
+bool xtx_two(const XtxArgs& x) {
+  const int r = x.plan.rad[x.plan.nst - 1], hk = (r + 1) / 2, n = x.plan.N / r * x.M, t = AnyPairs::kThreads;
+  return r >= 7 && 3 * ((n * ((hk + 1) / 2) + t - 1) / t) < 2 * ((n * hk + t - 1) / t);
+}
+
 template <class R> constexpr int time_threads() { return sizeof(R) == 4 ? 128 : 64; }
 
 template <class R>
@@ -1108,22 +1129,24 @@ void launch_np_kb(const FftArgs<R>& a, cudaStream_t s) {
   smem_optin((const void*)k_dct_any<R, NP, INV, KB>, kMaxSmem, &done);
   k_dct_any<R, NP, INV, KB><<<(unsigned)((a.npair + NP - 1) / NP), kThreads, fft_smem<R>(a.plan.N, NP), s>>>(a);
 }
-// Outputs per thread of a stage with an odd radix r: four in FP32 from r = 64, where every
-// thread then has work, else two; in a kernel of their own, as four take registers that
-// cost every other axis CTAs.  An iteration with two and with four: 508^2 x 32 1,156 and
-// 1,054 us, 1004^2 x 32 5,473 and 4,819 (one output at a time, its pairs formed anew: 1,398
-// and 7,297; before the fast transforms 1,174 and 5,112), 61^3 x 16 719 and 760,
-// 127^2 x 32 109 and 120; FP64 2801 x 2 x 2 3,956 and 4,490.
+// Outputs per thread of a stage with an odd radix r, each number in a kernel of its own, as
+// more take registers that cost other axes CTAs: two where the items of work then still
+// fill half the block (FP64, which waits for its few lanes and not for the loads: a warp),
+// four in FP32 from r = 64 where they fill it all, else one.  An iteration with one (every
+// pair formed anew for each output), two and four: 508^2 x 32 1,398, 1,156 and 1,052 us;
+// 1004^2 x 32 7,290, 5,473 and 4,802 (dense passes on the tensor cores, with the fused pass
+// of then: 1,174 and 5,112); 61^3 x 16 758, 719 and 760; 127^2 x 32 120, 109 and 120;
+// 61^2 x 32 44, 47 and 50; FP64 2801 x 2 x 2 8,493, 3,956 and 4,490; 37^3 x 16 944, 821 and
+// 938; 19 x 23 x 20 90, 94 and -.
 template <class R, int NP, bool INV>
 void launch_np(const FftArgs<R>& a, cudaStream_t s) {
   const int r = a.plan.rad[a.plan.nst - 1];   // the largest odd prime factor, if there is one
+  auto items = [&](int kb) { return a.plan.N / r * (((r + 1) / 2 + kb - 1) / kb) * NP; };
   if constexpr (sizeof(R) == 4) {
-    if (r >= 64 && a.plan.N / r * ((r + 7) / 8) * NP >= kThreads) {
-      launch_np_kb<R, NP, INV, 4>(a, s);
-      return;
-    }
+    if (r >= 64 && items(4) >= kThreads) return launch_np_kb<R, NP, INV, 4>(a, s);
   }
-  launch_np_kb<R, NP, INV, 2>(a, s);
+  if (r < 7 || items(2) < (sizeof(R) == 4 ? kThreads / 2 : 32)) launch_np_kb<R, NP, INV, 1>(a, s);
+  else launch_np_kb<R, NP, INV, 2>(a, s);
 }
 
 template <class R, int N, int NP, bool INV, bool ROWS>
@@ -1228,9 +1251,9 @@ void fast_poisson(const Geo& g, int G, const FastPoisson<R>& fp, const R* src, R
       x.np.f = make_fastdiv((unsigned)x.M);
       x.plan = make_plan(g.N[0]);
       x.sp = G > 1 ? fp.sp : nullptr;
-      static std::atomic<unsigned long long> done{0};
-      smem_optin((const void*)k_xtx, kMaxSmem, &done);
-      k_xtx<<<dim3((g.N[1] + 1) / 2, G), AnyPairs::kThreads, xtx_smem(g), s>>>(x);
+      const dim3 blocks((g.N[1] + 1) / 2, G);
+      if (xtx_two(x)) launch_xtx<2>(x, blocks, xtx_smem(g), s);
+      else launch_xtx<1>(x, blocks, xtx_smem(g), s);
       lc.launched(KID_SCALE);
       fft_axis<R, true>(g, G, 1, fp, fp.w1, dst, accum, true, s, lc);
       return;
