@@ -265,11 +265,16 @@ __device__ __forceinline__ void acc2_add_mul(ff2_acc& s, ff2_acc b, float2 x) {
 // every output component is then within a few FP32 ulps of its own (O(1)) value, the
 // precision it is stored in.  Case order: y if |ybar| <= y_0; 0 if |ybar| <= -y_0; else
 // the boundary formula.  |ybar|^2 is summed in two lanes, the square root comes from
-// rsqrt, and the boundary scale from its reciprocal with one correction from the remainder.
+// rsqrt and the boundary scale from its reciprocal r, two ulps at most off; CORRECT adds one
+// correction from the remainder.  The scale's error is common to a cone's components: on
+// 37 x 21 x 50 x 20 phi's error against 64 bits is 2.2e-7 without the correction and 2.1e-7
+// with it (the 3D pass takes it).  In 2D, over 60 instances solved to 1e-6, it lowers the
+// errors at a fixed iteration by some 7% but raises the mean count of iterations by 0.5% on
+// 256^2 x 64, 0.8% on 128^2 x 32 and 2.6% on 64^2 x 32 with obstacles (the 2D pass does not).
 // The three cases are one scale each for the high and low parts, without branches: zr = the
 // result rounded to FP32, pairs as P; *z0 and the returned z_{K-1} are those two components
 // as two-floats.
-template <int NP>
+template <int NP, bool CORRECT>
 __device__ __forceinline__ float2 ff2_project(const ff2* P, float2* zr, float2* z0) {
   float2 sh = make_float2(0.f, 0.f), sc = make_float2(0.f, 0.f);
 #pragma unroll
@@ -300,13 +305,11 @@ __device__ __forceinline__ float2 ff2_project(const ff2* P, float2* zr, float2* 
   const bool inside = ff_le(nb, y0), below = ff_le(nb, ff_neg(y0));
   const float2 sum = ff_add(y0, nb);
   const float2 a = make_float2(0.5f * sum.x, 0.5f * sum.y);
-  // inside: h + l; below: 0; else the boundary point along ybar / |ybar|, the quotient
-  // (y_0 + |ybar|) / 2 / |ybar| with one correction from its remainder (r alone is good to
-  // two ulps, and its error is the same for all components: phi's error against 64 bits on
-  // 37 x 21 x 50 x 20 was 2.2e-7 so, 2.1e-7 with it)
+  // inside: h + l; below: 0; else the boundary point along ybar / |ybar|
   const float m = inside ? 1.f : 0.f;
   const float as = a.x + a.y, sr = as * r;
-  const float scale = inside ? 1.f : below ? 0.f : fmaf(fmaf(-sr, nb.x, as), r, sr);
+  const float edge = CORRECT ? fmaf(fmaf(-sr, nb.x, as), r, sr) : sr;
+  const float scale = inside ? 1.f : below ? 0.f : edge;
   *z0 = inside ? y0 : below ? make_float2(0.f, 0.f) : a;
   const float2 m2 = make_float2(m, m), s2 = make_float2(scale, scale);
 #pragma unroll

@@ -26,11 +26,12 @@
 //
 // Bound by instruction issue and by the latency of a time step (two barriers, a
 // dependent chain of some 100 FP operations): on 256^2 x 64 136 M warp
-// instructions, 46% issue, 0.6 of the HBM bandwidth on its 1,026 MB, 251 us per launch;
-// 128^2 x 32 47.5 us, 32^2 x 16 10.4 us.  The form before it (a thread per halo cone,
-// faces dealt out in rounds, beta by TMA in component planes, 80 registers at two CTAs per
-// SM, fixed 16-time chunks): 245 M instructions, 357, 62 and 19.6 us; and for odd N_y,
-// where it could not use TMA, 262 us on 150 x 117 x 37 against 60 now.  Measured on the
+// instructions, 48% issue, 0.64 of the HBM bandwidth on its 1,026 MB, 236 us per launch;
+// 128^2 x 32 40.8 us, 32^2 x 16 10.0 us (251, 47.5 and 10.4 with the sums of squared
+// increments in FP64 and one CTA-wide sum per work unit).  The form before it (a thread per
+// halo cone, faces dealt out in rounds, beta by TMA in component planes, 80 registers at two
+// CTAs per SM, fixed 16-time chunks): 245 M instructions, 357, 62 and 19.6 us; and for odd
+// N_y, where it could not use TMA, 262 us on 150 x 117 x 37 against 51 now.  Measured on the
 // way: this mapping at two CTAs of 8 rows and 80 registers 429 us (spills), one CTA of 12
 // rows and 128 registers 293; equal shares of work for every SM and beta in lane pairs
 // 267; a segment owning whole cones, whose last update needs one projection and one face
@@ -263,7 +264,7 @@ __device__ __forceinline__ void segment(const Geo& g, const FusedArgs& a, unsign
         if (yh) qd.y = a.q[2][i + 2 * P];
       }
       float2 z0;
-      const float2 z9 = ff2_project<5>(z, zc, &z0);
+      const float2 z9 = ff2_project<5, false>(z, zc, &z0);
       sz1[tid] = zc[1];
       sz3[lev + tid] = zc[3];
       // q_0 (diagonal 3): rhs = A_0 phi + alpha_0/sigma + u_9 - u_0 with u = z + beta/sigma;
@@ -477,9 +478,9 @@ int ntiles(const Geo& g, int tx) { return ((g.N[0] + tx - 1) / tx) * ((g.N[1] + 
 // smallest halo; smaller tiles give small grids more CTAs and shorter time steps.
 // A CTA's pass takes its share of the time nodes plus the cone time before each segment,
 // at a time per step that grows with the rows, so the choice is the least of that product
-// (with 1 + 0.2 rows for the step, the fit of: 32^2 x 16 10.3 us with 4 rows, 11.8 with
-// 8, 13.3 with 13; 64^2 x 32 22.5, 20.3, 22.6; 96^2 x 16 24.7, 22.0, 22.8; 128^2 x 32
-// 64.0, 47.6, 47.4; 150 x 117 x 37 77.6, 59.4, 59.9).
+// (with 1 + 0.2 rows for the step, the fit of these, taken with the sums still in FP64:
+// 32^2 x 16 10.3 us with 4 rows, 11.8 with 8, 13.3 with 13; 64^2 x 32 22.5, 20.3, 22.6;
+// 96^2 x 16 24.7, 22.0, 22.8; 128^2 x 32 64.0, 47.6, 47.4; 150 x 117 x 37 77.6, 59.4, 59.9).
 int rows_of(const Geo& g, int G) {
   const int rows[3] = {13, 8, 4};
   int best = 13;

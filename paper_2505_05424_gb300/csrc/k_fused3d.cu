@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(kConeThreads) k_cone3(const __grid_constant__ 
 #pragma unroll
     for (int k = 1; k < NP3; ++k) Y[k] = ff2_sub(two_prod2(s2, x_[k]), ff2_of(a.beta[k * n0 + i]));
     float2 zr[NP3], z0;
-    ff2_project<NP3>(Y, zr, &z0);
+    ff2_project<NP3, true>(Y, zr, &z0);
 #pragma unroll
     for (int k = 0; k < NP3; ++k) a.z[k * n0 + i] = zr[k];
     const float2 gp = ff_grad(a.phi[i], a.phi[i + P], a.ih[0]);
