@@ -1132,8 +1132,8 @@ void launch_np_kb(const FftArgs<R>& a, cudaStream_t s) {
   smem_optin((const void*)k_dct_any<R, NP, INV, KB>, kMaxSmem, &done);
   k_dct_any<R, NP, INV, KB><<<(unsigned)((a.npair + NP - 1) / NP), kThreads, fft_smem<R>(a.plan.N, NP), s>>>(a);
 }
-// Outputs per thread of a stage with an odd radix r, each number in a kernel of its own, as
-// more take registers that cost other axes CTAs: two where the items of work then still
+// Outputs per thread of a stage with an odd radix r (their number changes no value), each in a
+// kernel of its own, as more take registers that cost other axes CTAs: two where the items of work then still
 // fill half the block (FP64, which waits for its few lanes and not for the loads: a warp),
 // four in FP32 from r = 64 where they fill it all, else one.  An iteration with one (every
 // pair formed anew for each output), two and four: 508^2 x 32 1,398, 1,156 and 1,052 us;
